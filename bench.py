@@ -85,8 +85,8 @@ def screen_ops(cands) -> int:
 
 
 SEARCH_NAMES = {1: "general interval search", 2: "equal-layer closed form"}
-SEARCH_KERNELS = {1: "gsearch_kernel + wsearch_kernel (general threshold search: one thread per single-fit "
-                     "entry when there are at least 32 per SM, one warp per entry for the rest)",
+SEARCH_KERNELS = {1: "gsearch_kernel + wsearch_kernel (general threshold search: one thread per "
+                     "entry when there are at least 32 per SM, one warp per entry for what it leaves)",
                   2: "eq_search_kernel (equal-layer closed form)"}
 LANES_PER_SM = 128  # 4 SM sub-partitions x 32 lanes issue per clock; the SM count comes from the device
 

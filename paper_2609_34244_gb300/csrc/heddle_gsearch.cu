@@ -1,33 +1,45 @@
 // heddle_gsearch.cu -- general PartitionLayers + Evaluate (§3.1 listing,
 // §5.2 memory validation, §5.3 iteration time) for models whose layers
-// differ, one thread per worklist entry, wherever every stage could hold any
-// single layer of the model.
+// differ, one thread per worklist entry.
 //
-// Call a bound B "single-fit" when every stage could hold any one layer
-// within B (its most expensive layer's time plus its P2P at most B) and
-// within its memory (the largest single-layer state plus its in-flight
-// count times the largest single-layer activation).  At a single-fit bound:
-//   * the feasible ends after stage s form an interval [s, U_s]: an end up
-//     to U_{s-1} + 1 is reached one layer after its predecessor, one beyond
-//     only from U_{s-1} (the largest predecessor dominates); so a probe is
-//     the forward chain U_{s+1} = the furthest end stage s reaches from U_s
-//     (a binary search: stage time and memory grow with the end), feasible
-//     iff the last stage fits [U_{S-1}, L);
-//   * symmetrically the feasible starts of stages s .. S-1 form an interval
-//     [V_s, L - (S - s)], with V_s = the smallest start from which stage s
-//     reaches V_{s+1}; the lexicographically smallest optimal split is then
-//     a_{s+1} = max(a_s + 1, V_{s+1}) (a_s >= V_s, so [a_s, V_{s+1}) costs
-//     no more than [V_s, V_{s+1}), and a single layer always fits).
-// The search itself is that of the warp kernel (heddle_wsearch.cu): a
-// memory-only probe where the screen could not decide memory, the
-// saturating balance as first guess, each probe snapping the bracket to its
-// largest accepted or smallest rejected stage time (every bound in [hi, B]
-// or [B, lo) decides alike), galloping, then bisecting.  An entry that meets
-// a bound that is not single-fit is left to the warp kernel, which runs the
-// general set-based probe; it gets the list of those entries.  The kernel
-// runs only when the depth buckets hold at least PriceArgs::thread_min
-// entries (a few entries would leave it as long as its longest serial
-// chain); each warp takes 32 entries at a time, deepest first.
+// Stage s "holds" [i, j) at a bound B when the interval's time plus the
+// stage's P2P is at most B and its state plus in-flight activations fit the
+// stage's memory; both grow with the interval, so a stage that holds an
+// interval holds every part of it.
+//
+// Probe of a bound B.  U_0 = 0, and U_{s+1} bounds every feasible end of
+// stage s from above: the furthest end stage s reaches from U_s (a later
+// start reaches no less far), or, when it does not hold layer U_s at all
+// (every longer interval from a start up to U_s contains that layer), the
+// largest end j <= U_s whose last layer j - 1 it holds.
+//   * U_s runs out, or the last stage does not hold [U_{S-1}, L): no split
+//     exists, whatever the holes below U_s;
+//   * every stage advanced: the chain itself is a split, so B is feasible;
+//   * some stage stepped back: a split is built from the end, a_s the
+//     largest start at most U_s and below a_{s+1} whose last layer a_s - 1
+//     the stage before holds; if every stage holds its part, B is feasible.
+//     If not, the probe cannot decide: the entry goes to the warp kernel
+//     (heddle_wsearch.cu), which runs the set-based probe.
+// The answers are exact without any condition on the layers.  (Asking that
+// every stage hold any one layer of the model, as this kernel once did, sent
+// 45% of the entries of an 80-layer profile with a heavy first and last
+// layer to the warp kernel: 1.41 ms there per 300,007 candidates beside
+// 0.12 ms here.)
+//
+// The split at B*.  Symmetrically V_S = L and V_s bounds every feasible start
+// of stage s from below; the smallest boundary is at least
+// max(a_s + 1, V_{s+1}), and past that the next one whose first layer stage
+// s + 1 holds.  If every stage holds the part this gives it, no smaller
+// split exists; if not, the entry goes to the warp kernel.
+//
+// The search itself is that of the warp kernel: a memory-only probe where
+// the screen could not decide memory, the saturating balance as first
+// guess, each probe snapping the bracket to its largest accepted or smallest
+// rejected stage time (every bound in [hi, B] has that split, every bound
+// in [B, lo) meets the same rejections), galloping, then bisecting.  The
+// kernel runs only when the depth buckets hold at least
+// PriceArgs::thread_min entries (a few entries would leave it as long as its
+// longest serial chain); each warp takes 32 entries at a time, deepest first.
 
 #include <algorithm>
 
@@ -48,16 +60,15 @@ struct GTabs {
     const int64_t* p2p;    // [8][8][2] (index 128: no next stage, P2P 0)
     const int64_t* mem;    // [8]
     const int64_t* inter;  // [8]
-    const int64_t* qmax;   // [NT * 4] the most expensive single layer
     const float* rqavg;    // [NT * 4] 1 / the average layer time
-    int64_t smax, amax;    // the largest single-layer state and activation
     float avs, ava;        // the average layer state and activation bytes
     int L;
 };
 
 // Stage word (per thread, in shared memory): bits 0-4 the stage byte's type
 // and degree, bits 5-12 the P2P index, bits 13-18 the in-flight count f,
-// bits 19-26 V_s during the split.
+// bits 19-26 the memory run during the guess, then U_s during a probe and
+// V_s during the split.
 constexpr int kVShift = 19;
 constexpr uint32_t kNoV = (1u << kVShift) - 1;
 
@@ -163,35 +174,88 @@ __device__ __forceinline__ int reach_of(const GTabs& t, const GStage& st, int ro
     return lo;
 }
 
-// Exact probe of a single-fit bound B: the forward chain.  hi / lo: the
-// snap values (the largest stage time of the chain; the smallest stage time
-// that rejected an end).
-__device__ bool gprobe(const GTabs& t, const uint32_t* sw, int S, int64_t B, int64_t& hi, int64_t& lo,
-                       unsigned long long& checks) {
+// Stage holds [i, j) within B and its memory?
+__device__ __forceinline__ bool holds(const GTabs& t, const GStage& st, int i, int j, int64_t B) {
+    return cost(t, st, i, j) <= B && fits_mem(t, st, i, j);
+}
+
+__device__ __forceinline__ int pos_of(uint32_t w) { return (int)(w >> kVShift) & 255; }
+
+enum GProbe : int { kInfeasible = 0, kFeasible = 1, kUndecided = 2 };
+
+// The split of a probe in which some stage stepped back, built from the end
+// (see the head of this file); the U_s are in the stage words.  hi: its
+// largest stage time.
+__device__ __noinline__ bool split_below(const GTabs& t, const uint32_t* sw, int S, int64_t B, int64_t& hi,
+                                         unsigned long long& checks) {
+    int end = t.L;
+    hi = -1;
+    GStage st = unpack(sw[(S - 1) * kGBlock], t);
+    for (int s = S - 1; s >= 1; --s) {
+        const GStage before = unpack(sw[(s - 1) * kGBlock], t);
+        int x = min(end - 1, pos_of(sw[s * kGBlock]));
+        for (; x >= s; --x) {
+            ++checks;
+            if (holds(t, before, x - 1, x, B)) break;
+        }
+        ++checks;
+        if (x < s || !holds(t, st, x, end, B)) return false;
+        hi = max(hi, cost(t, st, x, end));
+        end = x;
+        st = before;
+    }
+    ++checks;
+    if (!holds(t, st, 0, end, B)) return false;
+    hi = max(hi, cost(t, st, 0, end));
+    return true;
+}
+
+// Probe of bound B (see the head of this file).  hi / lo: the snap values
+// (the largest stage time of the split found; the smallest stage time that
+// rejected an end).
+__device__ int gprobe(const GTabs& t, uint32_t* sw, int S, int64_t B, int64_t& hi, int64_t& lo,
+                      unsigned long long& checks) {
     const int L = t.L;
     hi = -1;
     lo = kInf;
     int u = 0;
+    bool back = false;
     for (int s = 0; s + 1 < S; ++s) {
         const uint32_t w = sw[s * kGBlock];
+        sw[s * kGBlock] = (w & kNoV) | ((uint32_t)u << kVShift);
         const GStage st = unpack(w, t);
         int64_t acc, rej;
-        const int r = reach_of(t, st, (w & 7) * 4 + ((w >> 3) & 3), u, L - (S - 1 - s), B, acc, rej, checks);
+        int r = reach_of(t, st, (w & 7) * 4 + ((w >> 3) & 3), u, L - (S - 1 - s), B, acc, rej, checks);
         lo = min(lo, rej);
-        if (r < s + 1) return false;
+        if (r == u) {
+            // layer u alone does not fit: the largest end at or below u
+            back = true;
+            for (; r > s; --r) {
+                ++checks;
+                if (fits_mem(t, st, r - 1, r)) {
+                    const int64_t v = cost(t, st, r - 1, r);
+                    if (v <= B) break;
+                    lo = min(lo, v);
+                }
+            }
+        }
+        if (r < s + 1) return kInfeasible;
         hi = max(hi, acc);
         u = r;
     }
-    const GStage st = unpack(sw[(S - 1) * kGBlock], t);
+    const uint32_t w = sw[(S - 1) * kGBlock];
+    sw[(S - 1) * kGBlock] = (w & kNoV) | ((uint32_t)u << kVShift);
+    const GStage st = unpack(w, t);
     ++checks;
-    if (!fits_mem(t, st, u, L)) return false;
+    if (!fits_mem(t, st, u, L)) return kInfeasible;
     const int64_t v = cost(t, st, u, L);
     if (v > B) {
         lo = min(lo, v);
-        return false;
+        return kInfeasible;
     }
     hi = max(hi, v);
-    return true;
+    if (back) return split_below(t, sw, S, B, hi, checks) ? kFeasible : kUndecided;
+    return kFeasible;
 }
 
 // Appends entry p to the list the warp kernel finishes.
@@ -208,7 +272,6 @@ template <bool kCount>
 __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ uint64_t bar;
-    __shared__ int64_t qmax[4 * kMaxTypes], single[2];
     __shared__ float rqavg[4 * kMaxTypes], cfl[129];
     __shared__ int end_of[kMaxStages + 2];
     const Layout& y = a.lay;
@@ -230,31 +293,10 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
     if (!wp::load_image(smem, a.img, y.bytes, &bar, a.err)) return;
     {
         const int64_t* P = reinterpret_cast<const int64_t*>(smem + y.offP);
-        const longlong2* SA = reinterpret_cast<const longlong2*>(smem + y.offSA);
-        // per (type, degree) the most expensive single layer and 1 / the
-        // average layer time; the largest single-layer state and activation
-        for (int r = warp; r <= 4 * y.NT; r += kGWarps) {
-            int64_t m0 = 0, m1 = 0;
-            for (int l = lane; l < L; l += 32) {
-                if (r < 4 * y.NT) {
-                    m0 = max(m0, P[r * (L + 1) + l + 1] - P[r * (L + 1) + l]);
-                } else {
-                    m0 = max(m0, (int64_t)(SA[l + 1].x - SA[l].x));
-                    m1 = max(m1, (int64_t)(SA[l + 1].y - SA[l].y));
-                }
-            }
-            m0 = wp::wmax64(m0);
-            m1 = wp::wmax64(m1);
-            if (lane == 0) {
-                if (r < 4 * y.NT) {
-                    qmax[r] = m0;
-                    const int64_t all = P[r * (L + 1) + L];
-                    rqavg[r] = all > 0 ? (float)L / u64_to_float((uint64_t)all) : 0.f;
-                } else {
-                    single[0] = m0;
-                    single[1] = m1;
-                }
-            }
+        // 1 / the average layer time per (type, degree)
+        for (int r = threadIdx.x; r < 4 * y.NT; r += blockDim.x) {
+            const int64_t all = P[r * (L + 1) + L];
+            rqavg[r] = all > 0 ? (float)L / u64_to_float((uint64_t)all) : 0.f;
         }
         const int64_t* p2p = reinterpret_cast<const int64_t*>(smem + y.offP2P);
         for (int i = threadIdx.x; i < 129; i += blockDim.x) cfl[i] = i < 128 ? u64_to_float((uint64_t)p2p[i]) : 0.f;
@@ -267,10 +309,7 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
     t.p2p = reinterpret_cast<const int64_t*>(smem + y.offP2P);
     t.mem = reinterpret_cast<const int64_t*>(smem + y.offMem);
     t.inter = reinterpret_cast<const int64_t*>(smem + y.offInter);
-    t.qmax = qmax;
     t.rqavg = rqavg;
-    t.smax = single[0];
-    t.amax = single[1];
     {
         const longlong2 all = t.SA[L];
         t.avs = u64_to_float((uint64_t)all.x) / (float)L;
@@ -282,8 +321,7 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
     uint32_t* sw = reinterpret_cast<uint32_t*>(smem + ((y.bytes + 127u) & ~127u)) + threadIdx.x;
 
     unsigned long long checks = 0, probes = 0, priced = 0;
-    // the entries filed in the depth buckets (the screen lists the others
-    // for the warp kernel directly)
+    // the entries filed in the depth buckets (every worklist entry)
     const int64_t entries = min((int64_t)*a.wl_count, (int64_t)a.wl_cap);
     const int64_t count = min((int64_t)end_of[1], entries);
     // each warp prices 32 entries (deepest first): its own first, then the
@@ -312,14 +350,12 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
         const bool memok = a.wl_memok[p] != 0;
         if (!in_range(c, a.n, a.err) || !in_range(S - 1, kMaxStages, a.err)) continue;
         if (kCount) ++priced;
-        // pack the stages; the single-fit threshold QC (no bound below it
-        // is single-fit), the memory test, a bound feasible whenever
-        // memory is, and each stage's memory run from layer 0 for the guess
+        // pack the stages; a bound no split beats (every stage holds at
+        // least its cheapest layer) and a bound feasible whenever memory is
         // (the entry's 32-byte row of stage bytes, read a byte per stage:
         // an array indexed by the stage would live in local memory)
         const uint8_t* row = a.wl_code + p * kMaxStages;
-        int64_t QC = 0, hiB = 0, LB = 0;
-        bool memall = true;
+        int64_t hiB = 0, LB = 0;
         int next = __ldg(row);
         for (int s = 0; s < S; ++s) {
             const int code = next;
@@ -331,27 +367,22 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
                 pidx = (gg * 8 + h) * 2 + ((gg == h) && ((1 << jj) + (1 << jn) <= maxn[gg]));
             }
             const int f = min(S - s, M);
-            uint32_t w = (uint32_t)(code & 31) | ((uint32_t)pidx << 5) | ((uint32_t)f << 13);
+            const uint32_t w = (uint32_t)(code & 31) | ((uint32_t)pidx << 5) | ((uint32_t)f << 13);
             const GStage st = unpack(w, t);
-            QC = max(QC, t.qmax[gg * 4 + jj] + st.c);
             LB = max(LB, minq[gg * 4 + jj] + st.c);
             hiB = max(hiB, t.P[st.row + L] + st.c);
-            memall &= t.smax + st.f * t.amax <= st.capk;
-            // the run of layers memory admits, estimated from the average
-            // layer footprint (for the guess only)
-            const int r0 = min(L, (int)layers_est(t, st, gg * 4 + jj, kInf));
-            w |= (uint32_t)r0 << kVShift;
             sw[s * kGBlock] = w;
-        }
-        if (!memall) {
-            defer(a, p);
-            continue;
         }
         int64_t shi, slo;
         if (!memok) {
             // memory only: OOM, else a tighter feasible bound
             ++probes;
-            if (!gprobe(t, sw, S, kInf, shi, slo, checks)) {
+            const int got = gprobe(t, sw, S, kInf, shi, slo, checks);
+            if (got == kUndecided) {
+                defer(a, p);
+                continue;
+            }
+            if (got == kInfeasible) {
                 a.T[c] = -1;
                 a.B[c] = -1;
                 a.ndp[c] = (uint16_t)n;
@@ -370,7 +401,11 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
             float inv = 0.f, cw = 0.f, flo = 0.f;
             for (int s = 0; s < S; ++s) {
                 const uint32_t w = sw[s * kGBlock];
-                const float rq = rqavg[(w & 7) * 4 + ((w >> 3) & 3)], cf = cfl[(w >> 5) & 255];
+                const int ri = (w & 7) * 4 + ((w >> 3) & 3);
+                const float rq = rqavg[ri], cf = cfl[(w >> 5) & 255];
+                // the run of layers memory admits, estimated from the
+                // average layer footprint
+                sw[s * kGBlock] = (w & kNoV) | ((uint32_t)layers_est(t, unpack(w, t), ri, kInf) << kVShift);
                 inv += rq;
                 cw += cf * rq;
                 if (rq > 0.f) flo = fmaxf(flo, cf + 1.0f / rq);
@@ -399,26 +434,19 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
             }
             B = (int64_t)float_to_u64(fmaxf(fminf(Bf, fhi), 0.f));
         }
-        // the threshold search on single-fit bounds (heddle_wsearch.cu's
-        // bracketing) from the lower bound LB (every stage holds at least
-        // its cheapest layer); a bracket entirely below QC goes to the warp
-        // kernel (with equal layers LB = QC, so that never happens)
+        // the threshold search (heddle_wsearch.cu's bracketing) from LB
         int64_t lo = LB, hi = hiB, step = 1;
-        bool lo_known = false, hi_known = false, deferred = false;
+        bool lo_known = false, hi_known = false, undecided = false;
         int it = 0;
         B = min(max(B, lo), hi - 1);
         while (lo < hi) {
-            if (B < QC) {
-                // the bracket reaches below the single-fit threshold: probe
-                // QC itself while it is inside, else leave the entry
-                if (QC >= hi) {
-                    deferred = true;
-                    break;
-                }
-                B = QC;
-            }
             ++probes;
-            if (gprobe(t, sw, S, B, shi, slo, checks)) {
+            const int got = gprobe(t, sw, S, B, shi, slo, checks);
+            if (got == kUndecided) {
+                undecided = true;
+                break;
+            }
+            if (got == kFeasible) {
                 hi = shi;
                 hi_known = true;
             } else {
@@ -441,27 +469,33 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
             B = min(max(B, lo), hi - 1);
         }
         const int64_t Bstar = hi;
-        if (deferred || Bstar < QC) {
+        if (undecided) {
             defer(a, p);
             continue;
         }
-        // the split: V_s, the smallest start from which stage s reaches
-        // V_{s+1} (V_S = L), into bits 19-26 of the stage words; then
-        // a_{s+1} = max(a_s + 1, V_{s+1})
+        // the split: the smallest start V_s from which stage s reaches
+        // V_{s+1} -- or, when it does not hold layer V_{s+1} - 1, the first
+        // start from V_{s+1} on whose layer it holds -- into bits 19-26 of
+        // the stage words
         {
             int v = L;
             for (int s = S - 1; s >= 1; --s) {
                 const uint32_t w = sw[s * kGBlock];
                 const GStage st = unpack(w, t);
-                // the most layers y + 1 ending at v that stage s holds
-                // within B* (v - 1 holds a single layer), from the estimate
                 const int vv = v;
-                const int y0 = (int)layers_est(t, st, (w & 7) * 4 + ((w >> 3) & 3), Bstar - st.c) - 1;
-                const int y = last_ok(0, vv - 1 - s, y0, [&](int yy) {
-                    ++checks;
-                    return cost(t, st, vv - 1 - yy, vv) <= Bstar && fits_mem(t, st, vv - 1 - yy, vv);
-                });
-                v = vv - 1 - y;
+                ++checks;
+                if (holds(t, st, vv - 1, vv, Bstar)) {
+                    // the most layers y + 1 ending at v that stage s holds, from the estimate
+                    const int y0 = (int)layers_est(t, st, (w & 7) * 4 + ((w >> 3) & 3), Bstar - st.c) - 1;
+                    const int y = last_ok(0, vv - 1 - s, y0, [&](int yy) {
+                        ++checks;
+                        return holds(t, st, vv - 1 - yy, vv, Bstar);
+                    });
+                    v = vv - 1 - y;
+                } else {
+                    while (v < L - (S - s) && !holds(t, st, v, v + 1, Bstar)) ++v;
+                    v = min(v, L - (S - s));
+                }
                 sw[s * kGBlock] = (w & kNoV) | ((uint32_t)v << kVShift);
             }
         }
@@ -473,8 +507,15 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
         for (int s = 0; s < S; ++s) {
             const uint32_t w = sw[s * kGBlock];
             const GStage st = unpack(w, t);
-            const int nxt = s + 1 == S ? L : max(at + 1, (int)((sw[(s + 1) * kGBlock] >> kVShift) & 255));
-            bad |= !fits_mem(t, st, at, nxt);
+            int nxt = L;
+            if (s + 1 < S) {
+                // the first boundary whose first layer the next stage holds
+                const uint32_t wn = sw[(s + 1) * kGBlock];
+                const GStage sn = unpack(wn, t);
+                nxt = max(at + 1, pos_of(wn));
+                while (nxt < L - (S - 1 - s) && !holds(t, sn, nxt, nxt + 1, Bstar)) ++nxt;
+            }
+            bad |= !holds(t, st, at, nxt, Bstar);
             if (a.bounds) a.bounds[(int64_t)(s + 1) * a.bstride + c] = (uint8_t)nxt;
             const int64_t ts = cost(t, st, at, nxt);
             tmax = max(tmax, ts);
@@ -493,7 +534,11 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
             a.bounds[c] = 0;
             for (int s = S + 1; s <= kMaxStages; ++s) a.bounds[(int64_t)s * a.bstride + c] = 0;
         }
-        if (bad || tmax != Bstar) atomicOr(a.err, kErrInternal);
+        if (bad) {
+            defer(a, p);  // the warp kernel writes the whole row
+            continue;
+        }
+        if (tmax != Bstar) atomicOr(a.err, kErrInternal);
         int64_t gmax = 0;
         if (n > 1) {
             // ring all-reduce over n replicas: ceil(2(n-1) G 1e9 / (n k bw))

@@ -13,9 +13,8 @@
 // which one of the searches then prices: the equal-layer closed form
 // (heddle_eqsearch.cu) when every layer costs the same, the paper's split
 // rule in that mode (heddle_distribute.cu), else the general exact
-// threshold search: one thread per entry while every stage fits any single
-// layer (heddle_gsearch.cu), one warp per entry for the rest
-// (heddle_wsearch.cu).
+// threshold search: one thread per entry (heddle_gsearch.cu), and one warp
+// per entry for what that leaves (heddle_wsearch.cu).
 
 #include <algorithm>
 #include <mutex>
@@ -67,8 +66,6 @@ __device__ __forceinline__ uint32_t stage_desc(int b, const Layout& y, const uns
 // (16-byte vector copies when the planes are aligned), the candidates are
 // counting-sorted by S, and thread i screens the i-th of that order, so the
 // lanes of a warp run stage loops of nearly equal length.
-// kGen: the general search follows (the single-fit routing below is live).
-template <bool kGen>
 __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
     __shared__ uint32_t desc[256];
     __shared__ uint8_t win[8 * 4 * 33];
@@ -81,40 +78,8 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
     __shared__ uint8_t order[kScreenBlock];
     __shared__ int bins[kMaxStages + 3];
     __shared__ int smax;
-    // general search only: per (type, degree, in-flight count) whether any
-    // single layer of the model fits the stage's memory; entries with a
-    // stage where not go straight to the warp-per-entry search's list
-    __shared__ uint8_t sfit[8 * 4 * 33];
-    __shared__ long long single[2];
     const Layout& y = a.lay;
     const int L = y.L;
-    constexpr bool gen = kGen;
-    if (gen) {
-        if (threadIdx.x < 32) {
-            const longlong2* SA = reinterpret_cast<const longlong2*>(a.img + y.offSA);
-            long long m0 = 0, m1 = 0;
-            for (int l = threadIdx.x; l < L; l += 32) {
-                const longlong2 u = SA[l], v = SA[l + 1];
-                m0 = max(m0, v.x - u.x);
-                m1 = max(m1, v.y - u.y);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, o));
-                m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, o));
-            }
-            if (threadIdx.x == 0) {
-                single[0] = m0;
-                single[1] = m1;
-            }
-        }
-        __syncthreads();
-        const int64_t* gmem = reinterpret_cast<const int64_t*>(a.img + y.offMem);
-        for (int i = threadIdx.x; i < 8 * 4 * 33; i += blockDim.x) {
-            const int g = i / 132, j = (i / 33) & 3, f = i % 33;
-            sfit[i] = g < y.NT && single[0] + (long long)f * single[1] <= (long long)(gmem[g] << j);
-        }
-    }
     {
         const int32_t* gcap = reinterpret_cast<const int32_t*>(a.img + y.offCap);
         for (int i = threadIdx.x; i < 256; i += blockDim.x) desc[i] = stage_desc(i, y, a.img, a.moe);
@@ -193,7 +158,6 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
         const bool live = threadIdx.x < nloc;  // padding sorts last
         const int64_t c = c0 + ci;
         int S = 0, M = 0, status = HEDDLE_CAND_INVALID;
-        uint32_t fits1 = 1;  // every stage could hold any single layer (general search)
         int64_t n = 0;
         if (live) {
             S = sS[ci] & 0x3f;
@@ -214,7 +178,6 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
                     const int w = win[wi];
                     run_sum += w;
                     run_min = min(run_min, w);
-                    if (gen) fits1 &= sfit[wi];
                 }
                 if (bad >> 31) {
                     status = HEDDLE_CAND_INVALID;
@@ -269,20 +232,9 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
                 }
             }
             // the entry in its depth's bucket, for the searches' order by
-            // decreasing depth -- or, for the general search when some
-            // stage cannot hold every single layer, in the list of the
-            // warp-per-entry search
-            const bool listed = gen && take && !fits1;
-            const unsigned bmask = __ballot_sync(0xffffffffu, take && !listed);
-            const unsigned lmask = __ballot_sync(0xffffffffu, listed);
-            if (lmask) {
-                int l0 = 0;
-                if (lane == __ffs(lmask) - 1) l0 = atomicAdd(a.wl_count + kWlGeneral, __popc(lmask));
-                l0 = __shfl_sync(0xffffffffu, l0, __ffs(lmask) - 1) + __popc(lmask & ((1u << lane) - 1));
-                if (listed && p < a.wl_cap && l0 < a.wl_cap) a.sv_idx[l0] = p;
-            }
-            if (take && !listed) {
-                const unsigned same = __match_any_sync(bmask, S);
+            // decreasing depth
+            if (take) {
+                const unsigned same = __match_any_sync(mask, S);
                 const int leader = __ffs(same) - 1;
                 int b0 = 0;
                 if (lane == leader) b0 = atomicAdd(a.wl_count + 1 + S, __popc(same));
@@ -306,8 +258,8 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
 
 }  // namespace
 
-// The general search: one thread per entry where every stage fits any single
-// layer (heddle_gsearch.cu), then one warp per entry it left (heddle_wsearch.cu).
+// The general search: one thread per entry (heddle_gsearch.cu), then one warp
+// per entry it left (heddle_wsearch.cu).
 cudaError_t launch_thread_search(const PriceArgs& a, int num_sms, cudaStream_t st);
 cudaError_t launch_warp_search(const PriceArgs& a, int num_sms, cudaStream_t st, bool listed);
 
@@ -318,12 +270,11 @@ cudaError_t launch_screen(const PriceArgs& a, int num_sms, cudaStream_t st, cuda
     if (e != cudaSuccess) return e;
     // one wave of resident CTAs, each looping over slices
     int screen_per_sm = 0;
-    e = resident_blocks(reinterpret_cast<const void*>(&screen_kernel<false>), kScreenBlock, 0, &screen_per_sm);
+    e = resident_blocks(reinterpret_cast<const void*>(&screen_kernel), kScreenBlock, 0, &screen_per_sm);
     if (e != cudaSuccess) return e;
     const int grid = (int)std::min<int64_t>((a.n + kScreenBlock - 1) / kScreenBlock,
                                             (int64_t)num_sms * std::max(screen_per_sm, 1));
-    if (!a.uniform && !a.split_mode) screen_kernel<true><<<grid, kScreenBlock, 0, st>>>(a);
-    else screen_kernel<false><<<grid, kScreenBlock, 0, st>>>(a);
+    screen_kernel<<<grid, kScreenBlock, 0, st>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (launches) launches[0] += 1;
     if (mid && (e = cudaEventRecord(mid, st)) != cudaSuccess) return e;

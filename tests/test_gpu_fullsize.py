@@ -79,7 +79,7 @@ def test_full_size(heddle_lib, oracle_mod, name, n, search, path):
 @pytest.mark.parametrize("thread_min", [0, 2**31 - 1], ids=["thread", "warp"])
 def test_full_size_general_routes(heddle_lib, oracle_mod, thread_min):
     """moe48 at full size with the general search's routing forced each way
-    (by default its few single-fit entries go to the warp kernel)."""
+    (by default the thread kernel runs when it has enough entries)."""
     h = heddle_lib
     name, n = "moe48", 1_000_000
     w, ref, top = _oracle_full(oracle_mod, name, n)

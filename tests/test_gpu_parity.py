@@ -60,10 +60,9 @@ def test_parity_small(h, W, oracle_mod, name, n, seed, route):
 
 
 def test_thread_search_defers_to_warp_search(h, W, oracle_mod):
-    """moe16 through the thread-per-entry search: entries whose bracket
-    falls below the single-fit threshold are handed to the warp search
-    (counted twice: the interval-test counters see both kernels), and the
-    results still equal the oracle's."""
+    """moe16 through the thread-per-entry search: entries whose
+    probe it cannot decide are handed to the warp search (counted
+    twice: the interval-test counters see both kernels), and the results still equal the oracle's."""
     w = W.make_workload("moe16", seed=0, n=4001)
     ref = oracle_mod.Oracle(w.cluster, w.model).price(w.cands, threads=8)
     both = G.price_gpu(h, w.cluster, w.model, w.cands, search=1, thread_min=0, count=True)
@@ -72,6 +71,36 @@ def test_thread_search_defers_to_warp_search(h, W, oracle_mod):
         assert got["errors"] == 0
         G.assert_same(got, ref, what="moe16")
     assert both["counters"]["priced"] > warp["counters"]["priced"], "no entry was handed on"
+
+
+@pytest.mark.parametrize("L", [1, 2, 3, 5, 31, 32, 33, 80, 255])
+@pytest.mark.parametrize("kind", ["heavy_ends", "alternating", "ragged", "free"])
+def test_thread_search_stepping_back(h, W, oracle_mod, L, kind):
+    """The thread-per-entry search where single layers do not fit single
+    stages -- a heavy first and last layer, every second layer heavy in
+    memory, layers of random size, layers that cost nothing -- at depths up
+    to the layer count, against the oracle and the warp search."""
+    rng = np.random.default_rng(L)
+    nt = 3
+    cluster = W.make_cluster([100.0, 400.0, 1000.0], [2 * 10**9, 4 * 10**9, 8 * 10**9], [10**11] * nt,
+                             [(0, 8, 10**10), (1, 4, 2 * 10**10), (2, 8, 5 * 10**10)] * 8)
+    w = {"heavy_ends": np.ones(L), "alternating": np.where(np.arange(L) % 2, 6.0, 0.5),
+         "ragged": rng.uniform(0.3, 3.0, L), "free": np.where(rng.random(L) < 0.5, 0.0, 1.0)}[kind].copy()
+    if kind == "heavy_ends":
+        w[0], w[-1] = 0.2, 4.0
+    flops = 1e13 * w * rng.uniform(0.9, 1.1, L)
+    state = (2.0e9 * w * min(1.0, 24.0 / L)).astype(np.int64)
+    model = W.make_model(flops, state // 8, state, state // 16, 10**6, 0, 10**6)
+    n = 2000
+    S = rng.integers(1, min(L, 32) + 1, n).astype(np.uint8)
+    code = W.encode(rng.integers(0, nt, (32, n)), rng.integers(0, 3, (32, n))).astype(np.uint8)
+    code[np.arange(32)[:, None] >= S[None, :]] = 0
+    cands = W.make_cands(S, rng.choice([1, 4, 64], n).astype(np.uint16), code)
+    ref = oracle_mod.Oracle(cluster, model).price(cands, threads=8)
+    for thread_min in (0, 2**31 - 1):
+        got = G.price_gpu(h, cluster, model, cands, search=1, thread_min=thread_min)
+        assert got["errors"] == 0
+        G.assert_same(got, ref, what="%s L %d thread_min %d" % (kind, L, thread_min))
 
 
 @pytest.mark.parametrize("name", ["tiny", "dense32", "dense80", "moe48", "stress128"])
