@@ -32,11 +32,11 @@
 // s + 1 holds.  If every stage holds the part this gives it, no smaller
 // split exists; if not, the entry goes to the warp kernel.
 //
-// The search itself is that of the warp kernel: a memory-only probe where
-// the screen could not decide memory, the saturating balance as first
-// guess, each probe snapping the bracket to its largest accepted or smallest
-// rejected stage time (every bound in [hi, B] has that split, every bound
-// in [B, lo) meets the same rejections), galloping, then bisecting.  The
+// The search: a memory-only probe where the screen could not decide memory,
+// the saturating balance as first guess, each probe snapping the bracket to
+// its largest accepted or smallest rejected stage time (every bound in
+// [hi, B] has that split, every bound in [B, lo) meets the same rejections),
+// galloping, then bisecting.  The
 // kernel runs only when the depth buckets hold at least
 // PriceArgs::thread_min entries (a few entries would leave it as long as its
 // longest serial chain); each warp takes 32 entries at a time, deepest first.
@@ -50,7 +50,14 @@ namespace {
 
 constexpr int kGBlock = 128;
 constexpr int kGWarps = kGBlock / 32;
+constexpr unsigned kFull = 0xffffffffu;
 constexpr int kGMaxIters = 256;
+constexpr int kStepShift = 7;
+// Undecided probes after which an entry goes to the warp kernel: they do not
+// snap the bracket, so closing it takes a bisection down to 1 ns, and a warp
+// waits for its slowest lane.
+constexpr int kMaxDoubts = 3;
+constexpr int64_t kNoBound = (int64_t)1 << 61;  // above every stage time
 constexpr int kGZeroP2P = 128;  // index of a zero after the 8 x 8 x 2 P2P table
 
 struct GTabs {
@@ -61,7 +68,8 @@ struct GTabs {
     const int64_t* mem;    // [8]
     const int64_t* inter;  // [8]
     const float* rqavg;    // [NT * 4] 1 / the average layer time
-    float avs, ava;        // the average layer state and activation bytes
+    const int64_t* minmid; // [NT * 4] the cheapest layer besides the first and the last
+    const uint8_t* win;    // [8 * 4][33] the longest run of layers within memory, per in-flight count
     int L;
 };
 
@@ -146,32 +154,75 @@ __device__ __forceinline__ int last_ok(int lo, int hi, int x0, F ok) {
     return a;
 }
 
-// Layers of stage st that a bound B and its memory admit, estimated from
-// the average layer time and footprint (for the searches' first guesses).
+// Layers of stage st that a bound and its memory admit, estimated from the
+// average layer time and the longest run of layers its memory holds anywhere
+// (for the searches' first guesses).
 __device__ __forceinline__ float layers_est(const GTabs& t, const GStage& st, int row_idx, int64_t room) {
     const float by_time = room > 0 ? u64_to_float((uint64_t)room) * t.rqavg[row_idx] : 0.f;
-    const float by_mem = u64_to_float((uint64_t)st.capk) / fmaxf(t.avs + (float)st.f * t.ava, 1.f);
-    return fminf(fminf(by_time, by_mem), (float)t.L);
+    return fminf(by_time, (float)t.win[row_idx * 33 + (int)st.f]);
 }
 
 // The furthest end j in (u, lim] of a stage starting at u within B and its
-// memory (u if none).  acc: the stage time at that end (-1 if none); rej:
-// the stage time at the next end if memory admits it there and its time is
-// above B (kInf otherwise).  checks counts the interval tests.
-__device__ __forceinline__ int reach_of(const GTabs& t, const GStage& st, int row_idx, int u, int lim, int64_t B,
-                                        int64_t& acc, int64_t& rej, unsigned long long& checks) {
-    const int x0 = u + (int)layers_est(t, st, row_idx, B - st.c);
-    const int lo = last_ok(u, lim, x0, [&](int j) {
-        ++checks;
-        return cost(t, st, u, j) <= B && fits_mem(t, st, u, j);
-    });
-    acc = lo > u ? cost(t, st, u, lo) : -1;
-    rej = kInf;
-    if (lo < lim && fits_mem(t, st, u, lo + 1)) {
-        const int64_t v = cost(t, st, u, lo + 1);
-        if (v > B) rej = v;
+// memory (u if none; for the last stage only L counts).  acc: the stage time
+// at that end (-1 if none); rej: the stage time at the next end (the last
+// stage: at L) if memory admits it there and its time is above B (kInf
+// otherwise).
+//
+// The terms of u move to the other side once (the memory sums stay below
+// 2^57, B - c + P[u] below 2^62), so a test is two loads, one multiplication
+// and two comparisons.  Four consecutive ends around the estimate are tested
+// side by side, whatever they say, and only a boundary outside them is
+// searched for: a warp's lanes stay together, where a gallop from the
+// estimate left 8.2 of 32 lanes active.
+__device__ __forceinline__ int reach_of(const GTabs& t, const GStage& st, int row_idx, int u, int lim, bool last,
+                                        int64_t B, int64_t& acc, int64_t& rej) {
+    const int64_t* P = t.P + st.row;
+    const longlong2 su = t.SA[u];
+    const int64_t Pu = P[u];
+    const int64_t time_lim = B - st.c + Pu, mem_lim = st.capk + su.x + st.f * (int64_t)su.y;
+    auto ok = [&](int j) {
+        const longlong2 sj = t.SA[j];
+        return P[j] <= time_lim && (int64_t)sj.x + st.f * (int64_t)sj.y <= mem_lim;
+    };
+    const int est = (int)layers_est(t, st, row_idx, B - st.c);
+    const int x0 = min(max(last ? lim : u + est - 1, u), max(lim - 3, u));
+    const bool o0 = x0 == u || ok(x0);
+    const bool o1 = ok(min(x0 + 1, lim)), o2 = ok(min(x0 + 2, lim)), o3 = ok(min(x0 + 3, lim));
+    int r = min(x0 - 1 + (int)o0 + (int)o1 + (int)o2 + (int)o3, lim);
+    if (!last) {
+        if (!o0) r = last_ok(u, x0 - 1, x0 - 1, ok);
+        else if (o3 && x0 + 3 < lim) r = last_ok(x0 + 3, lim, x0 + 4, ok);
     }
-    return lo;
+    acc = r > u ? P[r] - Pu + st.c : -1;
+    rej = kInf;
+    const int q = last ? lim : r + 1;
+    if (q > r && q <= lim && P[q] > time_lim) {
+        const longlong2 sq = t.SA[q];
+        if ((int64_t)sq.x + st.f * (int64_t)sq.y <= mem_lim) rej = P[q] - Pu + st.c;
+    }
+    return r;
+}
+
+// The smallest start i in [s, v) from which a stage reaches v within B and
+// its memory; v if it does not hold layer v - 1.
+__device__ __forceinline__ int start_of(const GTabs& t, const GStage& st, int row_idx, int s, int v, int64_t B) {
+    const int64_t* P = t.P + st.row;
+    const longlong2 sv = t.SA[v];
+    const int64_t time_lim = P[v] + st.c - B, mem_lim = (int64_t)sv.x + st.f * (int64_t)sv.y - st.capk;
+    auto ok = [&](int i) {
+        const longlong2 si = t.SA[i];
+        return P[i] >= time_lim && (int64_t)si.x + st.f * (int64_t)si.y >= mem_lim;
+    };
+    const int est = (int)layers_est(t, st, row_idx, B - st.c);
+    const int x0 = max(min(v - est - 1, v - 4), s);
+    const int held = (int)ok(x0) + (int)ok(min(x0 + 1, v - 1)) + (int)ok(min(x0 + 2, v - 1)) +
+                     (int)ok(min(x0 + 3, v - 1));
+    if (held == 4 && x0 > s) return x0 - last_ok(0, x0 - s, 1, [&](int y) { return ok(x0 - y); });
+    if (held == 0) {
+        if (x0 + 4 >= v || !ok(v - 1)) return v;
+        return v - 1 - last_ok(0, v - 1 - (x0 + 4), v - 1 - (x0 + 4), [&](int y) { return ok(v - 1 - y); });
+    }
+    return x0 + 4 - held;
 }
 
 // Stage holds [i, j) within B and its memory?
@@ -181,98 +232,48 @@ __device__ __forceinline__ bool holds(const GTabs& t, const GStage& st, int i, i
 
 __device__ __forceinline__ int pos_of(uint32_t w) { return (int)(w >> kVShift) & 255; }
 
-enum GProbe : int { kInfeasible = 0, kFeasible = 1, kUndecided = 2 };
-
 // The split of a probe in which some stage stepped back, built from the end
-// (see the head of this file); the U_s are in the stage words.  hi: its
-// largest stage time.
-__device__ __noinline__ bool split_below(const GTabs& t, const uint32_t* sw, int S, int64_t B, int64_t& hi,
-                                         unsigned long long& checks) {
+// (see the head of this file); the U_s are in the stage words.  Its largest
+// stage time, or -1 if a stage does not hold its part.
+__device__ __noinline__ int64_t split_below(const GTabs& t, const uint32_t* sw, int S, int64_t B) {
     int end = t.L;
-    hi = -1;
+    int64_t hi = -1;
     GStage st = unpack(sw[(S - 1) * kGBlock], t);
     for (int s = S - 1; s >= 1; --s) {
         const GStage before = unpack(sw[(s - 1) * kGBlock], t);
         int x = min(end - 1, pos_of(sw[s * kGBlock]));
-        for (; x >= s; --x) {
-            ++checks;
-            if (holds(t, before, x - 1, x, B)) break;
-        }
-        ++checks;
-        if (x < s || !holds(t, st, x, end, B)) return false;
+        while (x >= s && !holds(t, before, x - 1, x, B)) --x;
+        if (x < s || !holds(t, st, x, end, B)) return -1;
         hi = max(hi, cost(t, st, x, end));
         end = x;
         st = before;
     }
-    ++checks;
-    if (!holds(t, st, 0, end, B)) return false;
-    hi = max(hi, cost(t, st, 0, end));
-    return true;
+    return holds(t, st, 0, end, B) ? max(hi, cost(t, st, 0, end)) : -1;
 }
 
-// Probe of bound B (see the head of this file).  hi / lo: the snap values
-// (the largest stage time of the split found; the smallest stage time that
-// rejected an end).
-__device__ int gprobe(const GTabs& t, uint32_t* sw, int S, int64_t B, int64_t& hi, int64_t& lo,
-                      unsigned long long& checks) {
-    const int L = t.L;
-    hi = -1;
-    lo = kInf;
-    int u = 0;
-    bool back = false;
-    for (int s = 0; s + 1 < S; ++s) {
-        const uint32_t w = sw[s * kGBlock];
-        sw[s * kGBlock] = (w & kNoV) | ((uint32_t)u << kVShift);
-        const GStage st = unpack(w, t);
-        int64_t acc, rej;
-        int r = reach_of(t, st, (w & 7) * 4 + ((w >> 3) & 3), u, L - (S - 1 - s), B, acc, rej, checks);
-        lo = min(lo, rej);
-        if (r == u) {
-            // layer u alone does not fit: the largest end at or below u
-            back = true;
-            for (; r > s; --r) {
-                ++checks;
-                if (fits_mem(t, st, r - 1, r)) {
-                    const int64_t v = cost(t, st, r - 1, r);
-                    if (v <= B) break;
-                    lo = min(lo, v);
-                }
-            }
-        }
-        if (r < s + 1) return kInfeasible;
-        hi = max(hi, acc);
-        u = r;
-    }
-    const uint32_t w = sw[(S - 1) * kGBlock];
-    sw[(S - 1) * kGBlock] = (w & kNoV) | ((uint32_t)u << kVShift);
-    const GStage st = unpack(w, t);
-    ++checks;
-    if (!fits_mem(t, st, u, L)) return kInfeasible;
-    const int64_t v = cost(t, st, u, L);
-    if (v > B) {
-        lo = min(lo, v);
-        return kInfeasible;
-    }
-    hi = max(hi, v);
-    if (back) return split_below(t, sw, S, B, hi, checks) ? kFeasible : kUndecided;
-    return kFeasible;
-}
-
-// Appends entry p to the list the warp kernel finishes.
-__device__ __forceinline__ void defer(const PriceArgs& a, int64_t p) {
+// Appends entry p to the list the warp kernel finishes, with the bracket
+// [lo, hi] of B* (hi a feasible bound, -1: memory is undecided; probed: a
+// probe found the split of hi).
+__device__ __forceinline__ void defer(const PriceArgs& a, int64_t p, int64_t hi, int64_t lo, bool probed) {
     const int pos = atomicAdd(a.wl_count + kWlGeneral, 1);
-    if (in_range(pos, a.wl_cap, a.err)) a.sv_idx[pos] = (int32_t)p;
+    if (in_range(pos, a.wl_cap, a.err)) {
+        a.sv_idx[pos] = (int32_t)p;
+        a.sv_T[pos] = hi;
+        a.sv_nM[pos] = probed ? 1 : 0;
+        a.wl_T[p] = lo;
+    }
 }
 
 // Below a.thread_min bucketed entries the kernel returns at once and the
-// warp kernel prices the whole worklist.  Four CTAs per SM (the table
-// image and the stage words fill shared memory there), so up to 128
-// registers a thread.
+// warp kernel prices the whole worklist.  Five CTAs per SM at 90 registers a
+// thread: a cap that lets in six or eight measured 0.38 and 0.43 ms beside
+// 0.35 ms (profiled 80-layer model, 300,007 candidates).
 template <bool kCount>
 __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ uint64_t bar;
     __shared__ float rqavg[4 * kMaxTypes], cfl[129];
+    __shared__ int64_t minmid[4 * kMaxTypes];
     __shared__ int end_of[kMaxStages + 2];
     const Layout& y = a.lay;
     const int L = y.L;
@@ -293,10 +294,17 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
     if (!wp::load_image(smem, a.img, y.bytes, &bar, a.err)) return;
     {
         const int64_t* P = reinterpret_cast<const int64_t*>(smem + y.offP);
-        // 1 / the average layer time per (type, degree)
-        for (int r = threadIdx.x; r < 4 * y.NT; r += blockDim.x) {
-            const int64_t all = P[r * (L + 1) + L];
-            rqavg[r] = all > 0 ? (float)L / u64_to_float((uint64_t)all) : 0.f;
+        // per (type, degree) 1 / the average layer time and the cheapest
+        // layer besides the first and the last
+        for (int r = warp; r < 4 * y.NT; r += kGWarps) {
+            int64_t m = kInf;
+            for (int l = 1 + lane; l + 1 < L; l += 32) m = min(m, P[r * (L + 1) + l + 1] - P[r * (L + 1) + l]);
+            m = wp::wmin64(m);
+            if (lane == 0) {
+                minmid[r] = m;
+                const int64_t all = P[r * (L + 1) + L];
+                rqavg[r] = all > 0 ? (float)L / u64_to_float((uint64_t)all) : 0.f;
+            }
         }
         const int64_t* p2p = reinterpret_cast<const int64_t*>(smem + y.offP2P);
         for (int i = threadIdx.x; i < 129; i += blockDim.x) cfl[i] = i < 128 ? u64_to_float((uint64_t)p2p[i]) : 0.f;
@@ -310,14 +318,10 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
     t.mem = reinterpret_cast<const int64_t*>(smem + y.offMem);
     t.inter = reinterpret_cast<const int64_t*>(smem + y.offInter);
     t.rqavg = rqavg;
-    {
-        const longlong2 all = t.SA[L];
-        t.avs = u64_to_float((uint64_t)all.x) / (float)L;
-        t.ava = u64_to_float((uint64_t)all.y) / (float)L;
-    }
+    t.minmid = minmid;
+    t.win = smem + y.offWin;
     t.L = L;
     const int32_t* maxn = reinterpret_cast<const int32_t*>(smem + y.offMaxN);
-    const int64_t* minq = reinterpret_cast<const int64_t*>(smem + y.offMinQ);
     uint32_t* sw = reinterpret_cast<uint32_t*>(smem + ((y.bytes + 127u) & ~127u)) + threadIdx.x;
 
     unsigned long long checks = 0, probes = 0, priced = 0;
@@ -334,143 +338,198 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
     };
     for (int64_t base = ((int64_t)blockIdx.x * kGWarps + warp) * 32; base < count; base = take()) {
         const int64_t g = base + lane;
-        if (g >= count) continue;
-        int lo_d = 1, hi_d = kMaxStages;
-        while (lo_d < hi_d) {
-            const int mid = (lo_d + hi_d + 1) >> 1;
-            if (end_of[mid] > g) lo_d = mid; else hi_d = mid - 1;
-        }
-        const int64_t off = g - end_of[lo_d + 1];
-        if (!in_range(off, end_of[lo_d] - end_of[lo_d + 1], a.err)) continue;
-        const int64_t p = a.wl_bucket[(int64_t)(lo_d - 1) * a.wl_cap + off];
-        if (!in_range(p, entries, a.err)) continue;
-        const int64_t c = a.wl_idx[p];
-        const int S = a.wl_S[p], M = a.wl_M[p];
-        const int64_t n = a.wl_n[p];
-        const bool memok = a.wl_memok[p] != 0;
-        if (!in_range(c, a.n, a.err) || !in_range(S - 1, kMaxStages, a.err)) continue;
-        if (kCount) ++priced;
-        // pack the stages; a bound no split beats (every stage holds at
-        // least its cheapest layer) and a bound feasible whenever memory is
-        // (the entry's 32-byte row of stage bytes, read a byte per stage:
-        // an array indexed by the stage would live in local memory)
-        const uint8_t* row = a.wl_code + p * kMaxStages;
-        int64_t hiB = 0, LB = 0;
-        int next = __ldg(row);
-        for (int s = 0; s < S; ++s) {
-            const int code = next;
-            next = s + 1 < S ? __ldg(row + s + 1) : 0;
-            const int gg = code & 7, jj = (code >> 3) & 3;
-            int pidx = kGZeroP2P;
-            if (s + 1 < S) {
-                const int h = next & 7, jn = (next >> 3) & 3;
-                pidx = (gg * 8 + h) * 2 + ((gg == h) && ((1 << jj) + (1 << jn) <= maxn[gg]));
+        bool have = g < count;
+        int64_t p = 0;
+        if (have) {
+            int lo_d = 1, hi_d = kMaxStages;
+            while (lo_d < hi_d) {
+                const int mid = (lo_d + hi_d + 1) >> 1;
+                if (end_of[mid] > g) lo_d = mid; else hi_d = mid - 1;
             }
-            const int f = min(S - s, M);
-            const uint32_t w = (uint32_t)(code & 31) | ((uint32_t)pidx << 5) | ((uint32_t)f << 13);
-            const GStage st = unpack(w, t);
-            LB = max(LB, minq[gg * 4 + jj] + st.c);
-            hiB = max(hiB, t.P[st.row + L] + st.c);
-            sw[s * kGBlock] = w;
+            const int64_t off = g - end_of[lo_d + 1];
+            have = in_range(off, end_of[lo_d] - end_of[lo_d + 1], a.err);
+            if (have) p = a.wl_bucket[(int64_t)(lo_d - 1) * a.wl_cap + off];
+            have = have && in_range(p, entries, a.err);
         }
-        int64_t shi, slo;
-        if (!memok) {
-            // memory only: OOM, else a tighter feasible bound
-            ++probes;
-            const int got = gprobe(t, sw, S, kInf, shi, slo, checks);
-            if (got == kUndecided) {
-                defer(a, p);
-                continue;
-            }
-            if (got == kInfeasible) {
-                a.T[c] = -1;
-                a.B[c] = -1;
-                a.ndp[c] = (uint16_t)n;
-                a.status[c] = HEDDLE_CAND_OOM;
-                a.wl_T[p] = -1;
-                if (a.bounds)
-                    for (int s = 0; s <= kMaxStages; ++s) a.bounds[(int64_t)s * a.bstride + c] = 0;
-                continue;
-            }
-            hiB = shi;
-        }
-        // first guess: the saturating continuous balance with each stage's
-        // average layer time and memory run from layer 0
-        int64_t B;
-        {
-            float inv = 0.f, cw = 0.f, flo = 0.f;
+        const int64_t c = have ? a.wl_idx[p] : 0;
+        const int S = have ? a.wl_S[p] : 1, M = have ? a.wl_M[p] : 1;
+        const int64_t n = have ? a.wl_n[p] : 1;
+        const bool memok = have && a.wl_memok[p] != 0;
+        have = have && in_range(c, a.n, a.err) && in_range(S - 1, kMaxStages, a.err);
+        int64_t hiB = 0, LB = 0, B = 0;
+        if (have) {
+            if (kCount) ++priced;
+            // pack the stages; a bound no split beats and a bound feasible
+            // whenever memory is (the entry's 32-byte row of stage bytes, read a byte
+            // per stage: an array indexed by the stage would live in local memory)
+            const uint8_t* row = a.wl_code + p * kMaxStages;
+            int next = __ldg(row);
             for (int s = 0; s < S; ++s) {
-                const uint32_t w = sw[s * kGBlock];
-                const int ri = (w & 7) * 4 + ((w >> 3) & 3);
-                const float rq = rqavg[ri], cf = cfl[(w >> 5) & 255];
-                // the run of layers memory admits, estimated from the
-                // average layer footprint
-                sw[s * kGBlock] = (w & kNoV) | ((uint32_t)layers_est(t, unpack(w, t), ri, kInf) << kVShift);
-                inv += rq;
-                cw += cf * rq;
-                if (rq > 0.f) flo = fmaxf(flo, cf + 1.0f / rq);
+                const int code = next;
+                next = s + 1 < S ? __ldg(row + s + 1) : 0;
+                const int gg = code & 7, jj = (code >> 3) & 3;
+                int pidx = kGZeroP2P;
+                if (s + 1 < S) {
+                    const int h = next & 7, jn = (next >> 3) & 3;
+                    pidx = (gg * 8 + h) * 2 + ((gg == h) && ((1 << jj) + (1 << jn) <= maxn[gg]));
+                }
+                const int f = min(S - s, M);
+                const uint32_t w = (uint32_t)(code & 31) | ((uint32_t)pidx << 5) | ((uint32_t)f << 13);
+                const GStage st = unpack(w, t);
+                // the first stage holds layer 0, the last one layer L - 1, the
+                // others at least one layer besides these
+                const int64_t least = s == 0       ? t.P[st.row + 1] - t.P[st.row]
+                                      : s + 1 == S ? t.P[st.row + L] - t.P[st.row + L - 1]
+                                                   : t.minmid[gg * 4 + jj];
+                LB = max(LB, least + st.c);
+                hiB = max(hiB, t.P[st.row + L] + st.c);
+                sw[s * kGBlock] = w;
             }
-            const float fhi = u64_to_float((uint64_t)hiB);
-            float Bf = fmaxf(flo, inv > 0.f ? ((float)L + 0.5f * (float)S + cw) / inv : flo);
-            for (int it = 0; it < 3; ++it) {
-                Bf = fminf(Bf, fhi);
-                float cnt = 0.f, sl = 0.f, nb = 0.f;
+            // first guess: the saturating continuous balance with each stage's
+            // average layer time and memory run from layer 0
+            {
+                float inv = 0.f, cw = 0.f, flo = 0.f;
                 for (int s = 0; s < S; ++s) {
                     const uint32_t w = sw[s * kGBlock];
-                    const float rq = rqavg[(w & 7) * 4 + ((w >> 3) & 3)], cf = cfl[(w >> 5) & 255];
-                    const float mr = (float)((w >> kVShift) & 255);
-                    const float x = (Bf - cf) * rq;
-                    if (rq <= 0.f || x >= mr) {
-                        cnt += mr;
-                    } else {
-                        cnt += x;
-                        sl += rq;
-                        nb += 1.f;
+                    const int ri = (w & 7) * 4 + ((w >> 3) & 3);
+                    const float rq = rqavg[ri], cf = cfl[(w >> 5) & 255];
+                    // the longest run of layers memory admits
+                    sw[s * kGBlock] = (w & kNoV) | ((uint32_t)t.win[ri * 33 + ((w >> 13) & 63)] << kVShift);
+                    inv += rq;
+                    cw += cf * rq;
+                    if (rq > 0.f) flo = fmaxf(flo, cf + 1.0f / rq);
+                }
+                const float fhi = u64_to_float((uint64_t)hiB);
+                float Bf = fmaxf(flo, inv > 0.f ? ((float)L + 0.5f * (float)S + cw) / inv : flo);
+                for (int it = 0; it < 3; ++it) {
+                    Bf = fminf(Bf, fhi);
+                    float cnt = 0.f, sl = 0.f, nb = 0.f;
+                    for (int s = 0; s < S; ++s) {
+                        const uint32_t w = sw[s * kGBlock];
+                        const float rq = rqavg[(w & 7) * 4 + ((w >> 3) & 3)], cf = cfl[(w >> 5) & 255];
+                        const float mr = (float)((w >> kVShift) & 255);
+                        const float x = (Bf - cf) * rq;
+                        if (rq <= 0.f || x >= mr) {
+                            cnt += mr;
+                        } else {
+                            cnt += x;
+                            sl += rq;
+                            nb += 1.f;
+                        }
+                    }
+                    const float tgt = (float)L + 0.5f * nb;
+                    if (cnt >= tgt - 0.25f || sl <= 0.f) break;
+                    Bf += (tgt - cnt) / sl;
+                }
+                B = (int64_t)float_to_u64(fmaxf(fminf(Bf, fhi), 0.f));
+            }
+        }
+        // The threshold search on [lo, hi]; where the screen could not decide
+        // memory it begins with a probe of memory alone.  One pass of the
+        // loop is one stage of the lane's current probe: a lane whose probe
+        // ends starts its next one in the next pass, so the lanes of a warp
+        // wait for one another once per entry and not once per probe.
+        //
+        // An undecided bound moves lo like an infeasible one, but not
+        // lo_proven: the bracket left at the end goes to the warp kernel.
+        // The gallop's first step is the next breakpoint, then 2^-7 of the
+        // bound and doubling: with layers that differ the breakpoints lie too
+        // close for steps that start from 1 ns (at most 14 probes on the
+        // ragged 80-layer profile, not 32).
+        int64_t lo = LB, hi = hiB, lo_proven = LB, step = 1, shi = -1, slo = kInf;
+        bool lo_known = false, hi_known = false, oom = false, undecided = false, back = false;
+        int it = 0, s = 0, u = 0, doubts = 0;
+        const int64_t guess = min(max(B, lo), hi - 1);
+        B = memok ? guess : kNoBound;
+        bool run = have && !(memok && lo >= hi);
+        while (__any_sync(kFull, run)) {
+            if (!run) continue;
+            const uint32_t w = sw[s * kGBlock];
+            sw[s * kGBlock] = (w & kNoV) | ((uint32_t)u << kVShift);
+            const GStage st = unpack(w, t);
+            const bool last = s + 1 == S;
+            int64_t acc, rej;
+            int r = reach_of(t, st, (w & 7) * 4 + ((w >> 3) & 3), u, L - (S - 1 - s), last, B, acc, rej);
+            slo = min(slo, rej);
+            if (kCount) checks += 2;
+            if (r == u && !last) {
+                // layer u alone does not fit: the largest end at or below u
+                back = true;
+                for (; r > s; --r) {
+                    if (kCount) ++checks;
+                    if (fits_mem(t, st, r - 1, r)) {
+                        const int64_t v = cost(t, st, r - 1, r);
+                        if (v <= B) break;
+                        slo = min(slo, v);
                     }
                 }
-                const float tgt = (float)L + 0.5f * nb;
-                if (cnt >= tgt - 0.25f || sl <= 0.f) break;
-                Bf += (tgt - cnt) / sl;
             }
-            B = (int64_t)float_to_u64(fmaxf(fminf(Bf, fhi), 0.f));
+            const bool fails = last ? r < L : r < s + 1;
+            if (!fails) shi = max(shi, acc);
+            u = r;
+            ++s;
+            if (!fails && !last) continue;
+            // ---- the probe's answer moves the bracket
+            if (kCount) ++probes;
+            bool feasible = !fails, unsure = false;
+            if (feasible && back) {
+                shi = split_below(t, sw, S, B);
+                feasible = shi >= 0;
+                unsure = !feasible;
+            }
+            if (B == kNoBound) {
+                // memory only: OOM, else a tighter feasible bound
+                run = feasible && lo < shi;
+                oom = fails;
+                undecided = unsure;
+                hi = feasible ? shi : hi;
+                if (lo >= hi) lo_proven = hi;
+                B = min(guess, hi - 1);
+            } else {
+                if (feasible) {
+                    hi = shi;
+                    hi_known = true;
+                } else {
+                    lo = unsure ? B + 1 : min(slo, hi);
+                    if (!unsure) lo_proven = lo;
+                    lo_known = true;
+                }
+                if (!lo_known) {
+                    B = hi - step;
+                    step = max(2 * step, hi >> kStepShift);
+                } else if (!hi_known) {
+                    B = lo + step - 1;
+                    step = max(2 * step, lo >> kStepShift);
+                } else {
+                    B = lo + (hi - lo) / 2;
+                }
+                if (unsure) ++doubts;
+                run = lo < hi && doubts < kMaxDoubts;
+                if (++it > kGMaxIters) {
+                    atomicOr(a.err, kErrSearchBound);
+                    run = false;
+                }
+                B = min(max(B, lo), hi - 1);
+            }
+            s = u = 0;
+            shi = -1;
+            slo = kInf;
+            back = false;
         }
-        // the threshold search (heddle_wsearch.cu's bracketing) from LB
-        int64_t lo = LB, hi = hiB, step = 1;
-        bool lo_known = false, hi_known = false, undecided = false;
-        int it = 0;
-        B = min(max(B, lo), hi - 1);
-        while (lo < hi) {
-            ++probes;
-            const int got = gprobe(t, sw, S, B, shi, slo, checks);
-            if (got == kUndecided) {
-                undecided = true;
-                break;
-            }
-            if (got == kFeasible) {
-                hi = shi;
-                hi_known = true;
-            } else {
-                lo = min(slo, hi);
-                lo_known = true;
-            }
-            if (!lo_known) {
-                B = hi - step;
-                step *= 2;
-            } else if (!hi_known) {
-                B = lo + step - 1;
-                step *= 2;
-            } else {
-                B = lo + (hi - lo) / 2;
-            }
-            if (++it > kGMaxIters) {
-                atomicOr(a.err, kErrSearchBound);
-                lo = hi;
-            }
-            B = min(max(B, lo), hi - 1);
+        if (!have) continue;
+        if (oom) {
+            a.T[c] = -1;
+            a.B[c] = -1;
+            a.ndp[c] = (uint16_t)n;
+            a.status[c] = HEDDLE_CAND_OOM;
+            a.wl_T[p] = -1;
+            if (a.bounds)
+                for (int q = 0; q <= kMaxStages; ++q) a.bounds[(int64_t)q * a.bstride + c] = 0;
+            continue;
         }
         const int64_t Bstar = hi;
-        if (undecided) {
-            defer(a, p);
+        if (undecided || lo_proven < hi) {
+            defer(a, p, undecided ? -1 : hi, lo_proven, hi_known);
             continue;
         }
         // the split: the smallest start V_s from which stage s reaches
@@ -482,16 +541,10 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
             for (int s = S - 1; s >= 1; --s) {
                 const uint32_t w = sw[s * kGBlock];
                 const GStage st = unpack(w, t);
-                const int vv = v;
-                ++checks;
-                if (holds(t, st, vv - 1, vv, Bstar)) {
-                    // the most layers y + 1 ending at v that stage s holds, from the estimate
-                    const int y0 = (int)layers_est(t, st, (w & 7) * 4 + ((w >> 3) & 3), Bstar - st.c) - 1;
-                    const int y = last_ok(0, vv - 1 - s, y0, [&](int yy) {
-                        ++checks;
-                        return holds(t, st, vv - 1 - yy, vv, Bstar);
-                    });
-                    v = vv - 1 - y;
+                if (kCount) checks += 2;
+                const int from = start_of(t, st, (w & 7) * 4 + ((w >> 3) & 3), s, v, Bstar);
+                if (from < v) {
+                    v = from;
                 } else {
                     while (v < L - (S - s) && !holds(t, st, v, v + 1, Bstar)) ++v;
                     v = min(v, L - (S - s));
@@ -535,7 +588,7 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
             for (int s = S + 1; s <= kMaxStages; ++s) a.bounds[(int64_t)s * a.bstride + c] = 0;
         }
         if (bad) {
-            defer(a, p);  // the warp kernel writes the whole row
+            defer(a, p, Bstar, Bstar, true);  // the warp kernel writes the whole row
             continue;
         }
         if (tmax != Bstar) atomicOr(a.err, kErrInternal);

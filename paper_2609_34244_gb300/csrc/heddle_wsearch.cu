@@ -8,7 +8,8 @@
 // stage's average layer cost and its memory run from layer 0 (a few Newton
 // steps), then each probe snaps the bracket to the largest accepted or the
 // smallest rejected stage time and the next bound gallops from that value
-// (1, 2, 4, ... away) until both sides are known, then bisects.  The sets
+// (1 ns away, then 2^-7 of it and doubling) until both sides are known, then
+// bisects.  The sets
 // of the probe at B* give the canonical split; a feasible probe that closes
 // the bracket already holds them (every bound in [hi, B] takes the same
 // decisions), so only a bracket closed from below costs a final probe.
@@ -36,6 +37,7 @@ using wp::WarpArea;
 constexpr int kWBlock = 256;
 constexpr int kWarps = kWBlock / 32;
 constexpr int kMaxIters = 256;
+constexpr int kStepShift = 7;  // see heddle_gsearch.cu
 
 struct WTabs {
     const int64_t* qmax;  // [NT * 4] the most expensive single layer per (type, degree)
@@ -215,7 +217,19 @@ __global__ void __launch_bounds__(kWBlock, 3) wsearch_kernel(PriceArgs a, int th
         int64_t lo = 0, B = kInf, step = 1;
         bool lo_known = false, hi_known = false, oom = false;
         int phase = memok ? 1 : 0, it = 0;
-        if (memok) {
+        const int64_t left_hi = listed ? a.sv_T[e] : -1;
+        if (left_hi >= 0) {
+            // the bracket the thread-per-entry search left: hi is feasible,
+            // no bound below lo is
+            hi = left_hi;
+            lo = a.wl_T[p];
+            hi_known = a.sv_nM[e] != 0;
+            phase = lo >= hi ? 2 : 1;
+            B = lo >= hi   ? hi
+                : hi_known ? hi - 1
+                           : min(max(plain_guess(t.P, t.SA, mine.row, mine.c, mine.capk, mine.f, live, S, L, hi), lo),
+                                 hi - 1);
+        } else if (memok) {
             B = min(max(plain_guess(t.P, t.SA, mine.row, mine.c, mine.capk, mine.f, live, S, L, hi), lo), hi - 1);
             if (lo >= hi) {
                 phase = 2;
@@ -246,10 +260,10 @@ __global__ void __launch_bounds__(kWBlock, 3) wsearch_kernel(PriceArgs a, int th
                 }
                 if (!lo_known) {
                     B = hi - step;
-                    step *= 2;
+                    step = max(2 * step, hi >> kStepShift);
                 } else if (!hi_known) {
                     B = lo + step - 1;
-                    step *= 2;
+                    step = max(2 * step, lo >> kStepShift);
                 } else {
                     B = lo + (hi - lo) / 2;
                 }
