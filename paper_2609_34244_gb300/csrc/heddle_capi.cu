@@ -71,11 +71,8 @@ struct heddle_ctx {
     int64_t chunk = hd::kWorklistCap;
     // top-k merge scratch
     hd::TopkEntry* d_scratch = nullptr;
-    int32_t* d_scratch_count = nullptr;
     int scratch_blocks = 0;
-    hd::TopkEntry* d_scratch2 = nullptr;
-    int32_t* d_scratch2_count = nullptr;
-    int32_t* d_tickets = nullptr;  // [17], zero between top-k launches
+    hd::TopkMeet* d_meet = nullptr;  // zero between top-k launches
     // host-buffer path
     cudaStream_t s_h2d = nullptr, s_d2h = nullptr;
     // kStageSets staging sets: a batch's copies in wait only for the batch
@@ -480,20 +477,16 @@ heddle_status heddle_create(heddle_ctx** out, int32_t device) {
         return HEDDLE_E_CUDA;
     }
     x->num_sms = prop.multiProcessorCount;
-    x->scratch_blocks = 8 * x->num_sms;  // per-CTA lists of the top-k and of the fused search
+    x->scratch_blocks = 2 * x->num_sms;  // per-CTA lists of the top-k
     cudaError_t e = cudaMalloc(&x->d_flags, 4 * sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMemset(x->d_flags, 0, 4 * sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMalloc(&x->d_counters, 3 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(x->d_counters, 0, 3 * sizeof(unsigned long long));
     if (e == cudaSuccess)
-        e = cudaMalloc(&x->d_scratch, sizeof(hd::TopkEntry) * hd::kMaxTopK * x->scratch_blocks);
-    if (e == cudaSuccess) e = cudaMalloc(&x->d_scratch_count, sizeof(int32_t) * x->scratch_blocks);
+        e = cudaMalloc(&x->d_scratch, sizeof(hd::TopkEntry) * hd::kTopkListCap * x->scratch_blocks);
     if (e == cudaSuccess) e = alloc_worklist(x->wl[0]);
-    const int l2 = (x->scratch_blocks + 31) / 32;
-    if (e == cudaSuccess) e = cudaMalloc(&x->d_scratch2, sizeof(hd::TopkEntry) * hd::kMaxTopK * l2);
-    if (e == cudaSuccess) e = cudaMalloc(&x->d_scratch2_count, sizeof(int32_t) * l2);
-    if (e == cudaSuccess) e = cudaMalloc(&x->d_tickets, sizeof(int32_t) * 17);
-    if (e == cudaSuccess) e = cudaMemset(x->d_tickets, 0, sizeof(int32_t) * 17);
+    if (e == cudaSuccess) e = cudaMalloc(&x->d_meet, sizeof(hd::TopkMeet));
+    if (e == cudaSuccess) e = cudaMemset(x->d_meet, 0, sizeof(hd::TopkMeet));
 
     if (e != cudaSuccess) {
         heddle_destroy(x);
@@ -511,7 +504,6 @@ void heddle_destroy(heddle_ctx* x) {
     cudaFree(x->d_flags);
     cudaFree(x->d_counters);
     cudaFree(x->d_scratch);
-    cudaFree(x->d_scratch_count);
     for (int b = 0; b < heddle_ctx::kWlSets; ++b) {
         free_worklist(x->wl[b]);
         if (x->ev_searched[b]) cudaEventDestroy(x->ev_searched[b]);
@@ -520,9 +512,7 @@ void heddle_destroy(heddle_ctx* x) {
     for (int b = 0; b < 4; ++b)
         if (x->s_work[b]) cudaStreamDestroy(x->s_work[b]);
     if (x->ev_in) cudaEventDestroy(x->ev_in);
-    cudaFree(x->d_scratch2);
-    cudaFree(x->d_scratch2_count);
-    cudaFree(x->d_tickets);
+    cudaFree(x->d_meet);
     for (int b = 0; b < heddle_ctx::kStageSets; ++b) {
         cudaFree(x->st_S[b]);
         cudaFree(x->st_M[b]);
@@ -700,11 +690,8 @@ hd::TopkArgs topk_args(heddle_ctx* x, heddle_topk_state* state) {
     hd::TopkArgs a{};
     a.state = state;
     a.scratch = x->d_scratch;
-    a.scratch_count = x->d_scratch_count;
     a.max_blocks = x->scratch_blocks;
-    a.scratch2 = x->d_scratch2;
-    a.scratch2_count = x->d_scratch2_count;
-    a.tickets = x->d_tickets;
+    a.meet = x->d_meet;
     return a;
 }
 
@@ -813,6 +800,7 @@ heddle_status price_chunk(heddle_ctx* x, hd::PriceArgs& a, const heddle_candidat
         m.wl_T = survivors ? W.sv_T : W.T;
         m.wl_nM = survivors ? W.sv_nM : W.nM;
         m.wl_cap = hd::kWorklistCap;
+        m.survivors = survivors ? 1 : 0;
         m.thr = x->d_flags + 2;
         CU(hd::launch_topk_worklist(m, nb, x->num_sms, cs, nl ? nl + 2 : nullptr));
         if (x->time_phases) CU(cudaEventRecord(rec.e[4], cs));

@@ -233,6 +233,14 @@ inline int thread_search_min(int num_sms) { return num_sms * 32; }
 constexpr int kWlSurv = kWlMeta - 1;             // the survivor count (see PriceArgs::sv_count)
 
 
+// Entries a CTA of the top-k hands to the last one.
+constexpr int kTopkListCap = 128;
+// What the CTAs of one top-k launch share.
+struct TopkMeet {
+    int32_t tickets;  // CTAs that have handed over
+    int32_t entries;  // entries in the scratch list
+};
+
 struct TopkArgs {
     // results of a batch (heddle_topk) ...
     const uint16_t* M;
@@ -242,21 +250,16 @@ struct TopkArgs {
     int64_t n;
     int64_t base_index;
     heddle_topk_state* state;  // device, in/out
-    TopkEntry* scratch;        // [grid][kMaxTopK]
-    int32_t* scratch_count;    // [grid]
+    TopkEntry* scratch;        // [max_blocks * kTopkListCap]
     int32_t max_blocks;
+    TopkMeet* meet;            // all zero between launches
     // ... or the worklist of a priced chunk (heddle_price_topk)
     const int32_t* wl_count;
     const int32_t* wl_idx;
     const int64_t* wl_T;
     const uint32_t* wl_nM;
     int32_t wl_cap;
-    // second-level lists of the two-level merge (group lists of the
-    // one-launch worklist top-k), and that kernel's tickets: [16] per group,
-    // then one for the final merge; zero between launches
-    TopkEntry* scratch2;
-    int32_t* scratch2_count;
-    int32_t* tickets;
+    int32_t survivors;  // the worklist holds a threshold's survivors only
     // nullable: raised (atomicMax on the bits of a positive float) to the
     // new state's k-th key n*M / T in float times (1 - 2^-16) once the state
     // holds k entries.  Float conversions and the division are each within

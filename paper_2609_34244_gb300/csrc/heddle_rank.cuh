@@ -13,12 +13,14 @@
 
 namespace hd {
 
-typedef unsigned __int128 u128;
-
+// The products are 32 x 64 bits, compared as (upper 64, lower 32) bits.
 __device__ __forceinline__ bool better(const TopkEntry& a, const TopkEntry& b) {
-    const u128 l = (u128)a.nM * (u128)(uint64_t)b.T;
-    const u128 r = (u128)b.nM * (u128)(uint64_t)a.T;
-    if (l != r) return l > r;
+    const uint64_t Ta = (uint64_t)a.T, Tb = (uint64_t)b.T;
+    const uint64_t l0 = (uint64_t)a.nM * (uint32_t)Tb, r0 = (uint64_t)b.nM * (uint32_t)Ta;
+    const uint64_t l1 = (uint64_t)a.nM * (uint32_t)(Tb >> 32) + (l0 >> 32);
+    const uint64_t r1 = (uint64_t)b.nM * (uint32_t)(Ta >> 32) + (r0 >> 32);
+    if (l1 != r1) return l1 > r1;
+    if ((uint32_t)l0 != (uint32_t)r0) return (uint32_t)l0 > (uint32_t)r0;
     return a.idx < b.idx;
 }
 
@@ -59,29 +61,6 @@ __device__ inline void warp_offer(TopkEntry* list, int& cnt, int k, bool valid, 
         // re-check against the list as it is now (earlier lanes may have raised the bar)
         if (cnt < k || better(x, list[k - 1])) warp_insert(list, cnt, k, x);
     }
-}
-
-// One round of a warp's running top-32 of float keys: lane l holds the
-// (l+1)-th largest key so far (run); the round's 32 keys (one per lane) are
-// sorted by a bitonic network, reversed against run (the larger of each
-// pair is a bitonic sequence holding the 32 largest of both) and merged.
-__device__ __forceinline__ float warp_keep_top32(float run, float key) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int size = 2; size <= 32; size <<= 1)
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            const float o = __shfl_xor_sync(0xffffffffu, key, stride);
-            const bool desc = (lane & size) == 0 || size == 32;
-            key = (((lane & stride) == 0) == desc) ? fmaxf(key, o) : fminf(key, o);
-        }
-    float c = fmaxf(run, __shfl_sync(0xffffffffu, key, 31 - lane));
-#pragma unroll
-    for (int stride = 16; stride > 0; stride >>= 1) {
-        const float o = __shfl_xor_sync(0xffffffffu, c, stride);
-        c = (lane & stride) == 0 ? fmaxf(c, o) : fminf(c, o);
-    }
-    return c;
 }
 
 // Merge the sorted lists of the CTA's warps (lists[w], counts[w]) into

@@ -74,3 +74,38 @@ def test_topk_rising_batch_and_near_ties(heddle_lib, oracle_mod, k, n_top):
         _same_state(got2, exp2, "k=%d, %d best, second call" % (k, n_top))
     finally:
         h.heddle_destroy(ctx)
+
+
+@pytest.mark.parametrize("n", (1, 31, 32, 33, 127, 129, 1023, 1024, 1025, 2049, 40_000, 500_009))
+@pytest.mark.parametrize("kind", ("all_tie", "two_levels", "few_ok", "zero_time"))
+def test_topk_gather_edges(heddle_lib, oracle_mod, n, kind):
+    """Batch sizes around one entry a lane, one CTA and several, with ties
+    that overflow the gather (every throughput equal; half of them), fewer OK
+    entries than k, and iteration times of zero; two calls into one state."""
+    h = heddle_lib
+    rng = np.random.default_rng(n)
+    T = rng.integers(1 << 30, 1 << 40, 2 * n)
+    status = np.zeros(2 * n, np.uint8)
+    if kind == "all_tie":
+        T[:] = 1 << 35
+    elif kind == "two_levels":
+        T = np.where(rng.random(2 * n) < 0.5, 1 << 35, 1 << 34)
+    elif kind == "few_ok":
+        status[:] = 1
+        status[rng.choice(2 * n, min(2 * n, 5), replace=False)] = 0
+    else:
+        T[rng.random(2 * n) < 0.3] = 0
+    planes = {"T": T.astype(np.int64), "status": status, "n_dp": rng.integers(1, 3, 2 * n).astype(np.uint16)
+              if kind == "zero_time" else np.full(2 * n, 4, np.uint16), "M": np.full(2 * n, 16, np.uint16)}
+    ctx = h.heddle_create(0)
+    try:
+        for k in (1, 16, 64):
+            state = h.alloc_topk_state()
+            h.heddle_topk_reset(ctx, state, k)
+            for lo in (0, n):
+                got = _run_topk(h, ctx, {key: v[lo:lo + n] for key, v in planes.items()}, lo, state)
+                part = {key: v[:lo + n] for key, v in planes.items()}
+                exp = oracle_mod.topk(part, part["M"], k)
+                _same_state(got, exp, "%s n=%d k=%d up to %d" % (kind, n, k, lo + n))
+    finally:
+        h.heddle_destroy(ctx)
