@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
     }
     __syncthreads();
     if (end_of[1] < a.thread_min) return;
-    if (!wp::load_image(smem, a.img, y.bytes, &bar, a.err)) return;
+    if (!wp::load_image(smem, a.img, y.searchBytes, &bar, a.err)) return;
     {
         const int64_t* P = reinterpret_cast<const int64_t*>(smem + y.offP);
         // per (type, degree) 1 / the average layer time and the cheapest
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
     t.win = smem + y.offWin;
     t.L = L;
     const int32_t* maxn = reinterpret_cast<const int32_t*>(smem + y.offMaxN);
-    uint32_t* sw = reinterpret_cast<uint32_t*>(smem + ((y.bytes + 127u) & ~127u)) + threadIdx.x;
+    uint32_t* sw = reinterpret_cast<uint32_t*>(smem + ((y.searchBytes + 127u) & ~127u)) + threadIdx.x;
 
     unsigned long long checks = 0, probes = 0, priced = 0;
     // the entries filed in the depth buckets (every worklist entry)
@@ -626,7 +626,7 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
 
 template <bool kCount>
 cudaError_t launch(const PriceArgs& a, int num_sms, cudaStream_t st) {
-    const size_t smem = ((a.lay.bytes + 127u) & ~127u) + sizeof(uint32_t) * kMaxStages * kGBlock;
+    const size_t smem = ((a.lay.searchBytes + 127u) & ~127u) + sizeof(uint32_t) * kMaxStages * kGBlock;
     int per_sm = 0;
     const cudaError_t e = resident_blocks(reinterpret_cast<const void*>(&gsearch_kernel<kCount>), kGBlock, smem, &per_sm);
     if (e != cudaSuccess) return e;

@@ -43,9 +43,24 @@ __device__ __forceinline__ bool in_range(int64_t i, int64_t n, uint32_t* err) {
 constexpr uint32_t kTabBadValue = 1u;   // non-finite or negative per-layer cost
 constexpr uint32_t kTabTooLarge = 2u;   // a table total or P2P term above its limit
 
-// Byte layout of the cost-table image.  The pricing kernel copies the whole
-// image into shared memory with one bulk (TMA) copy per CTA, so every
-// section starts on a 16-byte boundary and the total is a multiple of 16.
+// What the screen looks up per stage byte and per type, in the form in which
+// it adds it up (see screen_kernel); one 16-byte-aligned section of the image.
+struct ScreenTabs {
+    float4 cap[kMaxTypes];      // capacity of class e in units of 2^e, plus 1/2
+    uint32_t desc[256];         // per stage byte: bit 31 inadmissible, else its demand per class
+    uint16_t run[32 * 33 + 256];  // [f * 32 + byte] the longest run of layers, kNoRun for none
+                                // (bytes above 31 are inadmissible and read on)
+    int32_t classes;            // 0: classes 0 and 3 decide, 1: 0, 2 and 3, 2: all four
+    int32_t pad[3];
+};
+static_assert(sizeof(ScreenTabs) % 16 == 0, "copied 16 bytes at a time");
+constexpr int kNoRun = 8192;  // above 32 runs of 255 layers
+// first bit of class e in a type's demand word (9, 8, 7 and 6 bits)
+__host__ __device__ constexpr int demand_shift(int e) { return e == 0 ? 0 : e == 1 ? 9 : e == 2 ? 17 : 24; }
+
+// Byte layout of the cost-table image.  The search kernels copy its first
+// searchBytes into shared memory with bulk (TMA) copies, so every section
+// starts on a 16-byte boundary and the totals are multiples of 16.
 struct Layout {
     int32_t L, NT;
     uint32_t offP;      // int64 [NT][4][L+1]   prefix of per-layer ns per (type, degree)
@@ -64,6 +79,8 @@ struct Layout {
     uint32_t offModel;  // int32 [4]             [0] every layer has the same state and
                         //                       activation bytes; [1] every layer has the
                         //                       same quantised cost per (type, degree)
+    uint32_t searchBytes;
+    uint32_t offScreen; // ScreenTabs
     uint32_t bytes;
 };
 
@@ -87,6 +104,8 @@ inline Layout make_layout(int L, int NT) {
     y.offCap = o;   o = align16(o + 4u * 8 * 4);
     y.offWin = o;   o = align16(o + 8u * 4 * 33);
     y.offModel = o; o = align16(o + 4u * 4);
+    y.searchBytes = o;
+    y.offScreen = o; o = align16(o + (uint32_t)sizeof(ScreenTabs));
     y.bytes = o;
     return y;
 }

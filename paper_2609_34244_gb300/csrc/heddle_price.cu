@@ -24,40 +24,39 @@
 namespace hd {
 namespace {
 
-__device__ __forceinline__ void write_rejected(const PriceArgs& a, int64_t c, int status, int64_t n) {
-    a.T[c] = -1;
-    a.B[c] = -1;
-    a.ndp[c] = (uint16_t)(status == HEDDLE_CAND_OOM ? n : 0);
-    a.status[c] = (uint8_t)status;
-    if (a.bounds)
-        for (int s = 0; s <= kMaxStages; ++s) a.bounds[(int64_t)s * a.bstride + c] = 0;
-}
-
 constexpr int kScreenBlock = 256;
 
-// floor(a / d) for 0 <= a < 2^16 and 1 <= d <= 256 as (a 2^8) ceil(2^24 / d)
-// / 2^32: the error a (ceil(2^24/d) - 2^24/d) / 2^24 < 2^-8 stays below 1/d,
-// the smallest distance from a / d up to the next integer
-__device__ __forceinline__ uint32_t div_small(uint32_t a, uint32_t d, const uint32_t* magic) {
-    return __umulhi(a << 8, magic[d]);
+// 1 / x to 1 ulp (infinity for zero)
+__device__ __forceinline__ float rcp(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
 
-// Per stage byte: bit 31 inadmissible; bits 24-26 type; bits 16-20 the bit
-// that adds the stage's units to its type's demand word; bits 0-10 the row
-// (type, degree) of the run table.
-__device__ __forceinline__ uint32_t stage_desc(int b, const Layout& y, const unsigned char* img, int moe) {
-    const int32_t* gmaxn = reinterpret_cast<const int32_t*>(img + y.offMaxN);
-    const int32_t* gpow2 = reinterpret_cast<const int32_t*>(img + y.offPow2);
-    const int32_t* ggpus = reinterpret_cast<const int32_t*>(img + y.offGpus);
-    const int g = b & 7, j = (b >> 3) & 3;
-    if ((b >> 5) != 0 || g >= y.NT || ggpus[g] <= 0 || (!moe && (1 << j) > gmaxn[g])) return 1u << 31;
-    const int unit = (1 << j) <= gmaxn[g] ? (1 << j) : gpow2[g];
-    const int uc = 31 - __clz(unit);
-    // the stage adds 2^(j - uc) units of 2^uc GPUs to field uc of its type's
-    // demand word (fields of 9, 8, 7 and 6 bits at bits 0, 9, 17, 24: at
-    // most 32 stages x 8 / 2^uc units)
-    const int off = uc == 0 ? 0 : uc == 1 ? 9 : uc == 2 ? 17 : 24;
-    return ((uint32_t)g << 24) | ((uint32_t)(j - uc + off) << 16) | (uint32_t)((g * 4 + j) * 33);
+// A small count as float: its bits under 2^23's exponent, less 2^23 (two
+// full-rate instructions; a conversion runs at a quarter of the rate).
+__device__ __forceinline__ float small_float(uint32_t n) { return __uint_as_float(n | 0x4b000000u) - 8388608.0f; }
+
+// min over the classes of (capacity + 1/2) / demand for one type, whose floor
+// is min floor(capacity / demand): the exact ratio lies at least
+// 1 / (2 demand) from a whole number, and capacities (at most 65,535) times
+// the rounding of two operations (2^-22) stay below 1/2.  A class without
+// demand gives infinity.
+template <int kClasses>
+__device__ __forceinline__ float type_ratio(uint32_t v, const float4& cap) {
+    float r = cap.x * rcp(small_float(v & 0x1ffu));
+    if (kClasses >= 2) r = fminf(r, cap.y * rcp(small_float((v >> 9) & 0xffu)));
+    if (kClasses >= 1) r = fminf(r, cap.z * rcp(small_float((v >> 17) & 0x7fu)));
+    return fminf(r, cap.w * rcp(small_float(v >> 24)));
+}
+
+template <int kClasses>
+__device__ __forceinline__ float min_ratio(const uint32_t* dem, const float4* cap, int NT) {
+    float r = __int_as_float(0x7f800000);
+    for (int g0 = 0; g0 < NT; g0 += 4)  // types past NT hold no demand
+#pragma unroll
+        for (int g = g0; g < g0 + 4; ++g) r = fminf(r, type_ratio<kClasses>(dem[g * kScreenBlock], cap[g]));
+    return r;
 }
 
 // Steps 1-2 and the memory screen for every candidate of the batch.  Each
@@ -66,26 +65,29 @@ __device__ __forceinline__ uint32_t stage_desc(int b, const Layout& y, const uns
 // (16-byte vector copies when the planes are aligned), the candidates are
 // counting-sorted by S, and thread i screens the i-th of that order, so the
 // lanes of a warp run stage loops of nearly equal length.
+//
+// Instructions bound it (and the search that overlaps it), so the tables are
+// kept in the form in which a stage adds them up: one word that adds the
+// stage to every class of its type's demand, one run length that marks "no
+// layer fits" in its size; the DP degree is one minimum of float ratios over
+// the classes that can decide on this cluster.  @FIG@
 __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
-    __shared__ uint32_t desc[256];
-    __shared__ uint8_t win[8 * 4 * 33];
-    __shared__ __align__(16) uint32_t cap[8 * 4];
-    __shared__ uint32_t magic[257];
-    __shared__ uint32_t dem[8 * kScreenBlock];  // per-thread units per class (see stage_desc), per type
+    __shared__ ScreenTabs tab;
+    __shared__ uint32_t dem[8 * kScreenBlock];  // per-thread demand word (see stage_desc), per type
     __shared__ __align__(16) uint8_t tile[kMaxStages * kScreenBlock];  // [stage][candidate of the slice]
     __shared__ uint8_t sS[kScreenBlock];
     __shared__ uint16_t sM[kScreenBlock];
     __shared__ uint8_t order[kScreenBlock];
+    __shared__ uint16_t sn[kScreenBlock];  // OOM: the DP degree
+    __shared__ uint8_t sstatus[kScreenBlock];
     __shared__ int bins[kMaxStages + 3];
     __shared__ int smax;
     const Layout& y = a.lay;
     const int L = y.L;
     {
-        const int32_t* gcap = reinterpret_cast<const int32_t*>(a.img + y.offCap);
-        for (int i = threadIdx.x; i < 256; i += blockDim.x) desc[i] = stage_desc(i, y, a.img, a.moe);
-        for (int i = threadIdx.x; i < 32; i += blockDim.x) cap[i] = (uint32_t)gcap[i];
-        for (int i = threadIdx.x; i < 8 * 4 * 33; i += blockDim.x) win[i] = a.img[y.offWin + i];
-        for (int i = threadIdx.x; i < 257; i += blockDim.x) magic[i] = i >= 1 ? ((1u << 24) + i - 1) / i : 0;
+        const uint4* from = reinterpret_cast<const uint4*>(a.img + y.offScreen);
+        uint4* to = reinterpret_cast<uint4*>(&tab);
+        for (int i = threadIdx.x; i < (int)(sizeof(ScreenTabs) / 16); i += kScreenBlock) to[i] = __ldg(from + i);
     }
     const bool memuni = reinterpret_cast<const int32_t*>(a.img + y.offModel)[0] != 0;
     const int s_lim = min(min(kMaxStages, a.s_max), L);
@@ -158,7 +160,7 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
         const bool live = threadIdx.x < nloc;  // padding sorts last
         const int64_t c = c0 + ci;
         int S = 0, M = 0, status = HEDDLE_CAND_INVALID;
-        int64_t n = 0;
+        int n = 0;
         if (live) {
             S = sS[ci] & 0x3f;
             M = sM[ci];
@@ -167,50 +169,31 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
 #pragma unroll
                 for (int g = 0; g < 8; ++g) mydem[g * kScreenBlock] = 0;
                 uint32_t bad = 0;
-                int run_sum = 0, run_min = 255;
+                int run_sum = 0;
                 const uint8_t* col = tile + ci;
+                const int f_lim = min(M, kMaxStages) * 32;
+                int f = S * 32;
+#pragma unroll 4
                 for (int s = 0; s < S; ++s) {
-                    const uint32_t d = desc[col[s * kScreenBlock]];
+                    const int b = col[s * kScreenBlock];
+                    const uint32_t d = tab.desc[b];
                     bad |= d;
-                    const int g = (d >> 24) & 7;
-                    mydem[g * kScreenBlock] += 1u << ((d >> 16) & 31);
-                    const int wi = (d & 0x7ff) + min(S - s, M);
-                    const int w = win[wi];
-                    run_sum += w;
-                    run_min = min(run_min, w);
+                    mydem[(b & 7) * kScreenBlock] += d;
+                    run_sum += tab.run[min(f, f_lim) + b];
+                    f -= 32;
                 }
-                if (bad >> 31) {
-                    status = HEDDLE_CAND_INVALID;
-                } else {
-                    // n = min over (type, class e) of capacity / GPUs in units
-                    // >= 2^e; a class with no group of its own size is
-                    // dominated by the class above it.  Every type is
-                    // visited (an absent type's demand word is zero), so the
-                    // eight chains of loads are independent
-                    uint32_t nn = 0xffffffffu;
-#pragma unroll
-                    for (int g = 0; g < 8; ++g) {
-                        const uint32_t v = mydem[g * kScreenBlock];
-                        const uint4 cg = *reinterpret_cast<const uint4*>(cap + g * 4);
-                        // GPUs per class from the unit counts
-                        const uint32_t f3 = (v >> 24) << 3, f2 = ((v >> 17) & 0x7fu) << 2;
-                        const uint32_t f1 = ((v >> 9) & 0xffu) << 1, f0 = v & 0x1ffu;
-                        const uint32_t d3 = f3, d2 = d3 + f2, d1 = d2 + f1, d0 = d1 + f0;
-                        const uint32_t q3 = div_small(cg.w, d3, magic), q2 = div_small(cg.z, d2, magic);
-                        const uint32_t q1 = div_small(cg.y, d1, magic), q0 = div_small(cg.x, d0, magic);
-                        nn = min(nn, min(min(f3 ? q3 : 0xffffffffu, f2 ? q2 : 0xffffffffu),
-                                         min(f1 ? q1 : 0xffffffffu, f0 ? q0 : 0xffffffffu)));
-                    }
-                    n = nn;
-                    if (n == 0)
-                        status = HEDDLE_CAND_NO_FIT;
-                    else if (run_min < 1 || run_sum < L)
-                        status = HEDDLE_CAND_OOM;
-                    else
-                        status = HEDDLE_CAND_OK;
+                if (!(bad >> 31)) {
+                    const int cls = tab.classes;
+                    n = (int)(cls == 0   ? min_ratio<0>(mydem, tab.cap, y.NT)
+                              : cls == 1 ? min_ratio<1>(mydem, tab.cap, y.NT)
+                                         : min_ratio<2>(mydem, tab.cap, y.NT));
+                    status = n == 0                                  ? HEDDLE_CAND_NO_FIT
+                             : run_sum >= kNoRun || run_sum < L ? HEDDLE_CAND_OOM
+                                                                     : HEDDLE_CAND_OK;
                 }
             }
-            if (status != HEDDLE_CAND_OK) write_rejected(a, c, status, n);
+            sstatus[ci] = (uint8_t)status;
+            sn[ci] = (uint16_t)(status == HEDDLE_CAND_OOM ? n : 0);
         }
         // compact the candidates that need the search (one atomic per warp)
         const bool take = live && status == HEDDLE_CAND_OK;
@@ -243,16 +226,27 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
             }
             // each taken candidate's row of 32 stage bytes, written by the
             // whole warp (lane = stage; zero past its depth)
-            for (unsigned m = mask; m; m &= m - 1) {
-                const int src = __ffs(m) - 1;
-                const int pc = __shfl_sync(0xffffffffu, p, src);
-                const int cc = __shfl_sync(0xffffffffu, ci, src);
-                const int Sc = __shfl_sync(0xffffffffu, S, src);
+            const int where = ci | (S << 8);
+            int pc = base;
+            for (unsigned m = mask; m; m &= m - 1, ++pc) {
+                const int from = __shfl_sync(0xffffffffu, where, __ffs(m) - 1);
                 if (pc < a.wl_cap)
-                    a.wl_code[(int64_t)pc * kMaxStages + lane] = lane < Sc ? tile[lane * kScreenBlock + cc] : 0;
+                    a.wl_code[(int64_t)pc * kMaxStages + lane] =
+                        lane < (from >> 8) ? tile[lane * kScreenBlock + (from & 0xff)] : 0;
             }
         }
         __syncthreads();  // the tile, S, M and order are reused by the next slice
+        // the rejected candidates' results, in candidate order (coalesced;
+        // sn and sstatus are next written three barriers on)
+        if (threadIdx.x < nloc && sstatus[threadIdx.x] != HEDDLE_CAND_OK) {
+            const int64_t r = c0 + threadIdx.x;
+            a.T[r] = -1;
+            a.B[r] = -1;
+            a.ndp[r] = sn[threadIdx.x];
+            a.status[r] = sstatus[threadIdx.x];
+            if (a.bounds)
+                for (int s = 0; s <= kMaxStages; ++s) a.bounds[(int64_t)s * a.bstride + r] = 0;
+        }
     }
 }
 

@@ -36,6 +36,20 @@ __device__ int64_t round_half_away(double v) {
 
 __device__ int64_t ceil_div(u128 a, u128 b) { return (int64_t)((a + b - 1) / b); }
 
+// Per stage byte: inadmissible (bit 31), or what the stage adds to its
+// type's demand word -- per class e the GPUs of groups placed in units of at
+// least 2^e GPUs, in units of 2^e (a stage of 2^j GPUs is placed whole, or, on
+// a type whose nodes are smaller, in the largest power of two a node holds).
+__device__ uint32_t stage_desc(int b, int NT, int moe, const int32_t* gpus, const int32_t* maxn,
+                               const int32_t* pow2) {
+    const int g = b & 7, j = (b >> 3) & 3;
+    if ((b >> 5) != 0 || g >= NT || gpus[g] <= 0 || (!moe && (1 << j) > maxn[g])) return 1u << 31;
+    const int unit = (1 << j) <= maxn[g] ? (1 << j) : pow2[g];
+    uint32_t d = 0;
+    for (int e = 0; (1 << e) <= unit && e < 4; ++e) d += (uint32_t)((1 << j) >> e) << demand_shift(e);
+    return d;
+}
+
 __global__ void __launch_bounds__(kThreads) build_tables_kernel(TableArgs a) {
     const Layout& y = a.lay;
     const int L = y.L, NT = y.NT;
@@ -205,6 +219,28 @@ __global__ void __launch_bounds__(kThreads) build_tables_kernel(TableArgs a) {
             }
         }
         win[t] = (uint8_t)best;
+    }
+    __syncthreads();
+
+    // the screen's tables
+    ScreenTabs* sc = reinterpret_cast<ScreenTabs*>(a.img + y.offScreen);
+    for (int b = tid; b < 256; b += blockDim.x) sc->desc[b] = stage_desc(b, NT, a.moe, gpus, maxn, pow2);
+    for (int t = tid; t < 32 * 33 + 256; t += blockDim.x) {
+        const int f = t / 32, b = t & 31;
+        const int w = f >= 1 && f <= 32 ? win[((b & 7) * 4 + (b >> 3)) * 33 + f] : 0;
+        sc->run[t] = (uint16_t)(w ? w : kNoRun);
+    }
+    if (tid < kMaxTypes)
+        sc->cap[tid] = make_float4((float)cap[tid * 4] + 0.5f, (float)(cap[tid * 4 + 1] >> 1) + 0.5f,
+                                   (float)(cap[tid * 4 + 2] >> 2) + 0.5f, (float)(cap[tid * 4 + 3] >> 3) + 0.5f);
+    if (tid == 0) {
+        // a class whose capacity equals the class below's is dominated by it
+        // (no less demand on the same GPUs)
+        int need = 0;
+        for (int g = 0; g < NT; ++g)
+            for (int e = 1; e < 4; ++e)
+                if (cap[g * 4 + e] != cap[g * 4 + e - 1]) need |= 1 << e;
+        sc->classes = (need & 2) ? 2 : (need & 4) ? 1 : 0;
     }
 
     // P2P: forward activation plus backward gradient (2 x boundary bytes)

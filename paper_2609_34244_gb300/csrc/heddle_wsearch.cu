@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(kWBlock, 3) wsearch_kernel(PriceArgs a, int th
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ uint64_t bar;
     __shared__ int64_t qmax[4 * kMaxTypes], single[2];
-    if (!wp::load_image(smem, a.img, a.lay.bytes, &bar, a.err)) return;
+    if (!wp::load_image(smem, a.img, a.lay.searchBytes, &bar, a.err)) return;
     const Layout& y = a.lay;
     {
         // the most expensive single layer per (type, degree), and the
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(kWBlock, 3) wsearch_kernel(PriceArgs a, int th
     t.L = y.L;
     const int L = y.L;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    WarpArea& wa = reinterpret_cast<WarpArea*>(smem + ((y.bytes + 127u) & ~127u))[warp];
+    WarpArea& wa = reinterpret_cast<WarpArea*>(smem + ((y.searchBytes + 127u) & ~127u))[warp];
 
     unsigned long long checks = 0, probes = 0, priced = 0;
     int bucketed = a.wl_count[1 + 1 + lane];  // depth 1 + lane
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(kWBlock, 3) wsearch_kernel(PriceArgs a, int th
 
 template <bool kCount>
 cudaError_t launch(const PriceArgs& a, int num_sms, cudaStream_t st, bool listed) {
-    const size_t smem = ((a.lay.bytes + 127u) & ~127u) + sizeof(WarpArea) * kWarps;
+    const size_t smem = ((a.lay.searchBytes + 127u) & ~127u) + sizeof(WarpArea) * kWarps;
     int per_sm = 0;
     const cudaError_t e = resident_blocks(reinterpret_cast<const void*>(&wsearch_kernel<kCount>), kWBlock, smem, &per_sm);
     if (e != cudaSuccess) return e;
