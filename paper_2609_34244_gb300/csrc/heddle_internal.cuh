@@ -58,6 +58,22 @@ constexpr int kNoRun = 8192;  // above 32 runs of 255 layers
 // first bit of class e in a type's demand word (9, 8, 7 and 6 bits)
 __host__ __device__ constexpr int demand_shift(int e) { return e == 0 ? 0 : e == 1 ? 9 : e == 2 ? 17 : 24; }
 
+// What the equal-layer search looks up per stage: by stage byte (type and
+// degree, 0 .. 31), by P2P index (kZeroP2P: no next stage) and by pair of
+// consecutive stage bytes.
+constexpr int kZeroP2P = 128;  // a zero entry after the 8 x 8 x 2 P2P table
+struct EqTabs {
+    int64_t q[32];          // one layer's time
+    int64_t p2p[130];       // P2P per index
+    uint64_t D[32];         // slowest NIC times degree
+    float rq[32];           // 1 / q (0 for a free layer)
+    float qf[32];
+    float cf[132];
+    float rD[32];           // 1 / D
+    uint8_t pair[33 * 32];  // [next byte, 32: none][byte] P2P index
+};
+static_assert(sizeof(EqTabs) % 16 == 0, "copied 16 bytes at a time");
+
 // Byte layout of the cost-table image.  The search kernels copy its first
 // searchBytes into shared memory with bulk (TMA) copies, so every section
 // starts on a 16-byte boundary and the totals are multiples of 16.
@@ -81,6 +97,7 @@ struct Layout {
                         //                       same quantised cost per (type, degree)
     uint32_t searchBytes;
     uint32_t offScreen; // ScreenTabs
+    uint32_t offEq;     // EqTabs (of the first layer's costs)
     uint32_t bytes;
 };
 
@@ -106,6 +123,7 @@ inline Layout make_layout(int L, int NT) {
     y.offModel = o; o = align16(o + 4u * 4);
     y.searchBytes = o;
     y.offScreen = o; o = align16(o + (uint32_t)sizeof(ScreenTabs));
+    y.offEq = o;    o = align16(o + (uint32_t)sizeof(EqTabs));
     y.bytes = o;
     return y;
 }
@@ -340,9 +358,31 @@ __device__ __forceinline__ float u128_to_float(u128 v) {
     return __fmaf_rn(u64_to_float((uint64_t)(v >> 64)), 18446744073709551616.0f, u64_to_float((uint64_t)v));
 }
 
+//
+// The usual sizes (a quotient below 2^31, C below 2^50) need 64 bits only:
+// the estimate is off by at most 2^-20 of the quotient, so the remainder
+// stays below 2^62 and is exact modulo 2^64, and the second estimate is off
+// by at most one.
 __device__ inline uint64_t ceil_div_u128(u128 A, uint64_t C, bool* ok) {
     const float rc = 1.0f / u64_to_float(C);
     const float e = u128_to_float(A) * rc;
+    if (e < 2147483648.0f && C < ((uint64_t)1 << 50)) {
+        uint64_t q = (uint32_t)e;
+        int64_t r = (int64_t)((uint64_t)A - q * C);
+        const int d = (int)(u64_to_float((uint64_t)(r < 0 ? -r : r)) * rc);
+        q += (int64_t)(r < 0 ? -d : d);
+        r -= (int64_t)(r < 0 ? -d : d) * (int64_t)C;
+        for (int it = 0; it < 3 && r < 0; ++it) {
+            --q;
+            r += (int64_t)C;
+        }
+        for (int it = 0; it < 3 && r >= (int64_t)C; ++it) {
+            ++q;
+            r -= (int64_t)C;
+        }
+        if (r < 0 || r >= (int64_t)C) *ok = false;
+        return q + (r != 0 ? 1 : 0);
+    }
     uint64_t q = e < 4.0e18f ? float_to_u64(e) : 4000000000000000000ull;
     for (int it = 0; it < 6; ++it) {
         const u128 qc = (u128)q * C;

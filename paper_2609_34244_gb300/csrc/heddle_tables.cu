@@ -260,6 +260,30 @@ __global__ void __launch_bounds__(kThreads) build_tables_kernel(TableArgs a) {
         }
         p2p[t] = c;
     }
+    __syncthreads();
+
+    // the equal-layer search's tables
+    EqTabs* eq = reinterpret_cast<EqTabs*>(a.img + y.offEq);
+    for (int b = tid; b < 32; b += blockDim.x) {
+        const int g = b & 7, j = b >> 3;
+        const int64_t v = g < NT ? P[(size_t)(g * 4 + j) * (L + 1) + 1] : 0;
+        eq->q[b] = v;
+        eq->rq[b] = v > 0 ? 1.0f / (float)v : 0.0f;
+        eq->qf[b] = (float)v;
+        const uint64_t D = (uint64_t)inter[g] << j;
+        eq->D[b] = D;
+        eq->rD[b] = D > 0 ? 1.0f / (float)D : 0.0f;
+    }
+    for (int i = tid; i < 130; i += blockDim.x) {
+        eq->p2p[i] = i < kZeroP2P ? p2p[i] : 0;
+        eq->cf[i] = i < kZeroP2P ? (float)p2p[i] : 0.0f;
+    }
+    for (int t = tid; t < 33 * 32; t += blockDim.x) {
+        const int b = t & 31, nx = t >> 5;
+        const int g = b & 7, h = nx & 7;
+        const int same = g == h && (1 << (b >> 3)) + (1 << (nx >> 3)) <= maxn[g];
+        eq->pair[t] = (uint8_t)(nx == 32 ? kZeroP2P : (g * 8 + h) * 2 + same);
+    }
 }
 
 }  // namespace
