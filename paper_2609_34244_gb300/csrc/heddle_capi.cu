@@ -28,14 +28,20 @@ struct heddle_ctx {
     // device tables
     Layout lay{};
     bool tables_ready = false;
-    int32_t model_flags[4] = {0, 0, 0, 0};  // copy of the image's model flags
+    // every layer has the same memory; the same cost per (type, degree)
+    int32_t model_flags[2] = {0, 0};
     int32_t search_mode = HEDDLE_SEARCH_AUTO;
     int32_t thread_min = -1;  // heddle_set_thread_search_min (< 0: the default)
     unsigned char* d_img = nullptr;
     size_t img_cap = 0;
     int64_t* d_q = nullptr;
     size_t q_cap = 0;
-    uint32_t* d_flags = nullptr;            // [0] table build, [1] device errors, [2] top-k threshold
+    // the table builds' inputs (pinned, device) and what they found
+    unsigned char* h_in = nullptr;
+    unsigned char* d_in = nullptr;
+    size_t in_cap = 0;
+    hd::ModelInfo* h_info = nullptr;        // pinned
+    uint32_t* d_flags = nullptr;            // [0] tiled table build, [1] device errors, [2] top-k threshold
     unsigned long long* d_counters = nullptr;  // [3]
     bool count_next = false;
     // search worklist scratch (hd::kWorklistCap candidates); the other
@@ -44,7 +50,7 @@ struct heddle_ctx {
     // streams, so one chunk's screen and search overlap the earlier
     // chunks' searches and top-k)
     struct Worklist {
-        int32_t* count = nullptr;   // hd::kWlMeta ints
+        int32_t* count = nullptr;   // hd::kWlMeta ints, and a top-k threshold
         int32_t* bucket = nullptr;  // [32][2^20]
         int32_t* idx = nullptr;
         uint16_t* n = nullptr;
@@ -109,7 +115,7 @@ struct heddle_ctx {
         size_t img_cap = 0;
         int64_t* q = nullptr;
         size_t q_cap = 0;
-        int32_t flags[4] = {0, 0, 0, 0};
+        int32_t flags[2] = {0, 0};
     };
     int32_t mbs_levels = 0;
     std::vector<double> mbs_profile;  // [levels][types][4][L] seconds, or empty
@@ -200,7 +206,7 @@ constexpr int64_t kMemLimit = (int64_t)1 << 50;
 // layers, profile (nullable: the synthetic formula) and boundary bytes.
 heddle_status build_image(heddle_ctx* x, const std::vector<heddle_layer>& layers, const double* profile,
                           int64_t boundary_bytes, Layout& lay, unsigned char** img, size_t* img_cap,
-                          int64_t** qtab, size_t* q_cap, int32_t model_flags[4]) {
+                          int64_t** qtab, size_t* q_cap, int32_t model_flags[2]) {
     const int NT = (int)x->types.size(), L = (int)layers.size();
     // the gradient term stays below 2^56 ns: 2 * sum(param) * 1e9 / slowest NIC
     {
@@ -219,50 +225,52 @@ heddle_status build_image(heddle_ctx* x, const std::vector<heddle_layer>& layers
     lay = hd::make_layout(L, NT);
     CU(grow(img, img_cap, lay.bytes));
     CU(grow(qtab, q_cap, sizeof(int64_t) * (size_t)NT * 4 * L));
-    heddle_gpu_type* d_types = nullptr;
-    heddle_node* d_nodes = nullptr;
-    heddle_layer* d_layers = nullptr;
-    double* d_prof = nullptr;
-    cudaError_t e = cudaMalloc(&d_types, sizeof(heddle_gpu_type) * NT);
-    if (e == cudaSuccess) e = cudaMalloc(&d_nodes, sizeof(heddle_node) * x->nodes.size());
-    if (e == cudaSuccess) e = cudaMalloc(&d_layers, sizeof(heddle_layer) * L);
-    const size_t nprof = (size_t)NT * 4 * L;
-    if (e == cudaSuccess && profile) e = cudaMalloc(&d_prof, sizeof(double) * nprof);
-    if (e == cudaSuccess)
-        e = cudaMemcpy(d_types, x->types.data(), sizeof(heddle_gpu_type) * NT, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
-        e = cudaMemcpy(d_nodes, x->nodes.data(), sizeof(heddle_node) * x->nodes.size(),
-                       cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
-        e = cudaMemcpy(d_layers, layers.data(), sizeof(heddle_layer) * L, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && d_prof) e = cudaMemcpy(d_prof, profile, sizeof(double) * nprof, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(*img, 0, lay.bytes);
-    if (e == cudaSuccess) e = cudaMemset(x->d_flags, 0, sizeof(uint32_t));
-    if (e == cudaSuccess) {
-        hd::TableArgs a{};
-        a.lay = lay;
-        a.types = d_types;
-        a.nodes = d_nodes;
-        a.n_nodes = (int32_t)x->nodes.size();
-        a.layers = d_layers;
-        a.profile = d_prof;
-        a.boundary_bytes = boundary_bytes;
-        a.moe = x->moe;
-        a.img = *img;
-        a.q = *qtab;
-        a.flags = x->d_flags;
-        e = hd::launch_tables(a, 0);
+    // the inputs packed into one pinned buffer and copied at once (the build
+    // used to allocate, copy and free each array: a third of the time a
+    // planner spent on reloading a small cluster and model)
+    const size_t b_types = hd::align16((uint32_t)(sizeof(heddle_gpu_type) * NT));
+    const size_t b_nodes = (sizeof(heddle_node) * x->nodes.size() + 15) & ~(size_t)15;
+    const size_t b_layers = hd::align16((uint32_t)(sizeof(heddle_layer) * L));
+    const size_t b_prof = profile ? sizeof(double) * (size_t)NT * 4 * L : 0;
+    const size_t total = b_types + b_nodes + b_layers + b_prof;
+    // nothing enqueued on any stream may still read the tables or the buffers
+    CU(cudaDeviceSynchronize());
+    if (x->in_cap < total) {
+        cudaFreeHost(x->h_in);
+        x->h_in = nullptr;
+        x->in_cap = 0;
+        size_t cap = 0;
+        CU(cudaMallocHost((void**)&x->h_in, total));
+        CU(grow(&x->d_in, &cap, total));
+        x->in_cap = total;
     }
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    uint32_t flags = 0;
-    if (e == cudaSuccess) e = cudaMemcpy(&flags, x->d_flags, sizeof(uint32_t), cudaMemcpyDeviceToHost);
+    unsigned char* h = x->h_in;
+    memcpy(h, x->types.data(), sizeof(heddle_gpu_type) * NT);
+    memcpy(h + b_types, x->nodes.data(), sizeof(heddle_node) * x->nodes.size());
+    memcpy(h + b_types + b_nodes, layers.data(), sizeof(heddle_layer) * L);
+    if (b_prof) memcpy(h + b_types + b_nodes + b_layers, profile, b_prof);
+    hd::TableArgs a{};
+    a.lay = lay;
+    a.types = reinterpret_cast<const heddle_gpu_type*>(x->d_in);
+    a.nodes = reinterpret_cast<const heddle_node*>(x->d_in + b_types);
+    a.n_nodes = (int32_t)x->nodes.size();
+    a.layers = reinterpret_cast<const heddle_layer*>(x->d_in + b_types + b_nodes);
+    a.profile = b_prof ? reinterpret_cast<const double*>(x->d_in + b_types + b_nodes + b_layers) : nullptr;
+    a.boundary_bytes = boundary_bytes;
+    a.moe = x->moe;
+    a.img = *img;
+    a.q = *qtab;
+    cudaError_t e = cudaMemcpyAsync(x->d_in, h, total, cudaMemcpyHostToDevice, 0);
+    if (e == cudaSuccess) e = hd::launch_tables(a, 0);
     if (e == cudaSuccess)
-        e = cudaMemcpy(model_flags, *img + lay.offModel, sizeof(int32_t) * 4, cudaMemcpyDeviceToHost);
-    cudaFree(d_types);
-    cudaFree(d_nodes);
-    cudaFree(d_layers);
-    if (d_prof) cudaFree(d_prof);
+        e = cudaMemcpyAsync(x->h_info, *img + lay.offModel, sizeof(hd::ModelInfo), cudaMemcpyDeviceToHost, 0);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) return fail(x, HEDDLE_E_CUDA, "cost-table build: %s", cudaGetErrorString(e));
+    uint32_t flags = 0;
+    for (int i = 0; i < hd::table_ctas(NT); ++i) flags |= x->h_info->flags[i];
+    model_flags[0] = x->h_info->mem_uniform;
+    model_flags[1] = 1;
+    for (int i = 0; i < 4 * NT; ++i) model_flags[1] &= x->h_info->row_uniform[i];
     if (flags & hd::kTabBadValue)
         return fail(x, HEDDLE_E_ARG, "a per-layer cost is negative, not finite or above 4e18 ns");
     if (flags & hd::kTabTooLarge)
@@ -424,7 +432,7 @@ heddle_status check_ready(heddle_ctx* x) {
 
 cudaError_t alloc_worklist(heddle_ctx::Worklist& w) {
     const size_t cap = hd::kWorklistCap;
-    cudaError_t e = cudaMalloc(&w.count, sizeof(int32_t) * hd::kWlMeta);
+    cudaError_t e = cudaMalloc(&w.count, sizeof(int32_t) * (hd::kWlMeta + 1));
     if (e == cudaSuccess) e = cudaMalloc(&w.bucket, sizeof(int32_t) * HEDDLE_MAX_STAGES * cap);
     if (e == cudaSuccess) e = cudaMalloc(&w.idx, sizeof(int32_t) * cap);
     if (e == cudaSuccess) e = cudaMalloc(&w.n, sizeof(uint16_t) * cap);
@@ -480,6 +488,7 @@ heddle_status heddle_create(heddle_ctx** out, int32_t device) {
     x->scratch_blocks = 2 * x->num_sms;  // per-CTA lists of the top-k
     cudaError_t e = cudaMalloc(&x->d_flags, 4 * sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMemset(x->d_flags, 0, 4 * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&x->h_info, sizeof(hd::ModelInfo));
     if (e == cudaSuccess) e = cudaMalloc(&x->d_counters, 3 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(x->d_counters, 0, 3 * sizeof(unsigned long long));
     if (e == cudaSuccess)
@@ -501,6 +510,9 @@ void heddle_destroy(heddle_ctx* x) {
     DeviceGuard dg(x->device);
     cudaFree(x->d_img);
     cudaFree(x->d_q);
+    cudaFree(x->d_in);
+    cudaFreeHost(x->h_in);
+    cudaFreeHost(x->h_info);
     cudaFree(x->d_flags);
     cudaFree(x->d_counters);
     cudaFree(x->d_scratch);
@@ -731,10 +743,12 @@ void fill_price_args(heddle_ctx* x, const heddle_candidates* c, const heddle_ctx
 // One chunk [lo, lo + nb) of cands into r: screen and search on `ws` with
 // worklist set W, then (with a state) the top-k over the chunk's searched
 // candidates on `cs`, after the search when ws != cs.  `a` holds the
-// call-wide fields; its chunk fields are set here.
+// call-wide fields; its chunk fields are set here.  `only`: the call's one
+// chunk, whose threshold lies behind the worklist's counters and is cleared
+// with them (one launch less); else the caller has cleared x->d_flags[2].
 heddle_status price_chunk(heddle_ctx* x, hd::PriceArgs& a, const heddle_candidates* c, const heddle_results* r,
                           int64_t lo, int64_t nb, int set, cudaStream_t ws, heddle_topk_state* state,
-                          cudaStream_t cs, bool tiled, uint8_t* tiling) {
+                          cudaStream_t cs, bool tiled, uint8_t* tiling, bool only = false) {
     heddle_status st;
     const heddle_ctx::Worklist& W = x->wl[set];
     a.wl_count = W.count;
@@ -754,7 +768,8 @@ heddle_status price_chunk(heddle_ctx* x, hd::PriceArgs& a, const heddle_candidat
     a.sv_idx = W.sv_idx;
     a.sv_T = W.sv_T;
     a.sv_nM = W.sv_nM;
-    a.thr = x->d_flags + 2;
+    a.thr = only ? reinterpret_cast<uint32_t*>(W.count + hd::kWlMeta) : x->d_flags + 2;
+    a.wl_clear = hd::kWlMeta + (only ? 1 : 0);
     a.topk_k = state ? &state->k : nullptr;
     a.S = c->S + lo;
     a.M = c->M + lo;
@@ -801,7 +816,7 @@ heddle_status price_chunk(heddle_ctx* x, hd::PriceArgs& a, const heddle_candidat
         m.wl_nM = survivors ? W.sv_nM : W.nM;
         m.wl_cap = hd::kWorklistCap;
         m.survivors = survivors ? 1 : 0;
-        m.thr = x->d_flags + 2;
+        m.thr = a.thr;
         CU(hd::launch_topk_worklist(m, nb, x->num_sms, cs, nl ? nl + 2 : nullptr));
         if (x->time_phases) CU(cudaEventRecord(rec.e[4], cs));
     }
@@ -844,7 +859,7 @@ heddle_status price_impl(heddle_ctx* x, const heddle_candidates* c, const heddle
     const bool pipe = c->n > chunk;
     // the threshold starts at zero for each call: the state may have been
     // reset or replaced since the last one
-    if (state) CU(cudaMemsetAsync(x->d_flags + 2, 0, sizeof(uint32_t), cs));
+    if (state && pipe) CU(cudaMemsetAsync(x->d_flags + 2, 0, sizeof(uint32_t), cs));
     if (pipe) {
         if ((st = ensure_pipeline(x)) != HEDDLE_OK) return st;
         CU(cudaEventRecord(x->ev_in, cs));
@@ -860,7 +875,7 @@ heddle_status price_impl(heddle_ctx* x, const heddle_candidates* c, const heddle
             if (used[b]) CU(cudaStreamWaitEvent(ws, x->ev_wl_free[b], 0));
             used[b] = true;
         }
-        if ((st = price_chunk(x, a, c, r, lo, nb, b, ws, state, cs, tiled, tiling)) != HEDDLE_OK) return st;
+        if ((st = price_chunk(x, a, c, r, lo, nb, b, ws, state, cs, tiled, tiling, !pipe)) != HEDDLE_OK) return st;
         if (pipe) CU(cudaEventRecord(x->ev_wl_free[b], state ? cs : ws));
     }
     if (pipe && !state)

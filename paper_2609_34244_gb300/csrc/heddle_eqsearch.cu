@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(kEqBlock, 1024 / kEqBlock) eq_search_kernel(Pr
     __syncthreads();
     const EqTabs& t = sh.tab;
     const int64_t* PB = reinterpret_cast<const int64_t*>(a.img + y.offPB);
-    const int64_t pbytes = reinterpret_cast<const int32_t*>(a.img + y.offModel)[2] ? PB[1] - PB[0] : -1;
+    const int64_t pbytes = reinterpret_cast<const ModelInfo*>(a.img + y.offModel)->grad_uniform ? PB[1] - PB[0] : -1;
     uint32_t* mysw = sh.sw + threadIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 

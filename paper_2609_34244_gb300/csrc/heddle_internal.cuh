@@ -74,6 +74,17 @@ struct EqTabs {
 };
 static_assert(sizeof(EqTabs) % 16 == 0, "copied 16 bytes at a time");
 
+// CTAs of the table build: one per (type, degree), one per type, one more.
+__host__ __device__ constexpr int table_ctas(int NT) { return 4 * NT + kMaxTypes + 1; }
+
+// What the build found out about the model; the host reads it back.
+struct ModelInfo {
+    int32_t mem_uniform;   // every layer has the same state and activation bytes
+    int32_t grad_uniform;  // every layer has the same gradient bytes
+    int32_t row_uniform[4 * kMaxTypes];  // every layer costs the same on this (type, degree)
+    uint32_t flags[table_ctas(kMaxTypes)];  // kTab* per CTA
+};
+
 // Byte layout of the cost-table image.  The search kernels copy its first
 // searchBytes into shared memory with bulk (TMA) copies, so every section
 // starts on a 16-byte boundary and the totals are multiples of 16.
@@ -85,16 +96,12 @@ struct Layout {
     uint32_t offP2P;    // int64 [8][8][2]       P2P ns (from, to, same-node)
     uint32_t offMem;    // int64 [8]             memory per GPU
     uint32_t offInter;  // int64 [8]             slowest NIC of the type
-    uint32_t offMinQ;   // int64 [NT][4]         cheapest single layer per (type, degree)
     uint32_t offMaxN;   // int32 [8]             largest node of the type
     uint32_t offPow2;   // int32 [8]             largest power of two <= largest node (<= 8)
     uint32_t offGpus;   // int32 [8]             GPUs of the type
-    uint32_t offCap;    // int32 [8][4]          sum over nodes of floor(gpus / 2^e) * 2^e
     uint32_t offWin;    // uint8 [8][4][33]      longest run of layers that fits memory per
                         //                       (type, degree, in-flight microbatches f)
-    uint32_t offModel;  // int32 [4]             [0] every layer has the same state and
-                        //                       activation bytes; [1] every layer has the
-                        //                       same quantised cost per (type, degree)
+    uint32_t offModel;  // ModelInfo
     uint32_t searchBytes;
     uint32_t offScreen; // ScreenTabs
     uint32_t offEq;     // EqTabs (of the first layer's costs)
@@ -114,13 +121,11 @@ inline Layout make_layout(int L, int NT) {
     y.offP2P = o;   o = align16(o + 8u * 8 * 8 * 2);
     y.offMem = o;   o = align16(o + 8u * 8);
     y.offInter = o; o = align16(o + 8u * 8);
-    y.offMinQ = o;  o = align16(o + 8u * NT * 4);
     y.offMaxN = o;  o = align16(o + 4u * 8);
     y.offPow2 = o;  o = align16(o + 4u * 8);
     y.offGpus = o;  o = align16(o + 4u * 8);
-    y.offCap = o;   o = align16(o + 4u * 8 * 4);
     y.offWin = o;   o = align16(o + 8u * 4 * 33);
-    y.offModel = o; o = align16(o + 4u * 4);
+    y.offModel = o; o = align16(o + (uint32_t)sizeof(ModelInfo));
     y.searchBytes = o;
     y.offScreen = o; o = align16(o + (uint32_t)sizeof(ScreenTabs));
     y.offEq = o;    o = align16(o + (uint32_t)sizeof(EqTabs));
@@ -146,7 +151,6 @@ struct TableArgs {
     int32_t moe;
     unsigned char* img;      // out
     int64_t* q;              // out [NT][4][L]
-    uint32_t* flags;         // out
 };
 cudaError_t launch_tables(const TableArgs& a, cudaStream_t st);
 
@@ -189,6 +193,7 @@ struct PriceArgs {
     int32_t* wl_bucket;  // [kMaxStages][wl_cap]: per depth S (row S - 1) the entries of
                          // that depth, in any order (equal-layer search)
     int32_t wl_cap;
+    int32_t wl_clear;    // ints of wl_count the screen's launch clears (kWlMeta, or one more with the threshold)
     int32_t uniform;     // search with the equal-layer closed form (model flags [0] and [1])
     int32_t mbs_shift;   // micro-batch size 2^shift: M >> shift micro-batches (invalid unless 2^shift | M)
     int32_t split_mode;  // 1: the paper's own split rule (distribute_kernel) instead of PartitionLayers

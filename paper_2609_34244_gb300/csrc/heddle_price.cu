@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
         uint4* to = reinterpret_cast<uint4*>(&tab);
         for (int i = threadIdx.x; i < (int)(sizeof(ScreenTabs) / 16); i += kScreenBlock) to[i] = __ldg(from + i);
     }
-    const bool memuni = reinterpret_cast<const int32_t*>(a.img + y.offModel)[0] != 0;
+    const bool memuni = reinterpret_cast<const ModelInfo*>(a.img + y.offModel)->mem_uniform != 0;
     const int s_lim = min(min(kMaxStages, a.s_max), L);
     const bool vec16 = ((reinterpret_cast<uintptr_t>(a.code) | (uintptr_t)a.stride) & 15) == 0;
     uint32_t* mydem = dem + threadIdx.x;
@@ -262,7 +262,7 @@ cudaError_t launch_warp_search(const PriceArgs& a, int num_sms, cudaStream_t st,
 cudaError_t launch_screen(const PriceArgs& a, int num_sms, cudaStream_t st, cudaEvent_t mid, int64_t* launches) {
     if (a.n <= 0) return cudaSuccess;
     if (a.n > a.wl_cap) return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemsetAsync(a.wl_count, 0, sizeof(int32_t) * kWlMeta, st);
+    cudaError_t e = cudaMemsetAsync(a.wl_count, 0, sizeof(int32_t) * a.wl_clear, st);
     if (e != cudaSuccess) return e;
     // one wave of resident CTAs, each looping over slices
     int screen_per_sm = 0;
