@@ -268,7 +268,11 @@ __device__ __forceinline__ void defer(const PriceArgs& a, int64_t p, int64_t hi,
 // warp kernel prices the whole worklist.  Five CTAs per SM at 90 registers a
 // thread: a cap that lets in six or eight measured 0.38 and 0.43 ms beside
 // 0.35 ms (profiled 80-layer model, 300,007 candidates).
-template <bool kCount>
+//
+// kMemOnly: only the probe of memory, ahead of the tiled search: an entry
+// without a split within memory is OOM, the others go on that search's list
+// with sv_T 0 (memory known) or -1 (undecided).
+template <bool kCount, bool kMemOnly>
 __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ uint64_t bar;
@@ -387,7 +391,7 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
             }
             // first guess: the saturating continuous balance with each stage's
             // average layer time and memory run from layer 0
-            {
+            if (!kMemOnly) {
                 float inv = 0.f, cw = 0.f, flo = 0.f;
                 for (int s = 0; s < S; ++s) {
                     const uint32_t w = sw[s * kGBlock];
@@ -441,7 +445,7 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
         int it = 0, s = 0, u = 0, doubts = 0;
         const int64_t guess = min(max(B, lo), hi - 1);
         B = memok ? guess : kNoBound;
-        bool run = have && !(memok && lo >= hi);
+        bool run = have && !(memok && (kMemOnly || lo >= hi));
         while (__any_sync(kFull, run)) {
             if (!run) continue;
             const uint32_t w = sw[s * kGBlock];
@@ -479,7 +483,7 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
             }
             if (B == kNoBound) {
                 // memory only: OOM, else a tighter feasible bound
-                run = feasible && lo < shi;
+                run = !kMemOnly && feasible && lo < shi;
                 oom = fails;
                 undecided = unsure;
                 hi = feasible ? shi : hi;
@@ -525,6 +529,10 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
             a.wl_T[p] = -1;
             if (a.bounds)
                 for (int q = 0; q <= kMaxStages; ++q) a.bounds[(int64_t)q * a.bstride + c] = 0;
+            continue;
+        }
+        if (kMemOnly) {
+            defer(a, p, undecided ? -1 : 0, 0, false);
             continue;
         }
         const int64_t Bstar = hi;
@@ -624,24 +632,28 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
     }
 }
 
-template <bool kCount>
+template <bool kCount, bool kMemOnly>
 cudaError_t launch(const PriceArgs& a, int num_sms, cudaStream_t st) {
     const size_t smem = ((a.lay.searchBytes + 127u) & ~127u) + sizeof(uint32_t) * kMaxStages * kGBlock;
     int per_sm = 0;
-    const cudaError_t e = resident_blocks(reinterpret_cast<const void*>(&gsearch_kernel<kCount>), kGBlock, smem, &per_sm);
+    const cudaError_t e = resident_blocks(reinterpret_cast<const void*>(&gsearch_kernel<kCount, kMemOnly>), kGBlock, smem, &per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     // the worklist length is only known on the device: one wave at most
     const int64_t need = (a.n + kGBlock - 1) / kGBlock;
     const int grid = (int)std::min<int64_t>(need, (int64_t)num_sms * per_sm);
-    gsearch_kernel<kCount><<<grid, kGBlock, smem, st>>>(a);
+    gsearch_kernel<kCount, kMemOnly><<<grid, kGBlock, smem, st>>>(a);
     return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_thread_search(const PriceArgs& a, int num_sms, cudaStream_t st) {
-    return a.counters ? launch<true>(a, num_sms, st) : launch<false>(a, num_sms, st);
+    return a.counters ? launch<true, false>(a, num_sms, st) : launch<false, false>(a, num_sms, st);
+}
+
+cudaError_t launch_memory_probe(const PriceArgs& a, int num_sms, cudaStream_t st) {
+    return launch<false, true>(a, num_sms, st);
 }
 
 }  // namespace hd

@@ -258,6 +258,11 @@ cudaError_t launch_plans(const PlanArgs& a, int num_sms, cudaStream_t st);
 cudaError_t launch_plan_mask(const uint8_t* n_tmpl, int slots, int t, const uint8_t* prev_status, uint8_t* skip,
                              int64_t n, int num_sms, cudaStream_t st);
 
+// Ahead of the tiled search (heddle_gsearch.cu): the entries no split fits
+// are priced OOM, the others listed at a.sv_idx (count at
+// wl_count[kWlGeneral]); does nothing below a.thread_min bucketed entries.
+cudaError_t launch_memory_probe(const PriceArgs& a, int num_sms, cudaStream_t st);
+
 // The paper's own layer split over the worklist (comparison mode).
 cudaError_t launch_distribute(const PriceArgs& a, int num_sms, cudaStream_t st);
 constexpr int32_t kWorklistCap = 1 << 20;

@@ -34,6 +34,7 @@
 //                  tilings and the smallest T wins (the smaller Y on ties).
 
 #include <algorithm>
+#include <climits>
 
 #include "heddle_tiled.cuh"
 #include "heddle_wprobe.cuh"
@@ -203,6 +204,13 @@ __global__ void __launch_bounds__(kTabThreads) tiled_tables_kernel(TiledTableArg
 
 // ------------------------------------------------------------------ search
 
+// The allowed, undominated tilings of a (type, degree): one for each EDP
+// exponent in most clusters, of up to ten.
+struct __align__(16) TileList {
+    uint8_t count;
+    uint8_t tiling[15];  // slot within the degree | EDP exponent << 4
+};
+
 struct TTabs {
     const int64_t* Pt;
     const longlong2* SA;
@@ -215,6 +223,7 @@ struct TTabs {
     const int32_t* maxn;
     const int64_t* intra;
     const uint8_t* code;
+    const TileList* lists;  // [8][4]
     int L;
 };
 
@@ -248,20 +257,21 @@ struct TiledCheck {
         r.f = __shfl_sync(wp::kFull, mine.f, s);
         return r;
     }
-    // not inlined: the probe calls it from several places, and inlined
-    // copies of its loop over the tilings made the kernel wait on
-    // instruction fetch
-    __device__ __noinline__ int eval(const TLane& st, int i, int e, int64_t B, int64_t* cost) const {
-        const int base = tile_base(st.j), cnt = (st.j + 1) * (st.j + 2) / 2;
+    __device__ __forceinline__ int eval(const TLane& st, int i, int e, int64_t B, int64_t* cost) const {
+        const longlong2 a = t.SA[i], b = t.SA[e];
+        const int64_t bare = (b.x - a.x) + st.f * (b.y - a.y), copies = t.ES[e] - t.ES[i];
+        const TileList& list = t.lists[st.g * 4 + st.j];
+        const int64_t* P = t.Pt + (size_t)(st.g * kTileSlots + tile_base(st.j)) * (t.L + 1);
+        const int cnt = list.count;
         int64_t best = kInf;
         for (int o = 0; o < cnt; ++o) {
-            const uint8_t cd = t.code[st.g * kTileSlots + base + o];
-            if ((cd & 0xc0) != 0x80) continue;  // not allowed, or dominated
-            if (!tfits(t, st, i, e, (cd >> 4) & 3)) continue;
-            const int64_t* P = t.Pt + (size_t)(st.g * kTileSlots + base + o) * (t.L + 1);
-            best = min(best, P[e] - P[i] + st.c);
+            const int cd = list.tiling[o];
+            const int64_t* row = P + (cd & 15) * (t.L + 1);
+            const int64_t v = row[e] - row[i];
+            if (bare + (((int64_t)1 << (cd >> 4)) - 1) * copies <= st.cap) best = min(best, v);
         }
         if (best == kInf) return 2;
+        best += st.c;
         *cost = best;
         return best <= B ? 0 : 1;
     }
@@ -301,9 +311,12 @@ __device__ __forceinline__ T pick4(const T (&v)[4], int k) {
     return k == 0 ? v[0] : k == 1 ? v[1] : k == 2 ? v[2] : v[3];
 }
 
-__global__ void __launch_bounds__(kTBlock, 3) tiled_search_kernel(PriceArgs a, TiledArgs ta) {
+// The entries launch_memory_probe listed, or the whole worklist when the depth
+// buckets hold fewer than thread_min entries (see wsearch_kernel).
+__global__ void __launch_bounds__(kTBlock, 3) tiled_search_kernel(PriceArgs a, TiledArgs ta, int thread_min) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ uint64_t bar;
+    __shared__ TileList lists[4 * kMaxTypes];
     if (!wp::load_image(smem, ta.timg, ta.tl.bytes, &bar, a.err)) return;
     const TiledLayout& y = ta.tl;
     TTabs t;
@@ -318,12 +331,27 @@ __global__ void __launch_bounds__(kTBlock, 3) tiled_search_kernel(PriceArgs a, T
     t.intra = reinterpret_cast<const int64_t*>(smem + y.offIntra);
     t.maxn = reinterpret_cast<const int32_t*>(smem + y.offMaxN);
     t.code = smem + y.offCode;
+    t.lists = lists;
     t.L = y.L;
+    if (threadIdx.x < 4 * kMaxTypes) {
+        const int g = threadIdx.x >> 2, j = threadIdx.x & 3;
+        int n = 0;
+        for (int o = 0; o < (j + 1) * (j + 2) / 2; ++o) {
+            const uint8_t cd = t.code[g * kTileSlots + tile_base(j) + o];
+            if ((cd & 0xc0) == 0x80) lists[threadIdx.x].tiling[n++] = (uint8_t)(o | (((cd >> 4) & 3) << 4));
+        }
+        lists[threadIdx.x].count = (uint8_t)n;
+    }
+    __syncthreads();
     const int L = y.L;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     wp::WarpArea& wa = reinterpret_cast<wp::WarpArea*>(smem + ((y.bytes + 127u) & ~127u))[warp];
     unsigned long long checks = 0;
-    const int64_t count = min((int64_t)*a.wl_count, (int64_t)a.wl_cap);
+    int bucketed = a.wl_count[1 + 1 + lane];  // depth 1 + lane
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) bucketed += __shfl_xor_sync(wp::kFull, bucketed, o);
+    const bool listed = bucketed >= thread_min;
+    const int64_t count = min((int64_t)(listed ? a.wl_count[kWlGeneral] : *a.wl_count), (int64_t)a.wl_cap);
     // each warp prices its own first entry, then the next untaken one
     // whenever it is free
     const int64_t first = (int64_t)gridDim.x * kTWarps;
@@ -332,7 +360,9 @@ __global__ void __launch_bounds__(kTBlock, 3) tiled_search_kernel(PriceArgs a, T
         if (lane == 0) e = atomicAdd(a.wl_count + kWlTakeWarp, 1);
         return first + __shfl_sync(wp::kFull, e, 0);
     };
-    for (int64_t p = (int64_t)blockIdx.x * kTWarps + warp; p < count; p = take()) {
+    for (int64_t e = (int64_t)blockIdx.x * kTWarps + warp; e < count; e = take()) {
+        const int64_t p = listed ? a.sv_idx[e] : e;
+        if (!in_range(p, a.wl_cap, a.err)) continue;
         const int64_t c = a.wl_idx[p];
         const int S = a.wl_S[p];
         if (!in_range(c, a.n, a.err) || !in_range(S - 1, kMaxStages, a.err)) continue;
@@ -361,9 +391,30 @@ __global__ void __launch_bounds__(kTBlock, 3) tiled_search_kernel(PriceArgs a, T
         int64_t Bhi = 0, Blo = 0, B = kInf, step = 1;
         bool lo_known = false, hi_known = false, oom = false;
         int phase = 0, it = 0;
+        if (listed && a.sv_T[e] >= 0) {
+            // a split within memory exists: each of its stages fits without
+            // EDP copies, so no stage takes longer than all layers on the
+            // fastest such tiling
+            int64_t most = 0;
+            if (live) {
+                const int base = tile_base(mine.j);
+                int64_t all = kInf;
+                for (int o = 0; o <= mine.j; ++o)  // (EDP exponent 0 comes first)
+                    if ((t.code[mine.g * kTileSlots + base + o] & 0xc0) == 0x80)
+                        all = min(all, t.Pt[(size_t)(mine.g * kTileSlots + base + o) * (L + 1) + L]);
+                most = all + mine.c;
+            }
+            Bhi = wp::wmax64(most);
+            phase = Bhi > 0 ? 1 : 2;
+            B = Bhi > 0 ? min(tiled_guess(t.code, t.Pt, t.SA, mine.g, mine.j, mine.c, mine.cap, mine.f, live, S, L,
+                                          Bhi),
+                              Bhi - 1)
+                        : Bhi;
+        }
         while (true) {
             int64_t hi, lo;
-            const bool feas = wp::probe(check, S, L, B, wa, hi, lo, checks);
+            const int quick = phase != 2 ? wp::forward_probe(check, S, L, B, hi, lo, checks) : -1;
+            const bool feas = quick >= 0 ? quick == 1 : wp::probe(check, S, L, B, wa, hi, lo, checks);
             if (phase == 0) {
                 if (!feas) {
                     oom = true;
@@ -532,7 +583,11 @@ cudaError_t launch_tiled_search(const PriceArgs& a, const TiledArgs& t, int num_
     // at most one wave
     const int64_t need = (a.n + kTWarps - 1) / kTWarps;
     const int grid = (int)std::min<int64_t>(need, (int64_t)num_sms * per_sm);
-    tiled_search_kernel<<<grid, kTBlock, smem, st>>>(a, t);
+    // the memory probe of a batch that cannot reach its threshold is not launched
+    const bool listed = a.n >= a.thread_min;
+    cudaError_t e2 = listed ? launch_memory_probe(a, num_sms, st) : cudaSuccess;
+    if (e2 != cudaSuccess) return e2;
+    tiled_search_kernel<<<grid, kTBlock, smem, st>>>(a, t, listed ? a.thread_min : INT_MAX);
     return cudaGetLastError();
 }
 

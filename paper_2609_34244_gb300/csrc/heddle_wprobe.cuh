@@ -250,26 +250,20 @@ __device__ bool probe(const J& check, int S, int L, int64_t B, WarpArea& wa, int
     return feasible;
 }
 
-// The forward pass alone, for a bound B at which every stage could hold any
-// single layer of the model (its most expensive layer's time plus its P2P
-// within B, and the largest single-layer state and activation within its
-// memory; the caller checks this).  Then, by induction, the feasible
-// stage-s ends form the interval [s, U_s]: positions up to U_{s-1} + 1 are
-// reached one layer after their predecessor, those beyond only from U_{s-1}
-// (the largest predecessor dominates), so B is feasible iff the last stage
-// fits [U_{S-1}, L), and the chain of U_s is a split attaining every
-// accepted stage time.  The snap values therefore mean what they mean for
-// probe(): every bound in [hi, B] is feasible, every bound in [B, lo) is
-// not (the interval property holds at any bound >= B).  No sets are built:
-// the canonical split needs probe() at B*.
+// The forward pass alone: 1 feasible, 0 infeasible, -1 it cannot tell.  While
+// every stage advances (it holds its first layer), U_{s+1} is attained and
+// no start reaches further, so if the last stage fits [U_{S-1}, L) the chain
+// itself is a split, and if not there is none.  The snap values mean what
+// they mean for probe(): every bound in [hi, B] is feasible, every bound in
+// [B, lo) is not.  A stage that does not hold the layer after U_s leaves the
+// answer to probe(), whose sets the canonical split at B* needs as well.
 template <class J>
-__device__ bool forward_probe(const J& check, int S, int L, int64_t B, int64_t& hi_out, int64_t& lo_out,
-                              unsigned long long& checks) {
+__device__ int forward_probe(const J& check, int S, int L, int64_t B, int64_t& hi_out, int64_t& lo_out,
+                             unsigned long long& checks) {
     const int lane = threadIdx.x & 31;
     int64_t hi = -1, lo = kInf;
-    bool ok = true;
     int u = 0;
-    for (int s = 0; s + 1 < S && ok; ++s) {
+    for (int s = 0; s + 1 < S; ++s) {
         const typename J::Stage st = check.stage(s);
         const int lim = L - (S - 1 - s);
         int reach = u;
@@ -290,11 +284,11 @@ __device__ bool forward_probe(const J& check, int S, int L, int64_t B, int64_t& 
             }
             reach = base + 31;
         }
-        if (reach < s + 1) ok = false;
+        if (reach == u) return -1;
         u = reach;
     }
     bool feasible = false;
-    if (ok) {
+    {
         const typename J::Stage st = check.stage(S - 1);
         if (lane == 0) {
             int64_t v = 0;
@@ -311,7 +305,7 @@ __device__ bool forward_probe(const J& check, int S, int L, int64_t B, int64_t& 
     }
     hi_out = wmax64(hi);
     lo_out = wmin64(lo);
-    return feasible;
+    return feasible ? 1 : 0;
 }
 
 // The first guess of B* (warp-uniform): the saturating continuous balance

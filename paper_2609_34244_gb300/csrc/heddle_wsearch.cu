@@ -40,8 +40,6 @@ constexpr int kMaxIters = 256;
 constexpr int kStepShift = 7;  // see heddle_gsearch.cu
 
 struct WTabs {
-    const int64_t* qmax;  // [NT * 4] the most expensive single layer per (type, degree)
-    int64_t smax, amax;   // the largest single-layer state and activation bytes
     const int64_t* P;
     const longlong2* SA;
     const int64_t* PB;
@@ -113,43 +111,9 @@ template <bool kCount>
 __global__ void __launch_bounds__(kWBlock, 3) wsearch_kernel(PriceArgs a, int thread_min) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ uint64_t bar;
-    __shared__ int64_t qmax[4 * kMaxTypes], single[2];
     if (!wp::load_image(smem, a.img, a.lay.searchBytes, &bar, a.err)) return;
     const Layout& y = a.lay;
-    {
-        // the most expensive single layer per (type, degree), and the
-        // largest single-layer state and activation, for the forward-only
-        // probe's condition
-        const int64_t* P = reinterpret_cast<const int64_t*>(smem + y.offP);
-        const longlong2* SA = reinterpret_cast<const longlong2*>(smem + y.offSA);
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        for (int r = warp; r <= 4 * y.NT; r += kWarps) {
-            int64_t m0 = 0, m1 = 0;
-            for (int l = lane; l < y.L; l += 32) {
-                if (r < 4 * y.NT) {
-                    m0 = max(m0, P[r * (y.L + 1) + l + 1] - P[r * (y.L + 1) + l]);
-                } else {
-                    m0 = max(m0, (int64_t)(SA[l + 1].x - SA[l].x));
-                    m1 = max(m1, (int64_t)(SA[l + 1].y - SA[l].y));
-                }
-            }
-            m0 = wp::wmax64(m0);
-            m1 = wp::wmax64(m1);
-            if (lane == 0) {
-                if (r < 4 * y.NT) {
-                    qmax[r] = m0;
-                } else {
-                    single[0] = m0;
-                    single[1] = m1;
-                }
-            }
-        }
-        __syncthreads();
-    }
     WTabs t;
-    t.qmax = qmax;
-    t.smax = single[0];
-    t.amax = single[1];
     t.P = reinterpret_cast<const int64_t*>(smem + y.offP);
     t.SA = reinterpret_cast<const longlong2*>(smem + y.offSA);
     t.PB = reinterpret_cast<const int64_t*>(smem + y.offPB);
@@ -201,10 +165,6 @@ __global__ void __launch_bounds__(kWBlock, 3) wsearch_kernel(PriceArgs a, int th
             const int same = (g == h) && ((1 << j) + (1 << jn) <= t.maxn[g]);
             mine.c = t.p2p[(g * 8 + h) * 2 + same];
         }
-        // the forward-only probe is exact at bounds where every stage could
-        // hold any single layer (time and memory)
-        const int64_t qmc = live ? t.qmax[g * 4 + j] + mine.c : -1;
-        const bool memfit = !live || t.smax + mine.f * t.amax <= mine.capk;
         // a bound feasible whenever memory is
         int64_t hi = live ? t.P[mine.row + L] + mine.c : 0;
         hi = wp::wmax64(hi);
@@ -239,9 +199,9 @@ __global__ void __launch_bounds__(kWBlock, 3) wsearch_kernel(PriceArgs a, int th
         while (true) {
             int64_t shi, slo;
             if (kCount && lane == 0) ++probes;
-            const bool fast = phase != 2 && __all_sync(kFull, qmc <= B && memfit);
-            const bool feas = fast ? wp::forward_probe(check, S, L, B, shi, slo, checks)
-                                   : wp::probe(check, S, L, B, wa, shi, slo, checks);
+            const int quick = phase != 2 ? wp::forward_probe(check, S, L, B, shi, slo, checks) : -1;
+            const bool fast = quick >= 0;
+            const bool feas = fast ? quick == 1 : wp::probe(check, S, L, B, wa, shi, slo, checks);
             if (phase == 0) {
                 if (!feas) {
                     oom = true;
