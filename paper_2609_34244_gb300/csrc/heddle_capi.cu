@@ -139,8 +139,6 @@ struct heddle_ctx {
     bool nodes_on_device = false;  // d_node_* hold the loaded cluster's nodes
     uint8_t* plan_bounds[HEDDLE_MAX_TEMPLATES] = {nullptr, nullptr, nullptr, nullptr};
     size_t plan_bounds_cap[HEDDLE_MAX_TEMPLATES] = {0, 0, 0, 0};
-    uint8_t* skip_mask = nullptr;  // the plan slot being priced: candidates priced SKIPPED
-    size_t skip_mask_cap = 0;
     // expert tiling: the experts' byte counts and the tiled image
     bool have_experts = false, tiled_ready = false;
     std::vector<int64_t> expert_state, expert_param;
@@ -554,7 +552,6 @@ void heddle_destroy(heddle_ctx* x) {
     cudaFree(x->d_node_type);
     cudaFree(x->d_node_gpus);
     for (auto* b : x->plan_bounds) cudaFree(b);
-    cudaFree(x->skip_mask);
     for (auto& r : x->phase_recs)
         for (cudaEvent_t ev : r.e) x->ev_pool.push_back(ev);
     for (cudaEvent_t ev : x->ev_pool) cudaEventDestroy(ev);
@@ -893,7 +890,11 @@ struct PriceUnit {
     const heddle_ctx::Level* lvl;
     int shift;
     int64_t lo, nb;
-    const uint8_t* skip = nullptr;  // per candidate of c: price it SKIPPED (nullable)
+    // a plan slot (see PriceArgs; nullable, per candidate of c)
+    const uint8_t* n_tmpl = nullptr;
+    int32_t plan_slots = 0, plan_slot = 0;
+    const uint8_t* prev_status = nullptr;
+    bool bounds_scratch = false;
 };
 
 // Independent chunk pricings (no top-k, no tiling output) as one pipeline:
@@ -925,7 +926,11 @@ heddle_status price_units(heddle_ctx* x, const PriceUnit* u, int nu, void* strea
         const bool t = tiled && !u[k].lvl;
         hd::PriceArgs a{};
         fill_price_args(x, u[k].c, u[k].lvl, u[k].shift, t, a);
-        a.skip = u[k].skip ? u[k].skip + u[k].lo : nullptr;
+        a.n_tmpl = u[k].n_tmpl ? u[k].n_tmpl + u[k].lo : nullptr;
+        a.plan_slots = u[k].plan_slots;
+        a.plan_slot = u[k].plan_slot;
+        a.prev_status = u[k].prev_status ? u[k].prev_status + u[k].lo : nullptr;
+        a.bounds_scratch = u[k].bounds_scratch ? 1 : 0;
         if ((st = price_chunk(x, a, u[k].c, u[k].r, u[k].lo, u[k].nb, b, ws, nullptr, cs, t, nullptr)) != HEDDLE_OK)
             return st;
         if (pipe) CU(cudaEventRecord(x->ev_wl_free[b], ws));
@@ -1319,24 +1324,25 @@ heddle_status heddle_price_plans(heddle_ctx* x, const heddle_plans* pl, const he
     a.thr = pr->thr;
     a.err = x->d_flags + 1;
     // the slots priced as standalone candidates, slot by slot: slot t only
-    // for the plans whose templates 0 .. t-1 are each OK alone (the mask
+    // for the plans whose templates 0 .. t-1 are each OK alone (the screen
     // reads slot t - 1's statuses), the chunks of a slot pipelined over the
     // work streams.  The walk re-evaluates templates after the first from
     // their splits, so those slots need bounds
     heddle_results rs[HEDDLE_MAX_TEMPLATES];
-    CU(grow(&x->skip_mask, &x->skip_mask_cap, (size_t)pl->n));
     for (int t = 0; t < pl->slots; ++t) {
         rs[t] = pr->t[t];
         if (!rs[t].bounds && t > 0) {
             CU(grow(&x->plan_bounds[t], &x->plan_bounds_cap[t], (size_t)(HEDDLE_MAX_STAGES + 1) * pl->n));
             rs[t].bounds = x->plan_bounds[t];
         }
-        CU(hd::launch_plan_mask(pl->n_templates, pl->slots, t, t > 0 ? rs[t - 1].status : nullptr, x->skip_mask,
-                                pl->n, x->num_sms, sm));
         std::vector<PriceUnit> units;
         for (int64_t lo = 0; lo < pl->n; lo += x->chunk) {
             PriceUnit u{&pl->t[t], &rs[t], nullptr, 0, lo, std::min<int64_t>(x->chunk, pl->n - lo)};
-            u.skip = x->skip_mask;
+            u.n_tmpl = pl->n_templates;
+            u.plan_slots = pl->slots;
+            u.plan_slot = t;
+            u.prev_status = t > 0 ? rs[t - 1].status : nullptr;
+            u.bounds_scratch = !pr->t[t].bounds;
             units.push_back(u);
         }
         if ((st = price_units(x, units.data(), (int)units.size(), stream)) != HEDDLE_OK) return st;
@@ -1354,6 +1360,7 @@ heddle_status heddle_price_plans(heddle_ctx* x, const heddle_plans* pl, const he
         s.status = r.status;
         s.bounds = r.bounds;
         s.bstride = pl->n;
+        s.bounds_scratch = pr->t[t].bounds ? 0 : 1;
     }
     CU(hd::launch_plans(a, x->num_sms, sm));
     return ok(x);

@@ -350,7 +350,8 @@ __device__ __forceinline__ int64_t eq_evaluate(const PriceArgs& a, const EqTabs&
     if (pbytes >= 0) bestG *= (uint64_t)pbytes;
     if (a.bounds) {
         a.bounds[c] = 0;
-        for (int s = S + 1; s <= kMaxStages; ++s) a.bounds[(int64_t)s * a.bstride + c] = 0;
+        if (!a.bounds_scratch)
+            for (int s = S + 1; s <= kMaxStages; ++s) a.bounds[(int64_t)s * a.bstride + c] = 0;
     }
     if (pre != total) atomicOr(a.err, kErrInternal);
     int64_t gmax = 0;

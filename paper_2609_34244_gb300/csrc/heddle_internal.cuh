@@ -168,7 +168,14 @@ struct PriceArgs {
     const uint8_t* S;
     const uint16_t* M;
     const uint8_t* code;
-    const uint8_t* skip;  // nullable: nonzero prices the candidate SKIPPED (a template its plan does not reach)
+    // one template slot of a plan batch (n_tmpl nullable: none): a candidate is
+    // priced SKIPPED unless its plan reaches the slot on its templates' own
+    // prices -- it has more than plan_slot templates and, past the first
+    // slot, the previous one's status is OK (a SKIPPED one is not)
+    const uint8_t* n_tmpl;
+    int32_t plan_slots, plan_slot;
+    const uint8_t* prev_status;  // nullable: the first slot
+    int32_t bounds_scratch;      // only the planes 0 .. S of OK candidates are read: the others stay as they are
     int64_t n;
     int64_t stride;
     int32_t s_max;
@@ -237,6 +244,7 @@ struct PlanSlot {
     uint8_t* status;
     uint8_t* bounds;  // [33][bstride]
     int64_t bstride;
+    int32_t bounds_scratch;  // the caller passed none: nothing reads them afterwards
 };
 struct PlanArgs {
     Layout lay;
@@ -254,10 +262,6 @@ struct PlanArgs {
     uint32_t* err;
 };
 cudaError_t launch_plans(const PlanArgs& a, int num_sms, cudaStream_t st);
-// The SKIPPED mask of slot t of a plan batch (see plan_mask_kernel).
-cudaError_t launch_plan_mask(const uint8_t* n_tmpl, int slots, int t, const uint8_t* prev_status, uint8_t* skip,
-                             int64_t n, int num_sms, cudaStream_t st);
-
 // Ahead of the tiled search (heddle_gsearch.cu): the entries no split fits
 // are priced OOM, the others listed at a.sv_idx (count at
 // wl_count[kWlGeneral]); does nothing below a.thread_min bucketed entries.

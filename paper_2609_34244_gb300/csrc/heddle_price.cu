@@ -111,7 +111,9 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
             key = (S >= 1 && S <= s_lim && M >= 1 && whole) ? S : 0;
             // a plan's template that the plan cannot reach is priced SKIPPED
             // (bit 7 of its S byte; it sorts with the invalid ones)
-            const bool skipped = a.skip && a.skip[c0 + threadIdx.x];
+            const bool skipped =
+                a.n_tmpl && !(min((int)a.n_tmpl[c0 + threadIdx.x], a.plan_slots) > a.plan_slot &&
+                              (!a.prev_status || a.prev_status[c0 + threadIdx.x] == HEDDLE_CAND_OK));
             if (skipped) key = 0;
             sS[threadIdx.x] = (uint8_t)(key | (skipped ? 0x80 : 0));
             sM[threadIdx.x] = (uint16_t)M;
@@ -246,7 +248,7 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
             a.B[r] = -1;
             a.ndp[r] = sn[threadIdx.x];
             a.status[r] = sstatus[threadIdx.x];
-            if (a.bounds)
+            if (a.bounds && !a.bounds_scratch)
                 for (int s = 0; s <= kMaxStages; ++s) a.bounds[(int64_t)s * a.bstride + r] = 0;
         }
     }
