@@ -768,6 +768,7 @@ heddle_status price_chunk(heddle_ctx* x, hd::PriceArgs& a, const heddle_candidat
     a.thr = only ? reinterpret_cast<uint32_t*>(W.count + hd::kWlMeta) : x->d_flags + 2;
     a.wl_clear = hd::kWlMeta + (only ? 1 : 0);
     a.topk_k = state ? &state->k : nullptr;
+    a.chained = only && !x->time_phases ? 1 : 0;
     a.S = c->S + lo;
     a.M = c->M + lo;
     a.code = c->code + lo;
@@ -813,6 +814,7 @@ heddle_status price_chunk(heddle_ctx* x, hd::PriceArgs& a, const heddle_candidat
         m.wl_nM = survivors ? W.sv_nM : W.nM;
         m.wl_cap = hd::kWorklistCap;
         m.survivors = survivors ? 1 : 0;
+        m.chained = a.chained && !a.split_mode && !tiled;
         m.thr = a.thr;
         CU(hd::launch_topk_worklist(m, nb, x->num_sms, cs, nl ? nl + 2 : nullptr));
         if (x->time_phases) CU(cudaEventRecord(rec.e[4], cs));

@@ -389,6 +389,8 @@ __global__ void __launch_bounds__(kEqBlock, 1024 / kEqBlock) eq_search_kernel(Pr
         static_assert(sizeof(sh.run) % 16 == 0 && offsetof(ScreenTabs, run) % 16 == 0, "copied 16 bytes at a time");
         for (int i = threadIdx.x; i < (int)(sizeof(sh.run) / 16); i += kEqBlock) to2[i] = __ldg(from2 + i);
     }
+    allow_dependents();
+    await_previous();  // the screen's worklist
     if (threadIdx.x < 32) {
         // end_of[S] = entries of depths >= S: an inclusive scan of depths
         // 32 .. 1 in lanes 0 .. 31
@@ -564,8 +566,7 @@ cudaError_t launch(const PriceArgs& a, int num_sms, cudaStream_t st) {
     // start beside this search's last warps
     const int64_t need = (a.n + kEqBlock - 1) / kEqBlock;
     const int grid = (int)std::min<int64_t>(need, (int64_t)num_sms * std::min(per_sm, 7));
-    eq_search_kernel<kCount><<<grid, kEqBlock, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_after(a.chained, eq_search_kernel<kCount>, grid, kEqBlock, 0, st, a);
 }
 
 }  // namespace

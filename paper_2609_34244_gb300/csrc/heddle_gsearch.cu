@@ -282,6 +282,8 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
     const Layout& y = a.lay;
     const int L = y.L;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    allow_dependents();
+    await_previous();
     if (threadIdx.x < 32) {
         // end_of[S] = entries of depths >= S (see eq_search_kernel)
         int x = a.wl_count[1 + (kMaxStages - lane)];
@@ -642,8 +644,7 @@ cudaError_t launch(const PriceArgs& a, int num_sms, cudaStream_t st) {
     // the worklist length is only known on the device: one wave at most
     const int64_t need = (a.n + kGBlock - 1) / kGBlock;
     const int grid = (int)std::min<int64_t>(need, (int64_t)num_sms * per_sm);
-    gsearch_kernel<kCount, kMemOnly><<<grid, kGBlock, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_after(a.chained, gsearch_kernel<kCount, kMemOnly>, grid, kGBlock, smem, st, a);
 }
 
 }  // namespace

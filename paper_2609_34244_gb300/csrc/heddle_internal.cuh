@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "heddle.h"
 
 namespace hd {
@@ -161,6 +163,32 @@ cudaError_t launch_tables(const TableArgs& a, cudaStream_t st);
 // which a small pricing call would otherwise pay on every launch.
 cudaError_t resident_blocks(const void* func, int block, size_t smem, int* per_sm);
 
+// Programmatic dependent launch: a kernel launched by launch_after may start
+// while the previous kernel of its stream still runs, once every CTA of that
+// one has called allow_dependents (or exited); await_previous returns when
+// the previous kernel has completed and its writes are visible (at once when
+// the kernel was launched the ordinary way).  A call of one chunk chains its
+// kernels so: with a thousand candidates each runs for little longer than a
+// launch takes.
+__device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void await_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_after(bool chained, void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t st,
+                         A&&... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
 struct PriceArgs {
     Layout lay;
     const unsigned char* img;
@@ -201,6 +229,7 @@ struct PriceArgs {
                          // that depth, in any order (equal-layer search)
     int32_t wl_cap;
     int32_t wl_clear;    // ints of wl_count the screen's launch clears (kWlMeta, or one more with the threshold)
+    int32_t chained;     // the search may start while the screen still runs (see launch_after)
     int32_t uniform;     // search with the equal-layer closed form (model flags [0] and [1])
     int32_t mbs_shift;   // micro-batch size 2^shift: M >> shift micro-batches (invalid unless 2^shift | M)
     int32_t split_mode;  // 1: the paper's own split rule (distribute_kernel) instead of PartitionLayers
@@ -310,6 +339,7 @@ struct TopkArgs {
     const int64_t* wl_T;
     const uint32_t* wl_nM;
     int32_t wl_cap;
+    int32_t chained;    // launched behind its search (see launch_after)
     int32_t survivors;  // the worklist holds a threshold's survivors only
     // nullable: raised (atomicMax on the bits of a positive float) to the
     // new state's k-th key n*M / T in float times (1 - 2^-16) once the state

@@ -86,6 +86,7 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
     __shared__ int smax;
     const Layout& y = a.lay;
     const int L = y.L;
+    allow_dependents();
     {
         const uint4* from = reinterpret_cast<const uint4*>(a.img + y.offScreen);
         uint4* to = reinterpret_cast<uint4*>(&tab);

@@ -155,6 +155,7 @@ __global__ void __launch_bounds__(kSelBlock) topk_select_kernel(TopkArgs a) {
     __shared__ TopkEntry tmp[(kSelWarps / 2) * kMaxTopK];
     __shared__ int counts[kSelWarps], tmp_counts[kSelWarps / 2];
     __shared__ int n_cand, last_flag, first;
+    await_previous();
     const int k = state_k(a.state);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t n = kWorklist ? min((int64_t)*a.wl_count, (int64_t)a.wl_cap) : a.n;
@@ -375,9 +376,8 @@ cudaError_t launch_select(const TopkArgs& a, int64_t n, int num_sms, cudaStream_
     // small launch finds room sooner beside the next chunks' searches
     const int most = std::min(a.survivors ? 64 : 2 * num_sms, a.max_blocks);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((n + kPerCta - 1) / kPerCta, most));
-    topk_select_kernel<kWorklist><<<grid, kSelBlock, 0, st>>>(a);
     if (launches) *launches += 1;
-    return cudaGetLastError();
+    return launch_after(a.chained, topk_select_kernel<kWorklist>, grid, kSelBlock, 0, st, a);
 }
 
 __global__ void topk_reset_kernel(heddle_topk_state* s, int k) {

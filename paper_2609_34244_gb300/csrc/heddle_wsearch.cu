@@ -111,7 +111,10 @@ template <bool kCount>
 __global__ void __launch_bounds__(kWBlock, 3) wsearch_kernel(PriceArgs a, int thread_min) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ uint64_t bar;
-    if (!wp::load_image(smem, a.img, a.lay.searchBytes, &bar, a.err)) return;
+    allow_dependents();
+    const bool loaded = wp::load_image(smem, a.img, a.lay.searchBytes, &bar, a.err);
+    await_previous();  // (on every path: the next kernel waits for this one only)
+    if (!loaded) return;
     const Layout& y = a.lay;
     WTabs t;
     t.P = reinterpret_cast<const int64_t*>(smem + y.offP);
@@ -333,8 +336,7 @@ cudaError_t launch(const PriceArgs& a, int num_sms, cudaStream_t st, bool listed
     // at most one wave
     const int64_t need = (a.n + kWarps - 1) / kWarps;
     const int grid = (int)std::min<int64_t>(need, (int64_t)num_sms * per_sm);
-    wsearch_kernel<kCount><<<grid, kWBlock, smem, st>>>(a, listed ? a.thread_min : INT_MAX);
-    return cudaGetLastError();
+    return launch_after(a.chained, wsearch_kernel<kCount>, grid, kWBlock, smem, st, a, listed ? a.thread_min : INT_MAX);
 }
 
 }  // namespace
