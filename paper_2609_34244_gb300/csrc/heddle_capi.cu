@@ -733,6 +733,8 @@ void fill_price_args(heddle_ctx* x, const heddle_candidates* c, const heddle_ctx
     x->count_next = false;
     a.wl_cap = hd::kWorklistCap;
     a.uniform = !tiled && equal_layer_search(x, lvl ? lvl->flags : x->model_flags) ? 1 : 0;
+    const int32_t* flags = lvl ? lvl->flags : x->model_flags;
+    a.equal_layers = flags[0] && flags[1] ? 1 : 0;
     a.split_mode = x->search_mode == HEDDLE_SEARCH_DISTRIBUTE ? 1 : 0;
     a.thread_min = x->thread_min < 0 ? hd::thread_search_min(x->num_sms) : x->thread_min;
 }

@@ -18,15 +18,21 @@
 // splits the layers before the fill picks the DP degree, so the choice
 // cannot see the gradient term).  No alternative fits: OOM.
 //
-// One warp per worklist entry, one lane per stage (S <= 32): every
-// per-stage quantity lives in the lane's registers, and the split's sums,
-// ranks, scans and maxima are warp collectives.  The screen has already
-// rejected the candidates no split fits; the small tables are read through
-// the L1 cache.
+// Two kernels.  On a model whose layers all cost the same in time and memory
+// a stage's time is layers times one layer's and its memory is a run length,
+// so an alternative is a sum and a maximum over the stages: one thread per
+// entry, the warps taking 32 at a time, deepest first, like the equal-layer
+// search.  The floors come from float quotients corrected exactly; the
+// largest remainders from 32-bit keys (27 leading bits of the remainder and
+// the stage), compared with one another, and from the exact remainders where
+// two that differ share a key at the cut.  1e6 candidates of the largest
+// workload: 260 -> 62 us (one warp per entry, a lane per stage: 64-bit
+// divisions, sums and ranks by shuffles, half the lanes past the depth).
+// Other models keep that warp kernel, whose lanes read the prefix tables.
 
 #include <algorithm>
 
-#include "heddle_internal.cuh"
+#include "heddle_eq.cuh"
 
 namespace hd {
 namespace {
@@ -207,9 +213,249 @@ __global__ void __launch_bounds__(kDistBlock) distribute_kernel(PriceArgs a) {
     }
 }
 
+// ---- equal layers: one thread per entry
+
+struct SplitShared {
+    EqTabs tab;
+    uint16_t run[32 * 33 + 256];         // ScreenTabs::run
+    int64_t speed[32];                   // 2^40 / the time of all layers, per stage byte
+    uint32_t sw[kMaxStages * kEqBlock];  // stage words (heddle_eq.cuh): the cap field holds the stage's layers
+    uint32_t key[kMaxStages * kEqBlock];
+};
+
+// floor(share / V) and the remainder, the float quotient off by at most one
+// (the quotient is at most 255)
+__device__ __forceinline__ int share_floor(int64_t share, int64_t V, float rV, int64_t& rem) {
+    int q = (int)(u64_to_float((uint64_t)share) * rV);
+    rem = share - (int64_t)q * V;
+    if (rem < 0) {
+        --q;
+        rem += V;
+    } else if (rem >= V) {
+        ++q;
+        rem -= V;
+    }
+    return q;
+}
+
+// The weight of a stage under an alternative (0: speed, 2: memory run).
+__device__ __forceinline__ int64_t split_weight(const SplitShared& sh, uint32_t w, int alt) {
+    return alt == 0 ? sh.speed[w & 31] : (int64_t)run_of(w);
+}
+
+// The stages that gain a layer by exact remainders (only where keys cannot
+// tell): counts of stages with a larger remainder, or as large and earlier.
+__device__ __noinline__ void exact_gains(const SplitShared& sh, uint32_t* sw, int S, int L, int64_t V, float rV, int alt,
+                                         int missing) {
+    for (int s = 0; s < S; ++s) {
+        int64_t rs, rt;
+        share_floor((int64_t)L * split_weight(sh, sw[s * kEqBlock], alt), V, rV, rs);
+        int rank = 0;
+        for (int t = 0; t < S; ++t) {
+            share_floor((int64_t)L * split_weight(sh, sw[t * kEqBlock], alt), V, rV, rt);
+            rank += (rt > rs || (rt == rs && t < s)) ? 1 : 0;
+        }
+        if (rank < missing) sw[s * kEqBlock] += 1u << kCapShift;
+    }
+}
+
+// Layers per stage in proportion to the alternative's weights (sum V > 0),
+// into the cap fields (see share_count).
+__device__ __forceinline__ void proportional(const SplitShared& sh, uint32_t* sw, uint32_t* key, int S, int L, int64_t V,
+                                             int alt) {
+    const float rV = 1.0f / u64_to_float((uint64_t)V);
+    const int shift = max(0, 64 - __clzll(V) - 27);
+    int total = 0;
+    for (int s = 0; s < S; ++s) {
+        const uint32_t w = sw[s * kEqBlock] & kNoCap;
+        int64_t rem;
+        const int q = max(share_floor((int64_t)L * split_weight(sh, w, alt), V, rV, rem), 1);
+        sw[s * kEqBlock] = w | ((uint32_t)q << kCapShift);
+        key[s * kEqBlock] = ((uint32_t)(rem >> shift) << 5) | (uint32_t)(31 - s);
+        total += q;
+    }
+    const int missing = L - total;
+    if (missing > 0) {
+        // ranks of four stages at a time; the last key that gains, the first
+        // that does not
+        uint32_t cut = 0xffffffffu, next = 0;
+        for (int s0 = 0; s0 < S; s0 += 4) {
+            uint32_t k[4];
+            int r[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) k[i] = s0 + i < S ? key[(s0 + i) * kEqBlock] : 0xffffffffu;
+            for (int t = 0; t < S; ++t) {
+                const uint32_t kt = key[t * kEqBlock];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) r[i] += kt > k[i] ? 1 : 0;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (s0 + i >= S) continue;
+                if (r[i] < missing) {
+                    sw[(s0 + i) * kEqBlock] += 1u << kCapShift;
+                    cut = min(cut, k[i]);
+                } else {
+                    next = max(next, k[i]);
+                }
+            }
+        }
+        if (shift > 0 && missing < S && (cut >> 5) == (next >> 5)) {
+            // a tie at the cut: exact if one weight (the same remainder) has it all
+            bool same = true;
+            const uint32_t code = sw[(31 - (cut & 31)) * kEqBlock] & 31;
+            for (int s = 0; s < S; ++s)
+                same = same && ((key[s * kEqBlock] >> 5) != (cut >> 5) || (sw[s * kEqBlock] & 31) == code);
+            if (!same) {
+                for (int s = 0; s < S; ++s) {
+                    int64_t rem;
+                    const uint32_t w = sw[s * kEqBlock] & kNoCap;
+                    const int q = max(share_floor((int64_t)L * split_weight(sh, w, alt), V, rV, rem), 1);
+                    sw[s * kEqBlock] = w | ((uint32_t)q << kCapShift);
+                }
+                exact_gains(sh, sw, S, L, V, rV, alt, missing);
+            }
+        }
+    }
+    for (; total > L; --total) {
+        // the stage holding the most (the later one on ties) gives one up
+        int most = 0, at = 0;
+        for (int s = 0; s < S; ++s) {
+            const int c = cap_of(sw[s * kEqBlock]);
+            if (c >= most) {
+                most = c;
+                at = s;
+            }
+        }
+        if (most <= 1) break;  // (S <= L: never)
+        sw[at * kEqBlock] -= 1u << kCapShift;
+    }
+}
+
+__global__ void __launch_bounds__(kEqBlock, 5) split_kernel(PriceArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    SplitShared& sh = *reinterpret_cast<SplitShared*>(smem);
+    __shared__ int end_of[kMaxStages + 2];
+    const Layout& y = a.lay;
+    const int L = y.L;
+    load_eq_tables(a, sh.tab, sh.run);
+    depth_ends(a.wl_count, end_of);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int64_t all = sh.tab.q[threadIdx.x] * L;
+        sh.speed[threadIdx.x] = all > 0 ? ((int64_t)1 << 40) / all : ((int64_t)1 << 40);
+    }
+    __syncthreads();
+    const EqTabs& t = sh.tab;
+    const int64_t* PB = reinterpret_cast<const int64_t*>(a.img + y.offPB);
+    const int64_t pbytes = reinterpret_cast<const ModelInfo*>(a.img + y.offModel)->grad_uniform ? PB[1] - PB[0] : -1;
+    uint32_t* sw = sh.sw + threadIdx.x;
+    uint32_t* key = sh.key + threadIdx.x;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t entries = min((int64_t)*a.wl_count, (int64_t)a.wl_cap);
+    const int64_t count = min((int64_t)end_of[1], entries);
+    const int64_t first = (int64_t)gridDim.x * kEqBlock;
+    auto take = [&]() {
+        int b = 0;
+        if (lane == 0) b = atomicAdd(a.wl_count + kWlTakeThread, 32);
+        return first + __shfl_sync(kFull, b, 0);
+    };
+    for (int64_t base = ((int64_t)blockIdx.x * kEqWarps + warp) * 32; base < count; base = take()) {
+        const int64_t g = base + lane;
+        int64_t p = 0;
+        if (g >= count || !deepest_first(a, end_of, g, entries, p)) continue;
+        const int64_t c = a.wl_idx[p];
+        const int S = a.wl_S[p], M = a.wl_M[p];
+        const int64_t n = a.wl_n[p];
+        if (!in_range(c, a.n, a.err)) continue;
+        int64_t V0 = 0, csum = 0;
+        int V2 = 0;
+        for_stages(a, t, sh.run, p, S, M, [&](int s, int code, int pidx, uint32_t m) {
+            sw[s * kEqBlock] = (uint32_t)code | ((uint32_t)pidx << 5) | (m << 13);
+            V0 += sh.speed[code];
+            V2 += (int)m;
+            csum += t.p2p[pidx];
+        });
+        // the alternatives from the last to the first: an earlier one wins a
+        // tie, and the first, which fits most often, is left in the words
+        int best = -1;
+        int64_t bestPipe = 0, bestB = 0;
+        for (int alt = 2; alt >= 0; --alt) {
+            const int64_t V = alt == 0 ? V0 : V2;
+            if (alt != 1) {
+                if (V <= 0) continue;
+                proportional(sh, sw, key, S, L, V, alt);
+            } else {
+                // equal counts, the earlier stages one more
+                const int each = L / S, more = L - each * S;
+                for (int s = 0; s < S; ++s)
+                    sw[s * kEqBlock] = (sw[s * kEqBlock] & kNoCap) | ((uint32_t)(each + (s < more ? 1 : 0)) << kCapShift);
+            }
+            bool fits = true;
+            int64_t tmax = 0, tsum = csum;
+            for (int s = 0; s < S; ++s) {
+                const uint32_t w = sw[s * kEqBlock];
+                const int k = cap_of(w);
+                fits = fits && k <= run_of(w);
+                const int64_t ts = (int64_t)k * t.q[w & 31];
+                tsum += ts;
+                tmax = max(tmax, ts + t.p2p[p2p_of(w)]);
+            }
+            const int64_t pipe = (int64_t)(M - 1) * tmax + tsum;
+            if (fits && (best < 0 || pipe <= bestPipe)) {
+                best = alt;
+                bestPipe = pipe;
+                bestB = tmax;
+            }
+        }
+        a.ndp[c] = (uint16_t)n;  // OOM keeps the DP degree
+        a.wl_nM[p] = (uint32_t)n * (uint32_t)M;
+        if (best < 0) {
+            a.T[c] = -1;
+            a.B[c] = -1;
+            a.status[c] = HEDDLE_CAND_OOM;
+            a.wl_T[p] = -1;
+            if (a.bounds)
+                for (int s = 0; s <= kMaxStages; ++s) a.bounds[(int64_t)s * a.bstride + c] = 0;
+            continue;
+        }
+        if (best == 2) proportional(sh, sw, key, S, L, V2, 2);
+        GradMax grad;
+        int at = 0;
+        for (int s = 0; s < S; ++s) {
+            const uint32_t w = sw[s * kEqBlock];
+            const int each = L / S;
+            const int nxt = at + (best == 1 ? each + (s < L - each * S ? 1 : 0) : cap_of(w));
+            if (n > 1) grad.add(t, PB, pbytes, w & 31, at, nxt);
+            if (a.bounds) a.bounds[(int64_t)(s + 1) * a.bstride + c] = (uint8_t)nxt;
+            at = nxt;
+        }
+        if (at != L) atomicOr(a.err, kErrInternal);
+        if (a.bounds) {
+            a.bounds[c] = 0;
+            for (int s = S + 1; s <= kMaxStages; ++s) a.bounds[(int64_t)s * a.bstride + c] = 0;
+        }
+        const int64_t T = bestPipe + (n > 1 ? grad.sync_ns(n, pbytes, a.err) : 0);
+        a.T[c] = T;
+        a.B[c] = bestB;
+        a.status[c] = HEDDLE_CAND_OK;
+        a.wl_T[p] = T;
+    }
+}
+
 }  // namespace
 
 cudaError_t launch_distribute(const PriceArgs& a, int num_sms, cudaStream_t st) {
+    if (a.equal_layers) {
+        const size_t smem = sizeof(SplitShared);
+        int per_sm = 0;
+        const cudaError_t e = resident_blocks(reinterpret_cast<const void*>(&split_kernel), kEqBlock, smem, &per_sm);
+        if (e != cudaSuccess) return e;
+        if (per_sm < 1) return cudaErrorInvalidConfiguration;
+        const int grid = (int)std::min<int64_t>((a.n + kEqBlock - 1) / kEqBlock, (int64_t)num_sms * per_sm);
+        split_kernel<<<grid, kEqBlock, smem, st>>>(a);
+        return cudaGetLastError();
+    }
     // one warp per entry; the worklist length is only known on the device
     const int grid = (int)std::min<int64_t>((a.n + kDistBlock / 32 - 1) / (kDistBlock / 32), (int64_t)num_sms * 16);
     distribute_kernel<<<grid, kDistBlock, 0, st>>>(a);

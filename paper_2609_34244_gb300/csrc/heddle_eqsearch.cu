@@ -46,34 +46,14 @@
 // 19.1; 80-layer workload at four micro-batch sizes, 2.5e5: 37.7 -> 24.3.
 
 #include <algorithm>
-#include <cstddef>
 
-#include "heddle_internal.cuh"
+#include "heddle_eq.cuh"
 
 namespace hd {
 namespace {
 
-constexpr int kEqBlock = 128;
-constexpr int kEqWarps = kEqBlock / 32;
 constexpr int kMaxIters = 256;
 constexpr int kWalk = 4;  // breakpoints walked before the next probe
-
-struct EqShared {
-    EqTabs tab;
-    uint16_t run[32 * 33 + 256];  // ScreenTabs::run
-    uint32_t sw[kMaxStages * kEqBlock];  // stage words, [s][thread]
-};
-
-// Stage word: bits 0-4 cost index (the stage byte's type | degree bits),
-// bits 5-12 P2P index, bits 13-20 memory run m, bits 21-28 the cap.
-constexpr int kCapShift = 21;
-constexpr uint32_t kNoCap = 0x1fffffu;
-
-__device__ __forceinline__ int cap_of(uint32_t w) { return (int)(w >> kCapShift) & 255; }
-__device__ __forceinline__ int run_of(uint32_t w) { return (int)(w >> 13) & 255; }
-__device__ __forceinline__ int p2p_of(uint32_t w) { return (int)(w >> 5) & 255; }
-// a count below 2^23 as float (two full-rate instructions)
-__device__ __forceinline__ float count_float(uint32_t n) { return __uint_as_float(n | 0x4b000000u) - 8388608.0f; }
 
 // Continuous count at Bf (float): sum_s min(m_s, (Bf - c_s) / q_s), with
 // the slope sum 1/q_s and the number of stages below their run.
@@ -308,13 +288,7 @@ __device__ __forceinline__ int64_t eq_evaluate(const PriceArgs& a, const EqTabs&
     const int64_t c = a.wl_idx[p];
     if (!in_range(c, a.n, a.err)) return -1;
     int64_t tsum = 0;
-    // the stage with the largest G_s / (k_s bw_s): with equal gradient bytes
-    // per layer that is the largest layers / D, found in float (three
-    // roundings, 2^-22) and compared exactly (layers < 2^8 times D < 2^43)
-    // where two come within 2^-20 of each other
-    uint64_t bestG = 0, bestD = 1;
-    float bestf = -1.f;
-    constexpr float kNear = 1.0f / 1048576.0f;
+    GradMax grad;
     int pre = 0, at = 0;
     for (int s = 0; s < S; ++s) {
         const uint32_t w = sw[s * kEqBlock];
@@ -325,44 +299,16 @@ __device__ __forceinline__ int64_t eq_evaluate(const PriceArgs& a, const EqTabs&
         const int len = nxt - at;
         if (len > k) atomicOr(a.err, kErrInternal);
         tsum += (int64_t)len * t.q[w & 31] + t.p2p[p2p_of(w)];
-        if (n > 1) {
-            if (pbytes >= 0) {
-                const float f = count_float((uint32_t)len) * t.rD[w & 31];
-                if (f > bestf * (1.0f - kNear)) {
-                    const uint64_t D = t.D[w & 31];
-                    if (f > bestf * (1.0f + kNear) || (uint64_t)len * bestD > bestG * D) {
-                        bestf = f;
-                        bestG = (uint64_t)len;
-                        bestD = D;
-                    }
-                }
-            } else {
-                const uint64_t G = in_range(nxt, L + 1, a.err) ? (uint64_t)(PB[nxt] - PB[at]) : 0;
-                const uint64_t D = t.D[w & 31];
-                if (s == 0 || (u128)G * bestD > (u128)bestG * D) {
-                    bestG = G;
-                    bestD = D;
-                }
-            }
-        }
+        if (n > 1) grad.add(t, PB, pbytes, w & 31, at, nxt);
         at = nxt;
     }
-    if (pbytes >= 0) bestG *= (uint64_t)pbytes;
     if (a.bounds) {
         a.bounds[c] = 0;
         if (!a.bounds_scratch)
             for (int s = S + 1; s <= kMaxStages; ++s) a.bounds[(int64_t)s * a.bstride + c] = 0;
     }
     if (pre != total) atomicOr(a.err, kErrInternal);
-    int64_t gmax = 0;
-    if (n > 1) {
-        // ring all-reduce over n replicas: ceil(2(n-1) G 1e9 / (n k bw))
-        // (G < 2^50 and bandwidths < 2^40 keep n k bw below 2^64)
-        const u128 num = (u128)(2 * (uint64_t)(n - 1) * 1000000000ull) * bestG;
-        bool ok = true;
-        gmax = (int64_t)ceil_div_u128(num, (uint64_t)n * bestD, &ok);
-        if (!ok) atomicOr(a.err, kErrInternal);
-    }
+    const int64_t gmax = n > 1 ? grad.sync_ns(n, pbytes, a.err) : 0;
     const int64_t T = (int64_t)(M - 1) * Bstar + tsum + gmax;
     a.T[c] = T;
     a.wl_T[p] = T;
@@ -379,31 +325,10 @@ __global__ void __launch_bounds__(kEqBlock, 1024 / kEqBlock) eq_search_kernel(Pr
     __shared__ int end_of[kMaxStages + 2];  // entries of depths >= S, [S]
     const Layout& y = a.lay;
     const int L = y.L;
-    {
-        // the tables, as the image holds them
-        const uint4* from = reinterpret_cast<const uint4*>(a.img + y.offEq);
-        uint4* to = reinterpret_cast<uint4*>(&sh.tab);
-        for (int i = threadIdx.x; i < (int)(sizeof(EqTabs) / 16); i += kEqBlock) to[i] = __ldg(from + i);
-        const uint4* from2 = reinterpret_cast<const uint4*>(a.img + y.offScreen + offsetof(ScreenTabs, run));
-        uint4* to2 = reinterpret_cast<uint4*>(sh.run);
-        static_assert(sizeof(sh.run) % 16 == 0 && offsetof(ScreenTabs, run) % 16 == 0, "copied 16 bytes at a time");
-        for (int i = threadIdx.x; i < (int)(sizeof(sh.run) / 16); i += kEqBlock) to2[i] = __ldg(from2 + i);
-    }
+    load_eq_tables(a, sh.tab, sh.run);
     allow_dependents();
     await_previous();  // the screen's worklist
-    if (threadIdx.x < 32) {
-        // end_of[S] = entries of depths >= S: an inclusive scan of depths
-        // 32 .. 1 in lanes 0 .. 31
-        const int lane = threadIdx.x;
-        int x = a.wl_count[1 + (kMaxStages - lane)];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y2 = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y2;
-        }
-        end_of[kMaxStages - lane] = x;
-        if (lane == 0) end_of[kMaxStages + 1] = 0;
-    }
+    depth_ends(a.wl_count, end_of);
     __syncthreads();
     const EqTabs& t = sh.tab;
     const int64_t* PB = reinterpret_cast<const int64_t*>(a.img + y.offPB);
@@ -431,18 +356,7 @@ __global__ void __launch_bounds__(kEqBlock, 1024 / kEqBlock) eq_search_kernel(Pr
         int S = 0, M = 0;
         int64_t n = 0;
         int64_t T = -1;
-        if (have) {
-            // its depth: the largest S with end_of[S] > g (end_of falls with S)
-            int lo = 1, hi = kMaxStages;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (end_of[mid] > g) lo = mid; else hi = mid - 1;
-            }
-            const int64_t off = g - end_of[lo + 1];
-            if (!in_range(off, end_of[lo] - end_of[lo + 1], a.err)) have = false;
-            else p = a.wl_bucket[(int64_t)(lo - 1) * a.wl_cap + off];
-            if (have && !in_range(p, entries, a.err)) have = false;
-        }
+        if (have) have = deepest_first(a, end_of, g, entries, p);
         if (have) {
             S = a.wl_S[p];
             M = a.wl_M[p];
@@ -454,32 +368,13 @@ __global__ void __launch_bounds__(kEqBlock, 1024 / kEqBlock) eq_search_kernel(Pr
             // pack the stages; the unsaturated continuous balance, and the
             // least bound at which every stage holds a layer
             float inv = 0.f, cw = 0.f, flo = 0.f;
-            // the entry's row of stage bytes (zero past S), 16 at a time
-            uint32_t cw4[8];
-            {
-                const uint4* row = reinterpret_cast<const uint4*>(a.wl_code + p * kMaxStages);
-                const uint4 v0 = __ldg(row);
-                const uint4 v1 = S > 16 ? __ldg(row + 1) : make_uint4(0, 0, 0, 0);
-                cw4[0] = v0.x; cw4[1] = v0.y; cw4[2] = v0.z; cw4[3] = v0.w;
-                cw4[4] = v1.x; cw4[5] = v1.y; cw4[6] = v1.z; cw4[7] = v1.w;
-            }
-            const int f_lim = min(M, kMaxStages) * 32;
-            int f = S * 32;
-#pragma unroll
-            for (int s = 0; s < kMaxStages; ++s) {
-                if (s >= S) break;
-                const int code = (cw4[s >> 2] >> ((s & 3) * 8)) & 0x1f;
-                const int next =
-                    s + 1 < kMaxStages ? (cw4[(s + 1) >> 2] >> (((s + 1) & 3) * 8)) & 0x1f : 0;
-                const int pidx = t.pair[(s + 1 == S ? 32 : next) * 32 + code];
-                const uint32_t m = sh.run[min(f, f_lim) + code];
-                f -= 32;
+            for_stages(a, t, sh.run, p, S, M, [&](int s, int code, int pidx, uint32_t m) {
                 mysw[s * kEqBlock] = (uint32_t)code | ((uint32_t)pidx << 5) | (m << 13);
                 const float rq = t.rq[code], cf = t.cf[pidx];
                 inv += rq;
                 cw += cf * rq;
                 flo = fmaxf(flo, cf + t.qf[code]);
-            }
+            });
             // first guess: Newton on the saturating continuous count
             float Bf = fmaxf(flo, inv > 0.f ? ((float)L + 0.5f * (float)S + cw) / inv : flo);
             for (int it = 0; it < 3; ++it) {  // the exact probes finish the job

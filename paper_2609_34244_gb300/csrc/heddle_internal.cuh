@@ -232,6 +232,7 @@ struct PriceArgs {
     int32_t chained;     // the search may start while the screen still runs (see launch_after)
     int32_t uniform;     // search with the equal-layer closed form (model flags [0] and [1])
     int32_t mbs_shift;   // micro-batch size 2^shift: M >> shift micro-batches (invalid unless 2^shift | M)
+    int32_t equal_layers;  // every layer has the same time per (type, degree) and the same memory
     int32_t split_mode;  // 1: the paper's own split rule (distribute_kernel) instead of PartitionLayers
     int32_t thread_min;  // general search: the bucketed entries below which only the warp search runs
     // per worklist entry, written by the search: T (-1 unless OK) and n * M,

@@ -66,3 +66,33 @@ def test_distribute_never_beats_the_exact_bottleneck(h, W):
     assert ok.sum() > 100
     assert (exact["status"][ok] == 0).all()
     assert (dist["bottleneck"][ok] >= exact["bottleneck"][ok]).all()
+
+
+@pytest.mark.parametrize("L", [1, 2, 7, 31, 32, 33, 128, 255])
+@pytest.mark.parametrize("kind", ["near_tie", "wide", "tight"])
+def test_distribute_equal_layers(h, W, oracle_mod, L, kind):
+    """The thread-per-entry split of equal-layer models at every depth up to
+    the layer count: types of almost the same speed (remainders that differ
+    in their last bits), of very different speed (stages with no layer of
+    their own, surplus layers to take back), and memory that rejects the
+    first alternatives; the fused top-k as well."""
+    rng = np.random.default_rng(L)
+    nt = 5
+    tflops = 100.0 * (1.0 + 1e-9 * np.arange(nt)) if kind == "near_tie" else np.geomspace(1.0, 1000.0, nt)
+    mem = rng.integers(2, 9, nt) * 10**9 if kind == "tight" else np.full(nt, 10**15)
+    cluster = W.make_cluster(tflops, mem, rng.integers(50, 900, nt) * 10**9,
+                             [(g, z, int(rng.integers(1, 50)) * 10**9) for g in range(nt) for z in (2, 4, 8)] * 8)
+    model = W.make_model(np.full(L, 3.3e12), 10**8, 8 * 10**9 // max(1, L // 8), 10**8 // max(1, L // 8), 10**6, 0,
+                         10**6)
+    n = 3000
+    S = rng.integers(1, min(L, 32) + 1, n).astype(np.uint8)
+    code = W.encode(rng.integers(0, nt, (32, n)), rng.integers(0, 3, (32, n)))
+    code[np.arange(32)[:, None] >= S[None, :]] = 0
+    cands = W.make_cands(S, rng.choice([1, 3, 64], n).astype(np.uint16), code)
+    ref = oracle_mod.Oracle(cluster, model).set_split("distribute").price(cands, threads=8)
+    for fused in (False, True):
+        got = G.price_gpu(h, cluster, model, cands, k=16, search=h.SEARCH_DISTRIBUTE, fused=fused)
+        assert got["errors"] == 0
+        G.assert_same(got, ref, what="%s L %d" % (kind, L))
+        tk = oracle_mod.topk(ref, cands["M"], 16)
+        assert got["topk"]["idx"].tolist() == tk["idx"].tolist()
