@@ -260,15 +260,25 @@ struct TiledCheck {
     __device__ __forceinline__ int eval(const TLane& st, int i, int e, int64_t B, int64_t* cost) const {
         const longlong2 a = t.SA[i], b = t.SA[e];
         const int64_t bare = (b.x - a.x) + st.f * (b.y - a.y), copies = t.ES[e] - t.ES[i];
-        const TileList& list = t.lists[st.g * 4 + st.j];
         const int64_t* P = t.Pt + (size_t)(st.g * kTileSlots + tile_base(st.j)) * (t.L + 1);
-        const int cnt = list.count;
-        int64_t best = kInf;
-        for (int o = 0; o < cnt; ++o) {
-            const int cd = list.tiling[o];
+        // the first three tilings side by side (of up to ten, most stages
+        // keep no more): their loads do not wait for one another
+        const uint4 list = *reinterpret_cast<const uint4*>(t.lists + st.g * 4 + st.j);
+        const int cnt = list.x & 255;
+        int64_t v[3];
+#pragma unroll
+        for (int o = 0; o < 3; ++o) {
+            const int cd = o < cnt ? (list.x >> (8 * o + 8)) & 255 : 0;
             const int64_t* row = P + (cd & 15) * (t.L + 1);
-            const int64_t v = row[e] - row[i];
-            if (bare + (((int64_t)1 << (cd >> 4)) - 1) * copies <= st.cap) best = min(best, v);
+            v[o] = row[e] - row[i];
+            if (o >= cnt || bare + (((int64_t)1 << (cd >> 4)) - 1) * copies > st.cap) v[o] = kInf;
+        }
+        int64_t best = min(v[0], min(v[1], v[2]));
+        for (int o = 3; o < cnt; ++o) {
+            const int cd = t.lists[st.g * 4 + st.j].tiling[o];
+            const int64_t* row = P + (cd & 15) * (t.L + 1);
+            const int64_t x = row[e] - row[i];
+            if (bare + (((int64_t)1 << (cd >> 4)) - 1) * copies <= st.cap) best = min(best, x);
         }
         if (best == kInf) return 2;
         best += st.c;
@@ -360,7 +370,8 @@ __global__ void __launch_bounds__(kTBlock, 3) tiled_search_kernel(PriceArgs a, T
         if (lane == 0) e = atomicAdd(a.wl_count + kWlTakeWarp, 1);
         return first + __shfl_sync(wp::kFull, e, 0);
     };
-    for (int64_t e = (int64_t)blockIdx.x * kTWarps + warp; e < count; e = take()) {
+    // (a list shorter than the grid spreads over all SMs)
+    for (int64_t e = (int64_t)warp * gridDim.x + blockIdx.x; e < count; e = take()) {
         const int64_t p = listed ? a.sv_idx[e] : e;
         if (!in_range(p, a.wl_cap, a.err)) continue;
         const int64_t c = a.wl_idx[p];
@@ -413,8 +424,7 @@ __global__ void __launch_bounds__(kTBlock, 3) tiled_search_kernel(PriceArgs a, T
         }
         while (true) {
             int64_t hi, lo;
-            const int quick = phase != 2 ? wp::forward_probe(check, S, L, B, hi, lo, checks) : -1;
-            const bool feas = quick >= 0 ? quick == 1 : wp::probe(check, S, L, B, wa, hi, lo, checks);
+            const bool feas = wp::probe(check, S, L, B, wa, phase == 2, hi, lo, checks) != wp::kNo;
             if (phase == 0) {
                 if (!feas) {
                     oom = true;

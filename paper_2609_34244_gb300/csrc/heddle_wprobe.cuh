@@ -142,15 +142,22 @@ __device__ __forceinline__ int next_above(const uint32_t* C, int i, int L) {
     return (w << 5) + __ffs(m) - 1;
 }
 
-// Exact probe of bound B by one warp (all lanes call it; uniform result).
-// The sets land in wa; hi / lo are the snap values; checks counts the
+// Exact probe of bound B by one warp (all lanes call it; uniform result):
+// kNo, or kYes, or kSets with the sets in wa (always, of a feasible bound,
+// when `sets` asks for them).  hi / lo are the snap values; checks counts the
 // interval checks of this lane.
+//
+// While every stage of the forward pass advances (it holds its first layer),
+// U_{s+1} is attained and no start reaches further: if the last stage fits
+// [U_{S-1}, L) the chain itself is a split, and if not there is none, so the
+// backward sets are left out unless they are wanted.
+enum Answer : int { kNo = 0, kYes = 1, kSets = 2 };
 template <class J>
-__device__ bool probe(const J& check, int S, int L, int64_t B, WarpArea& wa, int64_t& hi_out, int64_t& lo_out,
-                      unsigned long long& checks) {
+__device__ int probe(const J& check, int S, int L, int64_t B, WarpArea& wa, bool sets, int64_t& hi_out,
+                     int64_t& lo_out, unsigned long long& checks) {
     const int lane = threadIdx.x & 31;
     int64_t hi = -1, lo = kInf;
-    bool ok = true;
+    bool ok = true, advances = true;
     // forward upper bounds on the boundaries
     int u = 0;
     if (lane == 0) wa.U[0] = 0;
@@ -175,13 +182,27 @@ __device__ bool probe(const J& check, int S, int L, int64_t B, WarpArea& wa, int
             }
             reach = base + 31;
         }
+        advances = advances && reach > u;
         if (reach < s + 1) ok = false;
         u = reach;
         if (lane == 0) wa.U[s + 1] = (uint8_t)reach;
     }
     __syncwarp();
+    const bool chain = !sets && advances;
+    if (ok && chain) {
+        const typename J::Stage st = check.stage(S - 1);
+        int r = 2;
+        if (lane == 0) {
+            int64_t v = 0;
+            r = check.eval(st, u, L, B, &v);
+            ++checks;
+            if (r == 0) hi = max(hi, v);
+            else if (r == 1) lo = min(lo, v);
+        }
+        ok = __shfl_sync(kFull, r, 0) == 0;
+    }
     // backward feasible-start sets: C_S = {L}, then stages S-1 .. 1
-    if (ok) {
+    if (ok && !chain) {
         if (lane < kSetWords) wa.C[S][lane] = lane == (L >> 5) ? 1u << (L & 31) : 0u;
         __syncwarp();
         int nmax = L;
@@ -228,8 +249,8 @@ __device__ bool probe(const J& check, int S, int L, int64_t B, WarpArea& wa, int
             nmax = newmax;
         }
     }
-    bool feasible = false;
-    if (ok) {
+    bool feasible = ok && chain;
+    if (ok && !chain) {
         const int succ0 = S == 1 ? L : next_above(wa.C[1], 0, L);
         const typename J::Stage st0 = check.stage(0);
         if (succ0 >= 0 && lane == 0) {
@@ -247,65 +268,7 @@ __device__ bool probe(const J& check, int S, int L, int64_t B, WarpArea& wa, int
     }
     hi_out = wmax64(hi);
     lo_out = wmin64(lo);
-    return feasible;
-}
-
-// The forward pass alone: 1 feasible, 0 infeasible, -1 it cannot tell.  While
-// every stage advances (it holds its first layer), U_{s+1} is attained and
-// no start reaches further, so if the last stage fits [U_{S-1}, L) the chain
-// itself is a split, and if not there is none.  The snap values mean what
-// they mean for probe(): every bound in [hi, B] is feasible, every bound in
-// [B, lo) is not.  A stage that does not hold the layer after U_s leaves the
-// answer to probe(), whose sets the canonical split at B* needs as well.
-template <class J>
-__device__ int forward_probe(const J& check, int S, int L, int64_t B, int64_t& hi_out, int64_t& lo_out,
-                             unsigned long long& checks) {
-    const int lane = threadIdx.x & 31;
-    int64_t hi = -1, lo = kInf;
-    int u = 0;
-    for (int s = 0; s + 1 < S; ++s) {
-        const typename J::Stage st = check.stage(s);
-        const int lim = L - (S - 1 - s);
-        int reach = u;
-        for (int base = u + 1; base <= lim; base += 32) {
-            const int j = base + lane;
-            int r = 1;
-            int64_t v = 0;
-            if (j <= lim) {
-                r = check.eval(st, u, j, B, &v);
-                ++checks;
-                if (r == 0) hi = max(hi, v);
-                else if (r == 1) lo = min(lo, v);
-            }
-            const unsigned rej = __ballot_sync(kFull, r != 0);
-            if (rej) {
-                reach = base + __ffs(rej) - 2;
-                break;
-            }
-            reach = base + 31;
-        }
-        if (reach == u) return -1;
-        u = reach;
-    }
-    bool feasible = false;
-    {
-        const typename J::Stage st = check.stage(S - 1);
-        if (lane == 0) {
-            int64_t v = 0;
-            const int r = check.eval(st, u, L, B, &v);
-            ++checks;
-            if (r == 0) {
-                hi = max(hi, v);
-                feasible = true;
-            } else if (r == 1) {
-                lo = min(lo, v);
-            }
-        }
-        feasible = __shfl_sync(kFull, feasible, 0);
-    }
-    hi_out = wmax64(hi);
-    lo_out = wmin64(lo);
-    return feasible ? 1 : 0;
+    return !feasible ? kNo : chain ? kYes : kSets;
 }
 
 // The first guess of B* (warp-uniform): the saturating continuous balance

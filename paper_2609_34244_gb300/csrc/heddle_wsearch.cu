@@ -143,7 +143,8 @@ __global__ void __launch_bounds__(kWBlock, 3) wsearch_kernel(PriceArgs a, int th
         if (lane == 0) e = atomicAdd(a.wl_count + kWlTakeWarp, 1);
         return first + __shfl_sync(kFull, e, 0);
     };
-    for (int64_t e = (int64_t)blockIdx.x * kWarps + warp; e < count; e = take()) {
+    // (a list shorter than the grid spreads over all SMs)
+    for (int64_t e = (int64_t)warp * gridDim.x + blockIdx.x; e < count; e = take()) {
         const int64_t p = listed ? a.sv_idx[e] : e;
         if (!in_range(p, a.wl_cap, a.err)) continue;
         const int64_t c = a.wl_idx[p];
@@ -202,9 +203,8 @@ __global__ void __launch_bounds__(kWBlock, 3) wsearch_kernel(PriceArgs a, int th
         while (true) {
             int64_t shi, slo;
             if (kCount && lane == 0) ++probes;
-            const int quick = phase != 2 ? wp::forward_probe(check, S, L, B, shi, slo, checks) : -1;
-            const bool fast = quick >= 0;
-            const bool feas = fast ? quick == 1 : wp::probe(check, S, L, B, wa, shi, slo, checks);
+            const int got = wp::probe(check, S, L, B, wa, phase == 2, shi, slo, checks);
+            const bool feas = got != wp::kNo;
             if (phase == 0) {
                 if (!feas) {
                     oom = true;
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kWBlock, 3) wsearch_kernel(PriceArgs a, int th
                     lo = hi;
                 }
                 // closed by a feasible full probe: its sets are those of B* = hi
-                if (lo >= hi && feas && !fast && it <= kMaxIters) break;
+                if (lo >= hi && got == wp::kSets && it <= kMaxIters) break;
             } else {
                 if (!feas && lane == 0) atomicOr(a.err, kErrInternal);
                 break;
