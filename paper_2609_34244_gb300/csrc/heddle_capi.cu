@@ -771,6 +771,7 @@ heddle_status price_chunk(heddle_ctx* x, hd::PriceArgs& a, const heddle_candidat
     a.wl_clear = hd::kWlMeta + (only ? 1 : 0);
     a.topk_k = state ? &state->k : nullptr;
     a.chained = only && !x->time_phases ? 1 : 0;
+    a.beside = ws != cs ? 1 : 0;
     a.S = c->S + lo;
     a.M = c->M + lo;
     a.code = c->code + lo;

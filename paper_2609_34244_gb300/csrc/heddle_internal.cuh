@@ -229,6 +229,7 @@ struct PriceArgs {
                          // that depth, in any order (equal-layer search)
     int32_t wl_cap;
     int32_t wl_clear;    // ints of wl_count the screen's launch clears (kWlMeta, or one more with the threshold)
+    int32_t beside;      // other chunks are searched meanwhile
     int32_t chained;     // the search may start while the screen still runs (see launch_after)
     int32_t uniform;     // search with the equal-layer closed form (model flags [0] and [1])
     int32_t mbs_shift;   // micro-batch size 2^shift: M >> shift micro-batches (invalid unless 2^shift | M)
