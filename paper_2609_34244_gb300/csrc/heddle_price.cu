@@ -59,12 +59,25 @@ __device__ __forceinline__ float min_ratio(const uint32_t* dem, const float4* ca
     return r;
 }
 
+__device__ __forceinline__ void copy_async16(void* to, const void* from) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from)
+                 : "memory");
+}
+
+constexpr int kRow = kScreenBlock + 16;  // bytes of a tile row: 256 candidates and a block's offset
+
 // Steps 1-2 and the memory screen for every candidate of the batch.  Each
-// CTA takes 256 consecutive candidates at a time: their S and M, and the
-// code planes up to the largest S among them, are copied to shared memory
-// (16-byte vector copies when the planes are aligned), the candidates are
+// CTA takes 256 consecutive candidates at a time: their code planes are
+// copied to shared memory while their S and M arrive, the candidates are
 // counting-sorted by S, and thread i screens the i-th of that order, so the
 // lanes of a warp run stage loops of nearly equal length.
+//
+// The planes are copied in aligned blocks of 16 bytes.  A plane stride that
+// is no multiple of 16 (any batch of odd size) puts plane s of the slice at
+// its own offset, (code + s stride + c0) mod 16, in a row of 272 bytes; only a
+// block that reaches past the arrays is read byte by byte.  (999,983
+// candidates, byte copies after the sort: 55.9 us on the 80-layer workload,
+// 53.6 on the largest, 33.5 on the expert one; these: 52.7, 50.0 and 30.3.)
 //
 // Instructions bound it (and the search that overlaps it), so the tables are
 // kept in the form in which a stage adds them up: one word that adds the
@@ -76,14 +89,13 @@ __device__ __forceinline__ float min_ratio(const uint32_t* dem, const float4* ca
 __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
     __shared__ ScreenTabs tab;
     __shared__ uint32_t dem[8 * kScreenBlock];  // per-thread demand word (see stage_desc), per type
-    __shared__ __align__(16) uint8_t tile[kMaxStages * kScreenBlock];  // [stage][candidate of the slice]
+    __shared__ __align__(16) uint8_t tile[kMaxStages * kRow];  // [stage][candidate of the slice, past its offset]
     __shared__ uint8_t sS[kScreenBlock];
     __shared__ uint16_t sM[kScreenBlock];
     __shared__ uint8_t order[kScreenBlock];
     __shared__ uint16_t sn[kScreenBlock];  // OOM: the DP degree
     __shared__ uint8_t sstatus[kScreenBlock];
     __shared__ int bins[kMaxStages + 3];
-    __shared__ int smax;
     const Layout& y = a.lay;
     const int L = y.L;
     allow_dependents();
@@ -94,11 +106,25 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
     }
     const bool memuni = reinterpret_cast<const ModelInfo*>(a.img + y.offModel)->mem_uniform != 0;
     const int s_lim = min(min(kMaxStages, a.s_max), L);
-    const bool vec16 = ((reinterpret_cast<uintptr_t>(a.code) | (uintptr_t)a.stride) & 15) == 0;
+    const uint8_t* code_end = a.code + (int64_t)(a.s_max - 1) * a.stride + a.n;
+    const int skew = (int)(a.stride & 15);  // each plane's offset against the one before
     uint32_t* mydem = dem + threadIdx.x;
     const int lane = threadIdx.x & 31;
     for (int64_t c0 = (int64_t)blockIdx.x * kScreenBlock; c0 < a.n; c0 += (int64_t)gridDim.x * kScreenBlock) {
         const int nloc = (int)min((int64_t)kScreenBlock, a.n - c0);
+        // ---- code planes of the slice into the tile
+        const int off0 = (int)(reinterpret_cast<uintptr_t>(a.code + c0) & 15);
+        for (int i = threadIdx.x; i < s_lim * (kRow / 16); i += kScreenBlock) {
+            const int s = i / (kRow / 16), o = (i % (kRow / 16)) * 16;
+            const uint8_t* from = a.code + (int64_t)s * a.stride + c0 + o - ((off0 + s * skew) & 15);
+            uint8_t* to = tile + s * kRow + o;
+            if (from >= a.code && from + 16 <= code_end) {
+                copy_async16(to, from);
+            } else {
+                for (int b = 0; b < 16; ++b)
+                    if (from + b >= a.code && from + b < code_end) to[b] = __ldg(from + b);
+            }
+        }
         // ---- S and M of the slice; S = 0 marks a depth or M outside range,
         //      bin kMaxStages + 1 the padding past the batch
         int key = kMaxStages + 1;
@@ -120,25 +146,9 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
             sM[threadIdx.x] = (uint16_t)M;
         }
         if (threadIdx.x < kMaxStages + 3) bins[threadIdx.x] = 0;
-        if (threadIdx.x == 0) smax = 0;
         __syncthreads();
         atomicAdd(&bins[key], 1);
-        if (key <= kMaxStages && key > 0) atomicMax(&smax, key);
         __syncthreads();
-        // ---- code planes 0 .. smax-1 of the slice into the tile
-        const int np = smax;
-        if (vec16 && nloc == kScreenBlock) {
-            for (int i = threadIdx.x; i < np * (kScreenBlock / 16); i += kScreenBlock) {
-                const int s = i / (kScreenBlock / 16), o = (i % (kScreenBlock / 16)) * 16;
-                *reinterpret_cast<uint4*>(tile + s * kScreenBlock + o) =
-                    __ldg(reinterpret_cast<const uint4*>(a.code + (int64_t)s * a.stride + c0 + o));
-            }
-        } else {
-            for (int i = threadIdx.x; i < np * kScreenBlock; i += kScreenBlock) {
-                const int s = i / kScreenBlock, o = i % kScreenBlock;
-                if (o < nloc) tile[i] = __ldg(a.code + (int64_t)s * a.stride + c0 + o);
-            }
-        }
         if (threadIdx.x < 32) {
             // exclusive scan of bins 0..33 by one warp (lane l: bin l, lane
             // 31 also bins 32 and 33)
@@ -160,6 +170,7 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
         }
         __syncthreads();
         order[atomicAdd(&bins[key], 1)] = (uint8_t)threadIdx.x;
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
         const int ci = order[threadIdx.x];
         const bool live = threadIdx.x < nloc;  // padding sorts last
@@ -176,11 +187,13 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
                 uint32_t bad = 0;
                 int run_sum = 0;
                 const uint8_t* col = tile + ci;
+                int off = off0;
                 const int f_lim = min(M, kMaxStages) * 32;
                 int f = S * 32;
 #pragma unroll 4
                 for (int s = 0; s < S; ++s) {
-                    const int b = col[s * kScreenBlock];
+                    const int b = col[s * kRow + (off & 15)];
+                    off += skew;
                     const uint32_t d = tab.desc[b];
                     bad |= d;
                     mydem[(b & 7) * kScreenBlock] += d;
@@ -231,13 +244,14 @@ __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
             }
             // each taken candidate's row of 32 stage bytes, written by the
             // whole warp (lane = stage; zero past its depth)
+            const uint8_t* row = tile + lane * kRow + ((off0 + lane * skew) & 15);
             const int where = ci | (S << 8);
             int pc = base;
             for (unsigned m = mask; m; m &= m - 1, ++pc) {
                 const int from = __shfl_sync(0xffffffffu, where, __ffs(m) - 1);
                 if (pc < a.wl_cap)
                     a.wl_code[(int64_t)pc * kMaxStages + lane] =
-                        lane < (from >> 8) ? tile[lane * kScreenBlock + (from & 0xff)] : 0;
+                        lane < (from >> 8) ? row[from & 0xff] : 0;
             }
         }
         __syncthreads();  // the tile, S, M and order are reused by the next slice

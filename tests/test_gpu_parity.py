@@ -103,6 +103,31 @@ def test_thread_search_stepping_back(h, W, oracle_mod, L, kind):
         G.assert_same(got, ref, what="%s L %d thread_min %d" % (kind, L, thread_min))
 
 
+@pytest.mark.parametrize("lo", [0, 1, 7, 15, 16, 17])
+@pytest.mark.parametrize("m", [1, 15, 16, 255, 256, 257, 771])
+def test_screen_plane_offsets(h, W, oracle_mod, lo, m):
+    """Candidates [lo, lo + m) of planes that end with them: the first and
+    last 16-byte blocks of a slice reach past the arrays, and each plane of
+    an odd stride begins at its own offset."""
+    w = W.make_workload("stress128", seed=2, n=lo + m)
+    ref = oracle_mod.Oracle(w.cluster, w.model).price(w.cands, threads=8)
+    ctx = h.heddle_create(0)
+    try:
+        h.heddle_load_cluster(ctx, w.cluster)
+        h.heddle_load_model(ctx, w.model)
+        dc = h.cands_to_device(w.cands)
+        res = h.alloc_results(m, bounds=True)
+        h.heddle_price_candidates(ctx, h.make_candidates(dc, lo, lo + m), res)
+        assert h.heddle_device_errors(ctx) == 0
+        got = h.results_to_numpy(res)
+    finally:
+        h.heddle_destroy(ctx)
+    for key in ("status", "n_dp", "T", "bottleneck"):
+        assert (got[key] == ref[key][lo:]).all(), key
+    ok = ref["status"][lo:] == 0
+    assert (got["bounds"][:, ok] == ref["bounds"][:, lo:][:, ok]).all()
+
+
 @pytest.mark.parametrize("name", ["tiny", "dense32", "dense80", "moe48", "stress128"])
 def test_tables_match_oracle(h, W, oracle_mod, name):
     w = W.make_workload(name, n=10)
