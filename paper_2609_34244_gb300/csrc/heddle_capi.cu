@@ -1216,7 +1216,6 @@ heddle_status heddle_price_mbs(heddle_ctx* x, const heddle_candidates* c, const 
     if (!r->T || !r->bottleneck || !r->n_dp || !r->status) return fail(x, HEDDLE_E_ARG, "null result array");
     DeviceGuard dg(x->device);
     cudaStream_t sm = (cudaStream_t)stream;
-    if (mbs) CU(cudaMemsetAsync(mbs, 0, (size_t)c->n, sm));
     const int nl = x->mbs_levels;
     const size_t cap = (size_t)std::min<int64_t>(c->n, x->chunk);
     for (int i = 1; i < nl; ++i) {
@@ -1251,14 +1250,13 @@ heddle_status heddle_price_mbs(heddle_ctx* x, const heddle_candidates* c, const 
             }
         }
         if ((st = price_units(x, units, nl, stream)) != HEDDLE_OK) return st;
-        for (int i = 1; i < nl; ++i) {
+        if (nl > 1) {
             hd::MbsMergeArgs m{};
             m.n = nb;
-            m.T_l = x->lv_T[i];
-            m.B_l = x->lv_B[i];
-            m.n_l = x->lv_n[i];
-            m.status_l = x->lv_status[i];
-            m.bounds_l = r->bounds ? x->lv_bounds[i] : nullptr;
+            m.levels = nl;
+            for (int i = 1; i < nl; ++i)
+                m.level[i] = hd::MbsLevel{x->lv_T[i], x->lv_B[i], x->lv_n[i], x->lv_status[i],
+                                          r->bounds ? x->lv_bounds[i] : nullptr};
             m.bstride_l = nb;
             m.T = r->T + lo;
             m.B = r->bottleneck + lo;
@@ -1267,8 +1265,9 @@ heddle_status heddle_price_mbs(heddle_ctx* x, const heddle_candidates* c, const 
             m.bounds = r->bounds ? r->bounds + lo : nullptr;
             m.bstride = c->n;
             m.mbs = mbs ? mbs + lo : nullptr;
-            m.level = i;
             CU(hd::launch_mbs_merge(m, x->num_sms, sm));
+        } else if (mbs) {
+            CU(cudaMemsetAsync(mbs + lo, 0, (size_t)nb, sm));
         }
     }
     return ok(x);

@@ -359,15 +359,20 @@ cudaError_t launch_topk_worklist(const TopkArgs& a, int64_t n, int num_sms, cuda
                                  int64_t* launches = nullptr);
 cudaError_t launch_topk_reset(heddle_topk_state* state, int32_t k, cudaStream_t st);
 
-// Micro-batch-size fill: fold the results of one size (level) into the
-// running best (smaller T wins, ties keep the earlier, smaller size).
+// Micro-batch-size fill: fold the results of the larger sizes (levels 1 ..
+// levels - 1) into the base size's (smaller T wins, ties keep the smaller
+// size).
+struct MbsLevel {
+    const int64_t* T;
+    const int64_t* B;
+    const uint16_t* ndp;
+    const uint8_t* status;
+    const uint8_t* bounds;  // nullable, plane stride MbsMergeArgs::bstride_l
+};
 struct MbsMergeArgs {
     int64_t n;
-    const int64_t* T_l;
-    const int64_t* B_l;
-    const uint16_t* n_l;
-    const uint8_t* status_l;
-    const uint8_t* bounds_l;  // nullable, plane stride bstride_l
+    int32_t levels;
+    MbsLevel level[HEDDLE_MAX_MBS_LEVELS];  // [0] unused
     int64_t bstride_l;
     int64_t* T;
     int64_t* B;
@@ -375,8 +380,7 @@ struct MbsMergeArgs {
     uint8_t* status;
     uint8_t* bounds;  // nullable, plane stride bstride
     int64_t bstride;
-    uint8_t* mbs;     // nullable
-    int32_t level;
+    uint8_t* mbs;     // nullable: the chosen level, 0 where none is OK
 };
 cudaError_t launch_mbs_merge(const MbsMergeArgs& a, int num_sms, cudaStream_t st);
 
