@@ -482,13 +482,14 @@ heddle_status heddle_get_search(heddle_ctx* ctx, int32_t* in_use);
 
 /* Routing of the general search (models whose layers differ, §3.1
  * PartitionLayers) between its two kernels.  The thread-per-entry search
- * takes the worklist entries whose stages could each hold any single layer
- * when there are at least min_entries of them, and the warp-per-entry
- * search prices the rest; with fewer, the warp search prices every entry
- * (a thread search with too few entries runs as long as its longest serial
- * chain).  min_entries < 0 restores the default, 32 x the device's SM
- * count; 0 always runs the thread search.  Both routes return identical
- * results.  Errors: E_ARG (ctx NULL). */
+ * takes the worklist entries when there are at least min_entries of them, and
+ * the warp-per-entry search prices those it cannot decide; with fewer, the
+ * warp search prices every entry (a thread search with too few entries runs
+ * as long as its longest serial chain).  min_entries < 0 restores the
+ * default, 32 x the device's SM count; 0 always runs the thread search, and
+ * the thread-per-entry kernels of the split rule and of the tiled search's
+ * memory probe, which otherwise run from a batch size on.  All routes return
+ * identical results.  Errors: E_ARG (ctx NULL). */
 heddle_status heddle_set_thread_search_min(heddle_ctx* ctx, int32_t min_entries);
 
 /* Work counters of the next heddle_price_candidates call on ctx, for the

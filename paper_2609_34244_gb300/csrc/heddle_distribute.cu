@@ -215,6 +215,8 @@ __global__ void __launch_bounds__(kDistBlock) distribute_kernel(PriceArgs a) {
 
 // ---- equal layers: one thread per entry
 
+constexpr int64_t kThreadSplitMin = 1 << 16;
+
 struct SplitShared {
     EqTabs tab;
     uint16_t run[32 * 33 + 256];         // ScreenTabs::run
@@ -446,7 +448,12 @@ __global__ void __launch_bounds__(kEqBlock, 5) split_kernel(PriceArgs a) {
 }  // namespace
 
 cudaError_t launch_distribute(const PriceArgs& a, int num_sms, cudaStream_t st) {
-    if (a.equal_layers) {
+    // (a thread's entry takes 30 us of latency, a warp's 15; past some ten
+    // thousand entries the thread kernel's five times fewer instructions
+    // decide: 443 candidates of 22 stages take 55 us a pass by threads and 39
+    // by warps, 35,373 of 32 stages 78 and 67, 141,586 of 27 stages 79 and 150;
+    // a thread_min of zero asks for threads at any size)
+    if (a.equal_layers && (a.n >= kThreadSplitMin || a.thread_min == 0)) {
         const size_t smem = sizeof(SplitShared);
         int per_sm = 0;
         const cudaError_t e = resident_blocks(reinterpret_cast<const void*>(&split_kernel), kEqBlock, smem, &per_sm);

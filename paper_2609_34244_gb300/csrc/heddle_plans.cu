@@ -23,11 +23,17 @@
 // over placed templates of n M 1e9 / T, each term rounded in IEEE double, in
 // template order.
 //
-// One warp walks a plan: a lane per stage for the demand and Evaluate, a lane
-// per (type, size class) for n, a lane per type for the placement.  Most
-// plans end at their first template, so walks are few and their latency is
-// the kernel's time: one thread a walk took 173 us for 200,003 plans of up to
+// Where few plans of a CTA walk, one warp walks a plan: a lane per stage for
+// the demand and Evaluate, a lane per (type, size class) for n, a lane per
+// type for the placement.  Deep plans mostly end at their first template, so
+// their walks are few and their latency is the kernel's time: one thread a walk took 173 us for 200,003 plans of up to
 // four templates on the 1,024-GPU cluster, this takes 66 us (a cold launch).
+// A CTA looks at no more plans at a time than spread the batch over all SMs
+// (1,308 plans of up to twelve stages: 229 -> 128 us a call, 212 by threads).
+// Where most plans of a large batch walk -- shallow templates -- a thread each
+// does several times the walks per instruction: from alone_min plans in a
+// CTA's queue on they are walked so, 128 at a time (52,002 plans of up to five
+// stages: 205 us a call by warps alone, 140 with both).
 
 #include <algorithm>
 
@@ -40,7 +46,9 @@ constexpr int kPlanBlock = 128;
 constexpr int kPlanWarps = kPlanBlock / 32;
 constexpr unsigned kFull = 0xffffffffu;
 
-__global__ void __launch_bounds__(kPlanBlock) plan_kernel(PlanArgs a) {
+inline size_t plan_smem(int NT, int vmax) { return (size_t)kPlanBlock * (2 * (size_t)NT * (vmax + 1) + 8 * kMaxTypes); }
+
+__global__ void __launch_bounds__(kPlanBlock, 8) plan_kernel(PlanArgs a) {
     const Layout& y = a.lay;
     const int L = y.L, NT = y.NT, V = a.vmax;
     const int64_t* P = reinterpret_cast<const int64_t*>(a.img + y.offP);
@@ -76,6 +84,170 @@ __global__ void __launch_bounds__(kPlanBlock) plan_kernel(PlanArgs a) {
     __shared__ int queued;
     if (threadIdx.x == 0) queued = 0;
     __syncthreads();
+    // ---- one thread a plan: per-thread arrays in shared memory, interleaved
+    // by thread (element e of thread t at [e * kPlanBlock + t]): the node
+    // histogram H(g, v) and the demand word my_dem[g] (GPUs of groups per size
+    // class e in 16-bit field e)
+    extern __shared__ __align__(16) unsigned char psm[];
+    uint64_t* my_dem = reinterpret_cast<uint64_t*>(psm) + threadIdx.x;  // [g * kPlanBlock]
+    uint16_t* my_hist = reinterpret_cast<uint16_t*>(psm + (size_t)8 * kMaxTypes * kPlanBlock) + threadIdx.x;
+    auto H = [&](int g, int v) -> uint16_t& { return my_hist[(size_t)(g * (V + 1) + v) * kPlanBlock]; };
+    auto walk_alone = [&](int64_t c) {
+        for (int g = 0; g < NT; ++g)
+            for (int v = 0; v <= V; ++v) H(g, v) = init[g][v];
+        const int nt = min((int)a.n_tmpl[c], a.slots);
+        bool ended = false;
+        int placed = 0;
+        double thr = 0.0;
+        // (the slots past the plan's templates were priced SKIPPED)
+        for (int t = 0; t < nt; ++t) {
+            const PlanSlot& sl = a.slot[t];
+            uint8_t st = HEDDLE_CAND_SKIPPED;
+            int64_t T = -1, B = -1;
+            int64_t n = 0;
+            const int S = sl.S[c];
+            const int M = sl.M[c];
+            if (!ended) {
+                const uint8_t st0 = sl.status[c];
+                if (st0 == HEDDLE_CAND_INVALID) {
+                    st = HEDDLE_CAND_INVALID;
+                } else {
+                    // demand per (type, size class) in GPUs of groups of that class
+                    for (int g = 0; g < NT; ++g) my_dem[g * kPlanBlock] = 0;
+                    uint32_t present = 0;
+                    for (int s = 0; s < S; ++s) {
+                        const int b = sl.code[(int64_t)s * sl.stride + c];
+                        const int g = b & 7, j = (b >> 3) & 3;
+                        const int unit = (1 << j) <= maxn[g] ? (1 << j) : pow2[g];
+                        my_dem[g * kPlanBlock] += (uint64_t)(1u << j) << (16 * (31 - __clz(unit)));
+                        present |= 1u << g;
+                    }
+                    // n = min over (type, class e) of floor(cap / demand),
+                    // cap = sum over nodes of floor(free / 2^e) 2^e
+                    int64_t best = -1;
+                    for (uint32_t pm = present; pm; pm &= pm - 1) {
+                        const int g = __ffs(pm) - 1;
+                        int64_t cap[4] = {0, 0, 0, 0};
+                        for (int v = 1; v <= V; ++v) {
+                            const int64_t h = H(g, v);
+                            if (!h) continue;
+                            cap[0] += h * v;
+                            cap[1] += h * ((v >> 1) << 1);
+                            cap[2] += h * ((v >> 2) << 2);
+                            cap[3] += h * ((v >> 3) << 3);
+                        }
+                        const uint64_t dw = my_dem[g * kPlanBlock];
+                        uint32_t d = 0;
+#pragma unroll
+                        for (int e = 3; e >= 0; --e) {
+                            const uint32_t f = (uint32_t)(dw >> (16 * e)) & 0xffffu;
+                            d += f;
+                            if (f == 0) continue;  // dominated by the class above
+                            const int64_t q = cap[e] / d;
+                            if (best < 0 || q < best) best = q;
+                        }
+                    }
+                    n = best < 0 ? 0 : best;
+                    if (n == 0) {
+                        st = HEDDLE_CAND_NO_FIT;
+                    } else if (st0 == HEDDLE_CAND_OOM) {
+                        st = HEDDLE_CAND_OOM;
+                    } else if (t == 0) {
+                        // the whole cluster is free: n, T and B are the standalone ones
+                        T = sl.T[c];
+                        B = sl.B[c];
+                        st = HEDDLE_CAND_OK;
+                        if (n != (int64_t)sl.ndp[c]) atomicOr(a.err, kErrInternal);
+                    } else {
+                        // Evaluate with this n: T = (M-1) max t_s + sum t_s + max g_s
+                        int64_t tmax = 0, tsum = 0;
+                        uint64_t bestG = 0, bestD = 1;
+                        int sg = -1;
+                        int hi = sl.bounds[c];
+                        for (int s = 0; s < S; ++s) {
+                            const int b = sl.code[(int64_t)s * sl.stride + c];
+                            const int g = b & 7, j = (b >> 3) & 3;
+                            const int lo = hi;
+                            hi = sl.bounds[(int64_t)(s + 1) * sl.bstride + c];
+                            int64_t cs = 0;
+                            if (s + 1 < S) {
+                                const int bn = sl.code[(int64_t)(s + 1) * sl.stride + c];
+                                const int h = bn & 7, jn = (bn >> 3) & 3;
+                                const int same = (g == h) && ((1 << j) + (1 << jn) <= maxn[g]);
+                                cs = p2p[(g * 8 + h) * 2 + same];
+                            }
+                            const int64_t* row = P + (g * 4 + j) * (L + 1);
+                            const int64_t ts = row[hi] - row[lo] + cs;
+                            tmax = max(tmax, ts);
+                            tsum += ts;
+                            const uint64_t G = (uint64_t)(PB[hi] - PB[lo]);
+                            const uint64_t D = (uint64_t)inter[g] << j;
+                            if (sg < 0 || (u128)G * bestD > (u128)bestG * D) {
+                                sg = s;
+                                bestG = G;
+                                bestD = D;
+                            }
+                        }
+                        int64_t gmax = 0;
+                        if (n > 1) {
+                            const u128 num = (u128)(2 * (uint64_t)(n - 1) * 1000000000ull) * bestG;
+                            bool ok = true;
+                            gmax = (int64_t)ceil_div_u128(num, (uint64_t)n * bestD, &ok);
+                            if (!ok) atomicOr(a.err, kErrInternal);
+                        }
+                        T = (int64_t)(M - 1) * tmax + tsum + gmax;
+                        B = tmax;
+                        st = HEDDLE_CAND_OK;
+                    }
+                    if (st == HEDDLE_CAND_OK) {
+                        thr = __dadd_rn(thr, __ddiv_rn(__dmul_rn((double)(n * (int64_t)M), 1e9), (double)T));
+                        placed = t + 1;
+                        // place n copies of the groups, largest first
+                        for (int e = 3; e >= 0; --e) {
+                            const int w = 1 << e;
+                            for (uint32_t pm = present; pm; pm &= pm - 1) {
+                                const int g = __ffs(pm) - 1;
+                                int64_t left = (int64_t)(((my_dem[g * kPlanBlock] >> (16 * e)) & 0xffffu) >> e) * n;
+                                while (left > 0) {
+                                    if (w <= V && H(g, w) > 0) {
+                                        // nodes with exactly w free: m of them filled
+                                        const int64_t m = min(left, (int64_t)H(g, w));
+                                        H(g, w) -= (uint16_t)m;
+                                        H(g, 0) += (uint16_t)m;
+                                        left -= m;
+                                        continue;
+                                    }
+                                    int v = w + 1;
+                                    while (v <= V && H(g, v) == 0) ++v;
+                                    if (v > V) {
+                                        atomicOr(a.err, kErrInternal);  // n came from these nodes
+                                        break;
+                                    }
+                                    H(g, v) -= 1;
+                                    H(g, v - w) += 1;
+                                    left -= 1;
+                                }
+                            }
+                        }
+                    }
+                }
+                if (st != HEDDLE_CAND_OK) ended = true;
+            }
+            if (t > 0) {  // the first template keeps its standalone results
+                sl.T[c] = T;
+                sl.B[c] = B;
+                sl.ndp[c] = (uint16_t)(st == HEDDLE_CAND_OK || st == HEDDLE_CAND_OOM ? n : 0);
+                sl.status[c] = st;
+                // an OK template keeps its standalone split; any other
+                // status clears the planes
+                if (st != HEDDLE_CAND_OK && !sl.bounds_scratch)
+                    for (int s = 0; s <= kMaxStages; ++s) sl.bounds[(int64_t)s * sl.bstride + c] = 0;
+            }
+        }
+        a.placed[c] = (uint8_t)placed;
+        a.thr[c] = thr;
+    };
+    // ---- one warp a plan
     auto walk = [&](int64_t c) {
         for (int i = lane; i < kMaxTypes * (V + 1); i += 32) hist[i / (V + 1)][i % (V + 1)] = init[i / (V + 1)][i % (V + 1)];
         __syncwarp();
@@ -224,14 +396,14 @@ __global__ void __launch_bounds__(kPlanBlock) plan_kernel(PlanArgs a) {
         }
         __syncwarp();  // the warp's histogram and demand are reused
     };
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    int64_t c0 = (int64_t)blockIdx.x * blockDim.x;
+    const int64_t stride = (int64_t)gridDim.x * a.per_pass;
+    int64_t c0 = (int64_t)blockIdx.x * a.per_pass;
     while (true) {
         const bool more = c0 < a.n;  // uniform over the CTA
         if (more) {
             const int64_t c = c0 + threadIdx.x;
             bool walks = false;
-            if (c < a.n) {
+            if ((int)threadIdx.x < a.per_pass && c < a.n) {
                 // a plan walks from its second template on; the others keep
                 // their slots as priced (templates past the first OK-alone
                 // prefix were priced SKIPPED) and take the first template's
@@ -261,12 +433,18 @@ __global__ void __launch_bounds__(kPlanBlock) plan_kernel(PlanArgs a) {
         __syncthreads();
         const int have = queued;
         __syncthreads();
-        if (have >= kPlanBlock || !more) {  // a warp each
-            for (int i = warp; i < have; i += kPlanWarps) walk(queue[i]);
-            if (threadIdx.x == 0) queued = 0;
+        if (have >= kPlanBlock || !more) {
+            if (have >= a.alone_min) {  // 128 at a time, a thread each, while that many are left
+                const int n1 = min(have, kPlanBlock);
+                if (threadIdx.x < n1) walk_alone(queue[have - n1 + threadIdx.x]);
+                if (threadIdx.x == 0) queued = have - n1;
+            } else {  // a warp each
+                for (int i = warp; i < have; i += kPlanWarps) walk(queue[i]);
+                if (threadIdx.x == 0) queued = 0;
+            }
         }
         __syncthreads();
-        if (!more) break;
+        if (!more && queued == 0) break;
         if (more) c0 += stride;
     }
 }
@@ -276,12 +454,16 @@ __global__ void __launch_bounds__(kPlanBlock) plan_kernel(PlanArgs a) {
 cudaError_t launch_plans(const PlanArgs& a, int num_sms, cudaStream_t st) {
     if (a.n <= 0) return cudaSuccess;
     if (a.vmax < 1 || a.vmax > kPlanMaxNode) return cudaErrorInvalidValue;
+    const size_t smem = plan_smem(a.lay.NT, a.vmax);
     int per_sm = 0;
-    const cudaError_t e = resident_blocks(reinterpret_cast<const void*>(&plan_kernel), kPlanBlock, 0, &per_sm);
+    const cudaError_t e = resident_blocks(reinterpret_cast<const void*>(&plan_kernel), kPlanBlock, smem, &per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    const int grid = (int)std::min<int64_t>((a.n + kPlanBlock - 1) / kPlanBlock, (int64_t)num_sms * per_sm);
-    plan_kernel<<<grid, kPlanBlock, 0, st>>>(a);
+    const int64_t most = (int64_t)num_sms * per_sm;
+    PlanArgs b = a;
+    b.per_pass = (int32_t)std::min<int64_t>(std::max<int64_t>((a.n + most - 1) / most, kPlanWarps), kPlanBlock);
+    const int grid = (int)std::min<int64_t>((a.n + b.per_pass - 1) / b.per_pass, most);
+    plan_kernel<<<grid, kPlanBlock, smem, st>>>(b);
     return cudaGetLastError();
 }
 

@@ -145,7 +145,7 @@ def take(cands, idx):
 
 
 def price_tiled_gpu(h, w_cluster, w_model, cands, expert_state, expert_param, k=16, fused=False, batch=None,
-                    chunk=None):
+                    chunk=None, thread_min=None):
     """Expert tiling on the GPU through the C ABI: heddle_price_tiled (with
     the tiling planes) and heddle_topk, or heddle_price_topk with ``fused``;
     ``batch`` splits the candidates into consecutive calls."""
@@ -157,6 +157,8 @@ def price_tiled_gpu(h, w_cluster, w_model, cands, expert_state, expert_param, k=
         h.heddle_load_experts(ctx, expert_state, expert_param)
         if chunk is not None:
             h.heddle_set_chunk(ctx, chunk)
+        if thread_min is not None:
+            h.heddle_set_thread_search_min(ctx, thread_min)
         n = int(cands["S"].shape[0])
         dc = h.cands_to_device(cands)
         res = h.alloc_results(n, bounds=False)

@@ -75,7 +75,8 @@ def test_distribute_equal_layers(h, W, oracle_mod, L, kind):
     the layer count: types of almost the same speed (remainders that differ
     in their last bits), of very different speed (stages with no layer of
     their own, surplus layers to take back), and memory that rejects the
-    first alternatives; the fused top-k as well."""
+    first alternatives; the fused top-k as well, and the warp kernel that
+    small batches take."""
     rng = np.random.default_rng(L)
     nt = 5
     tflops = 100.0 * (1.0 + 1e-9 * np.arange(nt)) if kind == "near_tie" else np.geomspace(1.0, 1000.0, nt)
@@ -90,8 +91,9 @@ def test_distribute_equal_layers(h, W, oracle_mod, L, kind):
     code[np.arange(32)[:, None] >= S[None, :]] = 0
     cands = W.make_cands(S, rng.choice([1, 3, 64], n).astype(np.uint16), code)
     ref = oracle_mod.Oracle(cluster, model).set_split("distribute").price(cands, threads=8)
-    for fused in (False, True):
-        got = G.price_gpu(h, cluster, model, cands, k=16, search=h.SEARCH_DISTRIBUTE, fused=fused)
+    for fused, thread_min in ((False, 0), (True, 0), (False, None)):
+        got = G.price_gpu(h, cluster, model, cands, k=16, search=h.SEARCH_DISTRIBUTE, fused=fused,
+                          thread_min=thread_min)
         assert got["errors"] == 0
         G.assert_same(got, ref, what="%s L %d" % (kind, L))
         tk = oracle_mod.topk(ref, cands["M"], 16)

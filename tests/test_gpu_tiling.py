@@ -56,6 +56,18 @@ def test_tiling_parity(h, W, oracle_mod, name, n, seed):
     assert got["topk"]["idx"].tolist() == tk["idx"].tolist()
 
 
+@pytest.mark.parametrize("name,n", [("moe16", 1), ("moe16", 33), ("moe16", 20011), ("moe48", 40009)])
+def test_tiling_memory_probe_first(h, W, oracle_mod, name, n):
+    """The memory probe ahead of the tiled search (forced at any size): the
+    entries it prices OOM, the list it leaves, and the tiling planes."""
+    w = W.make_workload(name, seed=3, n=n)
+    ref = _oracle(oracle_mod, w).price(w.cands, threads=8, tiling=True)
+    got = G.price_tiled_gpu(h, w.cluster, w.model, w.cands, *_experts(w), thread_min=0)
+    assert got["errors"] == 0
+    G.assert_same(got, ref, what="%s tiled" % name)
+    _assert_tiling(got, ref, name)
+
+
 def test_tiling_batches_and_fused_topk(h, W, oracle_mod):
     """Several calls with a ragged tail, and the fused price + top-k call."""
     w = W.make_workload("moe16", seed=2, n=9973)
