@@ -93,10 +93,10 @@ LANES_PER_SM = 128  # 4 SM sub-partitions x 32 lanes issue per clock; the SM cou
 # DRAM bytes (read + write) of one search launch on a 1e6-candidate batch of
 # the stress workload, from an ncu capture, with the SHA-256 of the kernel
 # sources it was taken on; reported as null once those sources change.
-TRAFFIC = {2: {"bytes": 15419136, "batch": 1000000,
-              "sha256": "fa830009fc0782dd6d8b53c00ed919aa761afde74f5a55b872bdc130ccdc3819"}}
+TRAFFIC = {2: {"bytes": 15634944, "batch": 1000000,
+              "sha256": "45336402be485e0894ecdb6ac8a8bf6d9901a6de7820f58abc8fd97c8155fa10"}}
 TRAFFIC_SOURCES = {1: ["heddle_gsearch.cu", "heddle_wsearch.cu", "heddle_wprobe.cuh", "heddle_internal.cuh"],
-                   2: ["heddle_eqsearch.cu", "heddle_internal.cuh"]}
+                   2: ["heddle_eqsearch.cu", "heddle_eq.cuh", "heddle_internal.cuh"]}
 
 
 def traffic_per_launch(search, batch):

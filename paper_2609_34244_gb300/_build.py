@@ -44,9 +44,10 @@ def _deps():
 
 # Variants of the library beside the product build, for the tests:
 # "checked" adds device-side bounds checks that raise an error flag instead of
-# reading or writing out of range, and shrinks the equal-layer search's queue
-# of open searches so its fallback path runs often; "asan" instruments the
-# host code with AddressSanitizer and UndefinedBehaviorSanitizer.
+# reading or writing out of range, and lets the equal-layer search walk no
+# breakpoints, so that its bracketing probes run on every entry; "asan"
+# instruments the host code with AddressSanitizer and
+# UndefinedBehaviorSanitizer.
 VARIANTS = {
     "checked": ["-DHEDDLE_CHECKED=1"],
     "asan": ["-Xcompiler", "-fsanitize=address", "-Xcompiler", "-fsanitize=undefined", "-Xcompiler",

@@ -53,7 +53,7 @@ namespace hd {
 namespace {
 
 constexpr int kMaxIters = 256;
-constexpr int kWalk = 4;  // breakpoints walked before the next probe
+constexpr int kWalk = kChecked ? 0 : 4;  // breakpoints walked before the next probe (the checked build probes only)
 
 // Continuous count at Bf (float): sum_s min(m_s, (Bf - c_s) / q_s), with
 // the slope sum 1/q_s and the number of stages below their run.
