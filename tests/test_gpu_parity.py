@@ -128,6 +128,39 @@ def test_screen_plane_offsets(h, W, oracle_mod, lo, m):
     assert (got["bounds"][:, ok] == ref["bounds"][:, lo:][:, ok]).all()
 
 
+@pytest.mark.parametrize("thread_min", [0, 2**31 - 1])
+@pytest.mark.parametrize("s_max", [1, 3, 4, 5, 8, 9, 16, 17, 32])
+def test_screen_rows_of_stage_bytes(h, W, oracle_mod, s_max, thread_min):
+    """Batches of every depth at which the screen's rows change (a word per 4
+    stages, four or eight lanes a row), after a batch of 32 stages and eight
+    types in the same context: what that one left in the rows past a
+    candidate's depth takes no part, in either search."""
+    old = W.make_workload("stress128", seed=3, n=4096)
+    w = W.make_workload("moe48", seed=4, n=10)
+    rng = np.random.default_rng(s_max)
+    n = 1500
+    S = rng.integers(1, s_max + 1, n).astype(np.uint8)
+    code = W.encode(rng.integers(0, 4, (s_max, n)), rng.integers(0, 3, (s_max, n))).astype(np.uint8)
+    code[np.arange(s_max)[:, None] >= S[None, :]] = 0
+    cands = W.make_cands(S, rng.choice([1, 4, 64], n).astype(np.uint16), code)
+    ref = oracle_mod.Oracle(w.cluster, w.model).price(cands, threads=8)
+    ctx = h.heddle_create(0)
+    try:
+        h.heddle_set_thread_search_min(ctx, thread_min)
+        for cluster, model, batch in ((old.cluster, old.model, old.cands), (w.cluster, w.model, cands)):
+            h.heddle_load_cluster(ctx, cluster)
+            h.heddle_load_model(ctx, model)
+            m = batch["S"].shape[0]
+            dc = h.cands_to_device(batch)
+            res = h.alloc_results(m, bounds=True)
+            h.heddle_price_candidates(ctx, h.make_candidates(dc, 0, m), res)
+            assert h.heddle_device_errors(ctx) == 0
+        got = h.results_to_numpy(res)
+    finally:
+        h.heddle_destroy(ctx)
+    G.assert_same(got, ref, what="s_max %d" % s_max)
+
+
 @pytest.mark.parametrize("name", ["tiny", "dense32", "dense80", "moe48", "stress128"])
 def test_tables_match_oracle(h, W, oracle_mod, name):
     w = W.make_workload(name, n=10)
