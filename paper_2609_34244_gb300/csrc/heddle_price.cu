@@ -77,7 +77,8 @@ constexpr int kRow = kScreenBlock + 16;  // bytes of a tile row: 256 candidates 
 // its own offset, (code + s stride + c0) mod 16, in a row of 272 bytes; only a
 // block that reaches past the arrays is read byte by byte.  (999,983
 // candidates, byte copies after the sort: 55.9 us on the 80-layer workload,
-// 53.6 on the largest, 33.5 on the expert one; these: 52.7, 50.0 and 30.3.)
+// 53.6 on the largest, 33.5 on the expert one; these: 52.7, 50.0 and 30.3;
+// with the rows written as below: 50.3, 50.1 and 29.2.)
 //
 // Instructions bound it (and the search that overlaps it), so the tables are
 // kept in the form in which a stage adds them up: one word that adds the
