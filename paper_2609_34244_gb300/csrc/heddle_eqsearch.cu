@@ -398,7 +398,9 @@ __global__ void __launch_bounds__(kEqBlock, 1024 / kEqBlock) eq_search_kernel(Pr
             // k <= 32): any k entries' smallest key is at most the call's
             // final k-th, so the raised value keeps the filter exact
             const uint32_t nM = (uint32_t)n * (uint32_t)M;
-            const float key = have && T > 0 ? (float)nM / (float)T : -1.0f;
+            // (T = 0, where every layer rounds to 0 ns: the key is infinite,
+            // and so is a threshold that k such entries raised)
+            const float key = have && T >= 0 ? (float)nM / (float)T : -1.0f;
             const int kk = min(max(__ldg(a.topk_k), 1), kMaxTopK);
             float own = 0.f;
             const float thr0 = __uint_as_float(__ldcg(a.thr));

@@ -109,3 +109,43 @@ def test_topk_gather_edges(heddle_lib, oracle_mod, n, kind):
                 _same_state(got, exp, "%s n=%d k=%d up to %d" % (kind, n, k, lo + n))
     finally:
         h.heddle_destroy(ctx)
+
+
+@pytest.mark.parametrize("layers", ("all_free", "some_types_free"))
+@pytest.mark.parametrize("chunk", (None, 701))
+def test_price_topk_keeps_iteration_times_of_zero(heddle_lib, oracle_mod, layers, chunk):
+    """Layers that round to 0 ns on every GPU type, or on the fast one only,
+    with no P2P and no gradient bytes: an OK candidate whose iteration time is
+    0 ranks first.  The fused call (one chunk, several) and the host call hold
+    the same state as the oracle's ranking of all results."""
+    from paper_2609_34244_gb300 import workloads as W
+    import gpu_helpers as G
+    h = heddle_lib
+    rng = np.random.default_rng(3)
+    cluster = W.make_cluster([1000.0, 100.0, 10.0], [10**12] * 3, [10**11] * 3,
+                             [(g, z, 10**10) for g in range(3) for z in (4, 8)] * 4)
+    # 3e5 FLOPs: 0.3 ns on the first type, 3 and 30 on the others
+    model = W.make_model(np.full(12, 0.0 if layers == "all_free" else 3e5), 0, 10**6, 10**5, 0, 0, 0)
+    n = 3001
+    S = rng.integers(1, 4, n).astype(np.uint8)
+    code = W.encode(rng.integers(0, 3, (3, n)), rng.integers(0, 3, (3, n)))
+    code[np.arange(3)[:, None] >= S[None, :]] = 0
+    cands = W.make_cands(S, rng.choice([1, 4, 64], n).astype(np.uint16), code)
+    ref = oracle_mod.Oracle(cluster, model).price(cands, threads=8)
+    assert ((ref["T"] == 0) & (ref["status"] == 0)).sum() > 64
+    for k in (1, 16, 64):
+        exp = oracle_mod.topk(ref, cands["M"], k)
+        for search in (0, 1):
+            got = G.price_gpu(h, cluster, model, cands, k=k, search=search, fused=True, chunk=chunk)
+            assert got["errors"] == 0
+            G.assert_same(got, ref, what=layers)
+            _same_state(got["topk"], exp, "%s k=%d search %d" % (layers, k, search))
+        ctx = h.heddle_create(0)
+        try:
+            h.heddle_load_cluster(ctx, cluster)
+            h.heddle_load_model(ctx, model)
+            state = h.new_topk_state(k)
+            h.heddle_price_topk_host(ctx, cands, None, state, chunk or n)
+            _same_state(h.topk_state_to_dict(state), exp, "%s k=%d host" % (layers, k))
+        finally:
+            h.heddle_destroy(ctx)
