@@ -42,7 +42,11 @@ __device__ int64_t round_half_away(double v) {
     return (int64_t)r;
 }
 
-__device__ int64_t ceil_div(u128 a, u128 b) { return (int64_t)((a + b - 1) / b); }
+// ceil(a / b), at most 2^63 - 1 (a P2P term at 1 byte/s needs 73 bits)
+__device__ int64_t ceil_div(u128 a, u128 b) {
+    const u128 q = (a + b - 1) / b;
+    return q > (u128)kInf ? kInf : (int64_t)q;
+}
 
 // Per stage byte: inadmissible (bit 31), or what the stage adds to its
 // type's demand word -- per class e the GPUs of groups placed in units of at

@@ -394,3 +394,25 @@ def test_call_errors(h, W):
             h.heddle_set_thread_search_min(ctx, v)
     finally:
         h.heddle_destroy(ctx)
+
+
+@pytest.mark.parametrize("boundary,nic,fits", [(1 << 42, 1, False), (1 << 42, 953, False), (1 << 42, 1000, False),
+                                               (549755813, 10**6, True), (549755814, 10**6, False)])
+def test_p2p_limit(h, W, boundary, nic, fits):
+    """A P2P term above 2^40 ns is refused whatever its size: the largest here
+    (2 x 2^42 bytes at 1 byte/s) does not fit 64 bits, and its low half is
+    negative."""
+    assert (-(-2 * boundary * 10**9 // nic) <= 1 << 40) == fits
+    cluster = W.make_cluster([100.0], [10**12], [10**11], [(0, 4, nic), (0, 4, nic)])
+    model = W.make_model(np.full(4, 1e9), 0, 10**6, 10**5, 0, 0, boundary)
+    ctx = h.heddle_create(0)
+    try:
+        h.heddle_load_cluster(ctx, cluster)
+        if fits:
+            h.heddle_load_model(ctx, model)
+        else:
+            with pytest.raises(h.HeddleError) as e:
+                h.heddle_load_model(ctx, model)
+            assert e.value.status == h.E_LIMIT
+    finally:
+        h.heddle_destroy(ctx)
