@@ -76,12 +76,13 @@ __device__ __forceinline__ bool deepest_first(const PriceArgs& a, const int* end
 template <class F>
 __device__ __forceinline__ void for_stages(const PriceArgs& a, const EqTabs& t, const uint16_t* run, int64_t p, int S,
                                            int M, F f) {
-    // the entry's row of stage bytes (zero past S), 16 at a time
+    // the entry's row of stage bytes (zero past S), 16 at a time (ordinary
+    // loads: the screen may have written it while this kernel already ran)
     uint32_t cw4[8];
     {
         const uint4* row = reinterpret_cast<const uint4*>(a.wl_code + p * kMaxStages);
-        const uint4 v0 = __ldg(row);
-        const uint4 v1 = S > 16 ? __ldg(row + 1) : make_uint4(0, 0, 0, 0);
+        const uint4 v0 = row[0];
+        const uint4 v1 = S > 16 ? row[1] : make_uint4(0, 0, 0, 0);
         cw4[0] = v0.x; cw4[1] = v0.y; cw4[2] = v0.z; cw4[3] = v0.w;
         cw4[4] = v1.x; cw4[5] = v1.y; cw4[6] = v1.z; cw4[7] = v1.w;
     }

@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(kEqBlock, 1024 / kEqBlock) eq_search_kernel(Pr
             // (T = 0, where every layer rounds to 0 ns: the key is infinite,
             // and so is a threshold that k such entries raised)
             const float key = have && T >= 0 ? (float)nM / (float)T : -1.0f;
-            const int kk = min(max(__ldg(a.topk_k), 1), kMaxTopK);
+            const int kk = min(max(*a.topk_k, 1), kMaxTopK);
             float own = 0.f;
             const float thr0 = __uint_as_float(__ldcg(a.thr));
             // (only if k of its entries lie above it)

@@ -367,12 +367,14 @@ __global__ void __launch_bounds__(kGBlock, 4) gsearch_kernel(PriceArgs a) {
             if (kCount) ++priced;
             // pack the stages; a bound no split beats and a bound feasible
             // whenever memory is (the entry's 32-byte row of stage bytes, read a byte
-            // per stage: an array indexed by the stage would live in local memory)
+            // per stage: an array indexed by the stage would live in local memory;
+            // ordinary loads: the screen may have written it while this kernel
+            // already ran)
             const uint8_t* row = a.wl_code + p * kMaxStages;
-            int next = __ldg(row);
+            int next = row[0];
             for (int s = 0; s < S; ++s) {
                 const int code = next;
-                next = s + 1 < S ? __ldg(row + s + 1) : 0;
+                next = s + 1 < S ? row[s + 1] : 0;
                 const int gg = code & 7, jj = (code >> 3) & 3;
                 int pidx = kGZeroP2P;
                 if (s + 1 < S) {

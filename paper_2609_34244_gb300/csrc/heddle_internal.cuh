@@ -167,7 +167,9 @@ cudaError_t resident_blocks(const void* func, int block, size_t smem, int* per_s
 // while the previous kernel of its stream still runs, once every CTA of that
 // one has called allow_dependents (or exited); await_previous returns when
 // the previous kernel has completed and its writes are visible (at once when
-// the kernel was launched the ordinary way).  A call of one chunk chains its
+// the kernel was launched the ordinary way).  What the previous kernels write
+// is read by ordinary loads only: the wait does not order the read-only path
+// (__ldg).  A call of one chunk chains its
 // kernels so: with a thousand candidates each runs for little longer than a
 // launch takes.
 __device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
