@@ -45,8 +45,8 @@ def _deps():
 # Variants of the library beside the product build, for the tests:
 # "checked" adds device-side bounds checks that raise an error flag instead of
 # reading or writing out of range, and lets the equal-layer search walk no
-# breakpoints, so that its bracketing probes run on every entry; "asan"
-# instruments the host code with AddressSanitizer and
+# breakpoints on every second entry, so that its bracketing probes run as well;
+# "asan" instruments the host code with AddressSanitizer and
 # UndefinedBehaviorSanitizer.
 VARIANTS = {
     "checked": ["-DHEDDLE_CHECKED=1"],

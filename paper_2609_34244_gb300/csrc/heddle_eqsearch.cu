@@ -53,7 +53,7 @@ namespace hd {
 namespace {
 
 constexpr int kMaxIters = 256;
-constexpr int kWalk = kChecked ? 0 : 4;  // breakpoints walked before the next probe (the checked build probes only)
+constexpr int kWalk = 4;  // breakpoints walked before the next probe
 
 // Continuous count at Bf (float): sum_s min(m_s, (Bf - c_s) / q_s), with
 // the slope sum 1/q_s and the number of stages below their run.
@@ -208,9 +208,9 @@ __device__ __noinline__ void eq_span(const EqTabs& t, const uint32_t* sw, int S,
 }
 
 // B* from the first guess B: returns it, leaves the caps at B* in the stage
-// words and their sum in total.
-__device__ __forceinline__ int64_t eq_threshold(const EqTabs& t, uint32_t* sw, int S, int L, int64_t B, int& total,
-                                                unsigned long long& probes, uint32_t* err) {
+// words and their sum in total.  (walk: kWalk, or 0 to probe only)
+__device__ __forceinline__ int64_t eq_threshold(const EqTabs& t, uint32_t* sw, int S, int L, int64_t B, int walk,
+                                                int& total, unsigned long long& probes, uint32_t* err) {
     int64_t lo = 0, hi = -1;        // B* in [lo, hi] (hi < 0: not computed yet)
     int64_t Blo = -1, Bhi = -1;     // last infeasible / feasible bound probed
     int clo = 0, chi = 0;           // layer counts of those probes
@@ -229,7 +229,7 @@ __device__ __forceinline__ int64_t eq_threshold(const EqTabs& t, uint32_t* sw, i
                     total = p.tot;
                     return p.hi;
                 }
-                if (w >= kWalk || p.tot - L > 2 * kWalk) break;
+                if (w >= walk || p.tot - L > 2 * walk) break;
                 eq_walk_down(t, sw, S, p);
             }
             if (hi < 0) eq_span(t, sw, S, lo, hi);
@@ -238,8 +238,8 @@ __device__ __forceinline__ int64_t eq_threshold(const EqTabs& t, uint32_t* sw, i
             chi = tot;
         } else {
             const int64_t next = p.lo;
-            if (!p.jump && L - tot <= 2 * kWalk) {
-                for (int w = 0; w < kWalk && p.lo < kInf; ++w) {
+            if (!p.jump && L - tot <= 2 * walk) {
+                for (int w = 0; w < walk && p.lo < kInf; ++w) {
                     eq_walk_up(t, sw, S, p);
                     if (p.feasible(L)) {
                         total = p.tot;
@@ -287,7 +287,7 @@ __device__ __forceinline__ int64_t eq_evaluate(const PriceArgs& a, const EqTabs&
                                                int64_t Bstar, int total) {
     const int64_t c = a.wl_idx[p];
     if (!in_range(c, a.n, a.err)) return -1;
-    int64_t tsum = 0;
+    int64_t tsum = 0, tmax = 0;
     GradMax grad;
     int pre = 0, at = 0;
     for (int s = 0; s < S; ++s) {
@@ -298,7 +298,9 @@ __device__ __forceinline__ int64_t eq_evaluate(const PriceArgs& a, const EqTabs&
         if (a.bounds) a.bounds[(int64_t)(s + 1) * a.bstride + c] = (uint8_t)nxt;
         const int len = nxt - at;
         if (len > k) atomicOr(a.err, kErrInternal);
-        tsum += (int64_t)len * t.q[w & 31] + t.p2p[p2p_of(w)];
+        const int64_t ts = (int64_t)len * t.q[w & 31] + t.p2p[p2p_of(w)];
+        tmax = max(tmax, ts);
+        tsum += ts;
         if (n > 1) grad.add(t, PB, pbytes, w & 31, at, nxt);
         at = nxt;
     }
@@ -307,7 +309,8 @@ __device__ __forceinline__ int64_t eq_evaluate(const PriceArgs& a, const EqTabs&
         if (!a.bounds_scratch)
             for (int s = S + 1; s <= kMaxStages; ++s) a.bounds[(int64_t)s * a.bstride + c] = 0;
     }
-    if (pre != total) atomicOr(a.err, kErrInternal);
+    // (a bound above B* would pass the test of the lengths)
+    if (pre != total || tmax != Bstar) atomicOr(a.err, kErrInternal);
     const int64_t gmax = n > 1 ? grad.sync_ns(n, pbytes, a.err) : 0;
     const int64_t T = (int64_t)(M - 1) * Bstar + tsum + gmax;
     a.T[c] = T;
@@ -386,8 +389,11 @@ __global__ void __launch_bounds__(kEqBlock, 1024 / kEqBlock) eq_search_kernel(Pr
                 Bf += (tgt - cnt) / sl;
             }
             int total = 0;
+            // (the checked build probes only for every second entry, so that
+            // both the walk and the bracketing run)
+            const int walk = kChecked && (p & 1) ? 0 : kWalk;
             const int64_t Bstar =
-                eq_threshold(t, mysw, S, L, (int64_t)float_to_u64(Bf), total, probes, a.err);
+                eq_threshold(t, mysw, S, L, (int64_t)float_to_u64(Bf), walk, total, probes, a.err);
             T = eq_evaluate(a, t, PB, pbytes, mysw, p, S, M, n, L, Bstar, total);
         }
         if (a.sv_count) {

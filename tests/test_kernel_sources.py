@@ -22,3 +22,12 @@ def test_dependent_kernels_read_only_the_tables_through_the_read_only_path():
         for arg in re.findall(r"__ldg\(([^()]*)\)", text):
             base = arg.split("+")[0].strip()
             assert base in tables, "%s: __ldg(%s)" % (os.path.basename(path), arg)
+
+
+def test_every_search_checks_that_its_split_attains_the_bound():
+    """A threshold search that returned a bound above B* would report it with a
+    split that keeps it; each of the three raises the consistency flag unless
+    the split's largest stage time equals the bound."""
+    for name in ("heddle_eqsearch.cu", "heddle_gsearch.cu", "heddle_wsearch.cu"):
+        text = open(os.path.join(CSRC, name)).read()
+        assert re.search(r"tmax != Bstar\) atomicOr\(a\.err, kErrInternal\)", text), name
