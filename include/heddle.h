@@ -485,10 +485,12 @@ heddle_status heddle_get_search(heddle_ctx* ctx, int32_t* in_use);
  * takes the worklist entries when there are at least min_entries of them, and
  * the warp-per-entry search prices those it cannot decide; with fewer, the
  * warp search prices every entry (a thread search with too few entries runs
- * as long as its longest serial chain).  min_entries < 0 restores the
- * default, 32 x the device's SM count; 0 always runs the thread search, and
- * the thread-per-entry kernels of the split rule and of the tiled search's
- * memory probe, which otherwise run from a batch size on.  All routes return
+ * as long as its longest serial chain).  The split rule of equal-layer models
+ * (DISTRIBUTE) has two such kernels as well.  min_entries < 0 restores the
+ * default, 32 x the device's SM count for the general search and, for the
+ * split rule, 5,000 and 550 more per stage of the deepest entry; 0 always runs
+ * the thread kernels, and the memory probe ahead of the tiled search, which
+ * otherwise runs from a batch size on.  All routes return
  * identical results.  Errors: E_ARG (ctx NULL). */
 heddle_status heddle_set_thread_search_min(heddle_ctx* ctx, int32_t min_entries);
 

@@ -737,6 +737,8 @@ void fill_price_args(heddle_ctx* x, const heddle_candidates* c, const heddle_ctx
     a.equal_layers = flags[0] && flags[1] ? 1 : 0;
     a.split_mode = x->search_mode == HEDDLE_SEARCH_DISTRIBUTE ? 1 : 0;
     a.thread_min = x->thread_min < 0 ? hd::thread_search_min(x->num_sms) : x->thread_min;
+    a.split_min = x->thread_min < 0 ? hd::kSplitThreadMin : x->thread_min;
+    a.split_per_stage = x->thread_min < 0 ? hd::kSplitThreadPerStage : 0;
 }
 
 // One chunk [lo, lo + nb) of cands into r: screen and search on `ws` with
@@ -817,7 +819,7 @@ heddle_status price_chunk(heddle_ctx* x, hd::PriceArgs& a, const heddle_candidat
         m.wl_nM = survivors ? W.sv_nM : W.nM;
         m.wl_cap = hd::kWorklistCap;
         m.survivors = survivors ? 1 : 0;
-        m.chained = a.chained && !a.split_mode && !tiled;
+        m.chained = a.chained && !tiled;
         m.thr = a.thr;
         CU(hd::launch_topk_worklist(m, nb, x->num_sms, cs, nl ? nl + 2 : nullptr));
         if (x->time_phases) CU(cudaEventRecord(rec.e[4], cs));

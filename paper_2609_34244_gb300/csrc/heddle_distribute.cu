@@ -28,7 +28,10 @@
 // two that differ share a key at the cut.  1e6 candidates of the largest
 // workload: 260 -> 62 us (one warp per entry, a lane per stage: 64-bit
 // divisions, sums and ranks by shuffles, half the lanes past the depth).
-// Other models keep that warp kernel, whose lanes read the prefix tables.
+// Other models keep that warp kernel, whose lanes read the prefix tables, and so
+// do few entries, for which a thread's serial chain is the longer: both are
+// launched, and by the entries per depth one of them returns at once (100
+// entries of 70,000 candidates: 74 us a pass by threads, 33 so).
 
 #include <algorithm>
 
@@ -85,8 +88,20 @@ __device__ int share_count(bool live, int S, int L, int64_t w, int64_t V, int la
     return cnt;
 }
 
-__global__ void __launch_bounds__(kDistBlock) distribute_kernel(PriceArgs a) {
+// Whether the entries are priced by a thread each (split_kernel) or a warp each
+// (distribute_kernel); every lane of a warp calls it.
+__device__ __forceinline__ bool split_by_threads(const PriceArgs& a) {
+    const int here = a.wl_count[1 + 1 + (threadIdx.x & 31)];  // entries of depth 1 + lane
+    const int deepest = 32 - __clz(__ballot_sync(kFull, here > 0));
+    return __reduce_add_sync(kFull, (unsigned)here) >= (unsigned)(a.split_min + a.split_per_stage * deepest);
+}
+
+// (both_launched: split_kernel follows, for the entries it takes)
+__global__ void __launch_bounds__(kDistBlock) distribute_kernel(PriceArgs a, int both_launched) {
     const Layout& y = a.lay;
+    allow_dependents();
+    await_previous();
+    if (both_launched && split_by_threads(a)) return;
     const int L = y.L;
     const int64_t* P = reinterpret_cast<const int64_t*>(a.img + y.offP);
     const longlong2* SA = reinterpret_cast<const longlong2*>(a.img + y.offSA);
@@ -215,8 +230,6 @@ __global__ void __launch_bounds__(kDistBlock) distribute_kernel(PriceArgs a) {
 
 // ---- equal layers: one thread per entry
 
-constexpr int64_t kThreadSplitMin = 1 << 16;
-
 struct SplitShared {
     EqTabs tab;
     uint16_t run[32 * 33 + 256];         // ScreenTabs::run
@@ -341,6 +354,9 @@ __global__ void __launch_bounds__(kEqBlock, 5) split_kernel(PriceArgs a) {
     const Layout& y = a.lay;
     const int L = y.L;
     load_eq_tables(a, sh.tab, sh.run);
+    allow_dependents();
+    await_previous();  // the screen's worklist
+    if (!split_by_threads(a)) return;  // distribute_kernel has priced it
     depth_ends(a.wl_count, end_of);
     __syncthreads();
     if (threadIdx.x < 32) {
@@ -448,25 +464,19 @@ __global__ void __launch_bounds__(kEqBlock, 5) split_kernel(PriceArgs a) {
 }  // namespace
 
 cudaError_t launch_distribute(const PriceArgs& a, int num_sms, cudaStream_t st) {
-    // (a thread's entry takes 30 us of latency, a warp's 15; past some ten
-    // thousand entries the thread kernel's five times fewer instructions
-    // decide: 443 candidates of 22 stages take 55 us a pass by threads and 39
-    // by warps, 35,373 of 32 stages 78 and 67, 141,586 of 27 stages 79 and 150;
-    // a thread_min of zero asks for threads at any size)
-    if (a.equal_layers && (a.n >= kThreadSplitMin || a.thread_min == 0)) {
-        const size_t smem = sizeof(SplitShared);
-        int per_sm = 0;
-        const cudaError_t e = resident_blocks(reinterpret_cast<const void*>(&split_kernel), kEqBlock, smem, &per_sm);
-        if (e != cudaSuccess) return e;
-        if (per_sm < 1) return cudaErrorInvalidConfiguration;
-        const int grid = (int)std::min<int64_t>((a.n + kEqBlock - 1) / kEqBlock, (int64_t)num_sms * per_sm);
-        split_kernel<<<grid, kEqBlock, smem, st>>>(a);
-        return cudaGetLastError();
-    }
     // one warp per entry; the worklist length is only known on the device
     const int grid = (int)std::min<int64_t>((a.n + kDistBlock / 32 - 1) / (kDistBlock / 32), (int64_t)num_sms * 16);
-    distribute_kernel<<<grid, kDistBlock, 0, st>>>(a);
-    return cudaGetLastError();
+    // (a batch too small for the thread kernel at any depth does without it)
+    const bool threads = a.equal_layers && a.n >= (int64_t)a.split_min + a.split_per_stage;
+    cudaError_t e = launch_after(a.chained, distribute_kernel, grid, kDistBlock, 0, st, a, threads ? 1 : 0);
+    if (e != cudaSuccess || !threads) return e;
+    const size_t smem = sizeof(SplitShared);
+    int per_sm = 0;
+    e = resident_blocks(reinterpret_cast<const void*>(&split_kernel), kEqBlock, smem, &per_sm);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    const int tgrid = (int)std::min<int64_t>((a.n + kEqBlock - 1) / kEqBlock, (int64_t)num_sms * per_sm);
+    return launch_after(a.chained, split_kernel, tgrid, kEqBlock, smem, st, a);
 }
 
 }  // namespace hd

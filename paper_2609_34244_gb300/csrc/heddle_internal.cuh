@@ -238,6 +238,7 @@ struct PriceArgs {
     int32_t equal_layers;  // every layer has the same time per (type, degree) and the same memory
     int32_t split_mode;  // 1: the paper's own split rule (distribute_kernel) instead of PartitionLayers
     int32_t thread_min;  // general search: the bucketed entries below which only the warp search runs
+    int32_t split_min, split_per_stage;  // split rule of equal layers: see split_by_threads
     // per worklist entry, written by the search: T (-1 unless OK) and n * M,
     // so a top-k can run over the searched candidates only
     int64_t* wl_T;
@@ -302,7 +303,14 @@ cudaError_t launch_plans(const PlanArgs& a, int num_sms, cudaStream_t st);
 // wl_count[kWlGeneral]); does nothing below a.thread_min bucketed entries.
 cudaError_t launch_memory_probe(const PriceArgs& a, int num_sms, cudaStream_t st);
 
-// The paper's own layer split over the worklist (comparison mode).
+// The paper's own layer split over the worklist (comparison mode).  On a model
+// of equal layers a thread prices each entry when the depth buckets hold at
+// least PriceArgs::split_min plus split_per_stage entries for each stage of the
+// deepest one, else a warp does (the device decides: few of a large batch may
+// reach the search).  A warp's entries take 1.8 to 2.2 us per thousand, a
+// thread's chain 5, 9, 18 or 41 us more than a warp's at 3, 8, 16 or 32 stages:
+// measured, they meet at some 6,800, 9,500, 14,500 and 22,000 entries.
+constexpr int32_t kSplitThreadMin = 5000, kSplitThreadPerStage = 550;
 cudaError_t launch_distribute(const PriceArgs& a, int num_sms, cudaStream_t st);
 constexpr int32_t kWorklistCap = 1 << 20;
 constexpr int kWlMeta = 1 + kMaxStages + 1 + 2 + 1;  // ints of a.wl_count

@@ -98,3 +98,20 @@ def test_distribute_equal_layers(h, W, oracle_mod, L, kind):
         G.assert_same(got, ref, what="%s L %d" % (kind, L))
         tk = oracle_mod.topk(ref, cands["M"], 16)
         assert got["topk"]["idx"].tolist() == tk["idx"].tolist()
+
+
+def test_distribute_routes_meet(h, W, oracle_mod):
+    """Both kernels of the equal-layer split launched, the entries just enough
+    for the thread kernel and one too few; one chunk and several."""
+    w = W.make_workload("stress128", seed=6, n=9001)
+    ref = oracle_mod.Oracle(w.cluster, w.model).set_split("distribute").price(w.cands, threads=8)
+    count = G.price_gpu(h, w.cluster, w.model, w.cands, bounds=False, count=True)["counters"]["priced"]
+    assert 0 < count < 9001
+    tk = oracle_mod.topk(ref, w.cands["M"], 16)
+    for thread_min in (count, count + 1, 9001):
+        for chunk in (None, 4000):
+            got = G.price_gpu(h, w.cluster, w.model, w.cands, k=16, search=h.SEARCH_DISTRIBUTE, fused=True,
+                              chunk=chunk, thread_min=thread_min)
+            assert got["errors"] == 0
+            G.assert_same(got, ref, what="thread_min %d chunk %s" % (thread_min, chunk))
+            assert got["topk"]["idx"].tolist() == tk["idx"].tolist()

@@ -1,0 +1,64 @@
+"""What a call costs follows from what has to be priced, not from the size of
+the buffers it lies in: passes timed with CUDA events against one another
+(medians; the limits leave a third for noise)."""
+
+import statistics
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def h(heddle_lib):
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    return heddle_lib
+
+
+@pytest.fixture(scope="module")
+def W():
+    from paper_2609_34244_gb300 import workloads
+    return workloads
+
+
+def pass_us(f, reps=20):
+    """Microseconds of one pass among others (the median of nine groups)."""
+    import torch
+    for _ in range(5):
+        f()
+    torch.cuda.synchronize()
+    out = []
+    for _ in range(9):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record()
+        for _ in range(reps):
+            f()
+        e1.record()
+        torch.cuda.synchronize()
+        out.append(e0.elapsed_time(e1) * 1e3 / reps)
+    return statistics.median(out)
+
+
+def test_split_rule_cost_follows_the_entries(h, W):
+    """A hundred admissible structures of 32 stages among 60,000 invalid ones
+    and among 140,000: a thread's chain of 32 stages is twice a warp's."""
+    us = []
+    for n in (60_000, 140_000):
+        w = W.make_workload("stress128", seed=7, n=n)
+        live = np.zeros(n, bool)
+        live[np.random.default_rng(1).choice(n, 100, replace=False)] = True
+        w.cands["code"][0, ~live] |= 0x20
+        ctx = h.heddle_create(0)
+        try:
+            h.heddle_load_cluster(ctx, w.cluster)
+            h.heddle_load_model(ctx, w.model)
+            h.heddle_set_search(ctx, h.SEARCH_DISTRIBUTE)
+            dc, res, state = h.cands_to_device(w.cands), h.alloc_results(n), h.alloc_topk_state()
+            h.heddle_topk_reset(ctx, state, 16)
+            us.append(pass_us(lambda: h.heddle_price_topk(ctx, dc, res, state)))
+            assert h.heddle_device_errors(ctx) == 0
+        finally:
+            h.heddle_destroy(ctx)
+    assert us[1] < 1.33 * us[0], us
