@@ -486,11 +486,13 @@ heddle_status heddle_get_search(heddle_ctx* ctx, int32_t* in_use);
  * the warp-per-entry search prices those it cannot decide; with fewer, the
  * warp search prices every entry (a thread search with too few entries runs
  * as long as its longest serial chain).  The split rule of equal-layer models
- * (DISTRIBUTE) has two such kernels as well.  min_entries < 0 restores the
- * default, 32 x the device's SM count for the general search and, for the
- * split rule, 5,000 and 550 more per stage of the deepest entry; 0 always runs
- * the thread kernels, and the memory probe ahead of the tiled search, which
- * otherwise runs from a batch size on.  All routes return
+ * (DISTRIBUTE) has two such kernels as well, and heddle_price_plans two walks:
+ * there min_entries counts the plans queued by one CTA (at most 255).
+ * min_entries < 0 restores the defaults: 32 x the device's SM count for the
+ * general search; 5,000 entries, and 550 more per stage of the deepest, for the
+ * split rule; 20 queued plans, and 5 more per stage of the deepest, for the plan
+ * walk.  0 always runs the thread kernels, and the memory probe ahead of the
+ * tiled search, which otherwise runs from a batch size on.  All routes return
  * identical results.  Errors: E_ARG (ctx NULL). */
 heddle_status heddle_set_thread_search_min(heddle_ctx* ctx, int32_t min_entries);
 

@@ -1326,11 +1326,7 @@ heddle_status heddle_price_plans(heddle_ctx* x, const heddle_plans* pl, const he
     a.node_gpus = x->d_node_gpus;
     a.n_nodes = (int32_t)nn;
     a.vmax = vmax;
-    // a warp's walks take about 4 us / 4 warps each, a thread's alone 20 us
-    // and 5 us a stage: they meet at 20 + 5 stages
-    int32_t deepest = 1;
-    for (int t = 0; t < pl->slots; ++t) deepest = std::max(deepest, pl->t[t].s_max);
-    a.alone_min = 20 + 5 * deepest;
+    a.alone_min = x->thread_min < 0 ? 0 : std::max(x->thread_min, 1);
     a.placed = pr->placed;
     a.thr = pr->thr;
     a.err = x->d_flags + 1;

@@ -292,7 +292,7 @@ struct PlanArgs {
     int32_t n_nodes;
     int32_t vmax;  // largest node (GPUs), <= kPlanMaxNode
     int32_t per_pass;   // plans a CTA looks at in one pass (at most 128): batches of few spread over all SMs
-    int32_t alone_min;  // queued plans of a CTA from which a thread walks each
+    int32_t alone_min;  // queued plans of a CTA from which a thread walks each (0: by their depth)
     uint8_t* placed;
     double* thr;
     uint32_t* err;

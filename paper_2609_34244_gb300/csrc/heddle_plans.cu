@@ -31,9 +31,13 @@
 // A CTA looks at no more plans at a time than spread the batch over all SMs
 // (1,308 plans of up to twelve stages: 229 -> 128 us a call, 212 by threads).
 // Where most plans of a large batch walk -- shallow templates -- a thread each
-// does several times the walks per instruction: from alone_min plans in a
-// CTA's queue on they are walked so, 128 at a time (52,002 plans of up to five
-// stages: 205 us a call by warps alone, 140 with both).
+// does several times the walks per instruction, 128 at a time.  A warp's walks
+// take about 4 us / 4 warps each, a thread's alone 20 us and 5 us a stage: from
+// 20 queued plans of a CTA on, and 5 more per stage of the deepest of them, they
+// are walked so (52,002 plans of up to five stages: 205 us a call by warps
+// alone, 140 with both).  The depth is the plans' own, not the planes of the
+// buffers they lie in: 200,003 plans of up to two stages in 32 planes took 540 us
+// by the planes, 267 in two.
 
 #include <algorithm>
 
@@ -81,8 +85,8 @@ __global__ void __launch_bounds__(kPlanBlock, 8) plan_kernel(PlanArgs a) {
     // such plans, and the others are queued in shared memory and walked a
     // warp each.
     __shared__ int32_t queue[2 * kPlanBlock];
-    __shared__ int queued;
-    if (threadIdx.x == 0) queued = 0;
+    __shared__ int queued, deepest;  // (of the queued plans' templates)
+    if (threadIdx.x == 0) queued = deepest = 0;
     __syncthreads();
     // ---- one thread a plan: per-thread arrays in shared memory, interleaved
     // by thread (element e of thread t at [e * kPlanBlock + t]): the node
@@ -403,15 +407,21 @@ __global__ void __launch_bounds__(kPlanBlock, 8) plan_kernel(PlanArgs a) {
         if (more) {
             const int64_t c = c0 + threadIdx.x;
             bool walks = false;
+            int depth = 0;
             if ((int)threadIdx.x < a.per_pass && c < a.n) {
                 // a plan walks from its second template on; the others keep
                 // their slots as priced (templates past the first OK-alone
                 // prefix were priced SKIPPED) and take the first template's
                 // throughput if it is OK
                 const int nt = min((int)a.n_tmpl[c], a.slots);
+                for (int t = 0; t < a.slots; ++t) {  // (loads beside the status's)
+                    const int S = a.slot[t].S[c];
+                    if (t < nt) depth = max(depth, min(S, kMaxStages));
+                }
                 const bool ok0 = nt >= 1 && a.slot[0].status[c] == HEDDLE_CAND_OK;
                 walks = ok0 && nt >= 2;
                 if (!walks) {
+                    depth = 0;
                     double thr = 0.0;
                     if (ok0) {
                         const PlanSlot& s0 = a.slot[0];
@@ -428,19 +438,22 @@ __global__ void __launch_bounds__(kPlanBlock, 8) plan_kernel(PlanArgs a) {
                 if (lane == __ffs(wm) - 1) q0 = atomicAdd(&queued, __popc(wm));
                 q0 = __shfl_sync(0xffffffffu, q0, __ffs(wm) - 1);
                 if (walks) queue[q0 + __popc(wm & ((1u << lane) - 1))] = (int32_t)(c0 + threadIdx.x);
+                const int deep = (int)__reduce_max_sync(kFull, (unsigned)depth);
+                if (lane == 0) atomicMax(&deepest, deep);
             }
         }
         __syncthreads();
         const int have = queued;
+        const int alone_min = a.alone_min > 0 ? a.alone_min : 20 + 5 * deepest;
         __syncthreads();
         if (have >= kPlanBlock || !more) {
-            if (have >= a.alone_min) {  // 128 at a time, a thread each, while that many are left
+            if (have >= alone_min) {  // 128 at a time, a thread each, while that many are left
                 const int n1 = min(have, kPlanBlock);
                 if (threadIdx.x < n1) walk_alone(queue[have - n1 + threadIdx.x]);
                 if (threadIdx.x == 0) queued = have - n1;
             } else {  // a warp each
                 for (int i = warp; i < have; i += kPlanWarps) walk(queue[i]);
-                if (threadIdx.x == 0) queued = 0;
+                if (threadIdx.x == 0) queued = deepest = 0;
             }
         }
         __syncthreads();

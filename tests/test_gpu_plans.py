@@ -25,7 +25,7 @@ def W():
     return workloads
 
 
-def price_plans_gpu(h, cluster, model, plans, search=None, bounds=False):
+def price_plans_gpu(h, cluster, model, plans, search=None, bounds=False, thread_min=None):
     import torch
     ctx = h.heddle_create(0)
     try:
@@ -33,6 +33,8 @@ def price_plans_gpu(h, cluster, model, plans, search=None, bounds=False):
         h.heddle_load_model(ctx, model)
         if search is not None:
             h.heddle_set_search(ctx, search)
+        if thread_min is not None:
+            h.heddle_set_thread_search_min(ctx, thread_min)
         dp = h.plans_to_device(plans)
         n = int(plans["n_tmpl"].shape[0])
         pr = h.alloc_plan_results(n, len(dp["slots"]), bounds=bounds)
@@ -159,3 +161,67 @@ def test_plans_limits(h, W):
         assert e.value.status == 3  # E_LIMIT: a node above the plan limit
     finally:
         h.heddle_destroy(ctx)
+
+
+ROUTES = {"threads": 0, "warps": 2**31 - 1, "default": None}
+
+
+def _bounds_same(orc, plans, got, idx=None):
+    """OK templates hold their standalone split (the oracle's), others zeros;
+    of every plan, or of plans idx."""
+    idx = slice(None) if idx is None else idx
+    for t, b in enumerate(got["bounds"]):
+        alone = orc.price({"S": np.ascontiguousarray(plans["S"][t][idx]), "M": np.ascontiguousarray(plans["M"][t][idx]),
+                           "code": np.ascontiguousarray(plans["code"][t][:, idx])}, bounds=True)
+        ok = got["status"][t][idx] == 0
+        assert (b[:, idx][:, ok] == alone["bounds"][:, ok]).all(), t
+        assert (b[:, got["status"][t] != 0] == 0).all(), t
+
+
+@pytest.mark.parametrize("name,n", [("tiny", 33), ("dense32", 1), ("dense32", 4001), ("moe48", 2003),
+                                    ("stress128", 1501)])
+@pytest.mark.parametrize("route", ROUTES)
+def test_plan_walk_routes(h, W, oracle_mod, name, n, route):
+    """Every walking plan by a thread, by a warp, and by the default rule, with
+    memory that most templates fit (so that plans walk to their last one)."""
+    w = W.make_workload(name, seed=2, n=n)
+    w.cluster["mem_bytes"][:] = 10**12
+    plans = W.make_plans(w, n, 4, seed=2)
+    orc = oracle_mod.Oracle(w.cluster, w.model)
+    ref = orc.price_plans(plans)
+    got = price_plans_gpu(h, w.cluster, w.model, plans, bounds=True, thread_min=ROUTES[route])
+    assert got["errors"] == 0
+    _same(got, ref, "%s %s" % (name, route))
+    _bounds_same(orc, plans, got)
+    if n > 1000:
+        assert (ref["placed"] >= 2).mean() > 0.2
+
+
+@pytest.mark.parametrize("deepest", [2, 5])
+def test_plan_walk_queues_fill(h, W, oracle_mod, deepest):
+    """200,003 plans, most of which walk: a CTA looks at 128 at a time, its
+    queue passes 128 and leaves a remainder.  The routes against each other,
+    and the default one against the oracle on a sample."""
+    n = 200_003
+    w = W.make_workload("dense32", seed=5, n=n)
+    w.cluster["mem_bytes"][:] = 10**12
+    plans = W.make_plans(w, n, 4, seed=5)
+    plans["S"] = np.minimum(plans["S"], deepest).astype(plans["S"].dtype)
+    plans["code"] = np.ascontiguousarray(plans["code"][:, :deepest])
+    plans["code"][np.arange(deepest)[None, :, None] >= plans["S"][:, None, :]] = 0
+    got = {r: price_plans_gpu(h, w.cluster, w.model, plans, bounds=True, thread_min=m) for r, m in ROUTES.items()}
+    walks = (got["warps"]["status"][0] == 0) & (plans["n_tmpl"] >= 2)
+    assert walks.mean() > 0.6
+    for r in ROUTES:
+        assert got[r]["errors"] == 0
+        _same(got[r], got["warps"], "%s against warps" % r)
+        for t in range(4):
+            assert (got[r]["bounds"][t] == got["warps"]["bounds"][t]).all(), (r, t)
+    idx = np.random.default_rng(1).choice(n, 3000, replace=False)
+    some = {"n_tmpl": plans["n_tmpl"][idx], "S": np.ascontiguousarray(plans["S"][:, idx]),
+            "M": np.ascontiguousarray(plans["M"][:, idx]), "code": np.ascontiguousarray(plans["code"][:, :, idx])}
+    orc = oracle_mod.Oracle(w.cluster, w.model)
+    ref = orc.price_plans(some)
+    d = got["default"]
+    _same({k: d[k][..., idx] for k in ("T", "bottleneck", "n_dp", "status", "placed", "thr")}, ref, "sample")
+    _bounds_same(orc, plans, d, idx)

@@ -62,3 +62,30 @@ def test_split_rule_cost_follows_the_entries(h, W):
         finally:
             h.heddle_destroy(ctx)
     assert us[1] < 1.33 * us[0], us
+
+
+def test_plan_walk_cost_follows_the_depth(h, W):
+    """Plans of up to two stages in buffers of two planes and of 32: the walk
+    goes by the plans' depth."""
+    n = 200_003
+    w = W.make_workload("dense32", seed=5, n=n)
+    w.cluster["mem_bytes"][:] = 192 * 10**9
+    plans = W.make_plans(w, n, 4, seed=5)
+    plans["S"] = np.minimum(plans["S"], 2).astype(plans["S"].dtype)
+    us = []
+    for planes in (2, 32):
+        code = np.zeros((4, planes, n), np.uint8)
+        code[:, :2] = plans["code"][:, :2]
+        code[:, 1][plans["S"] < 2] = 0
+        dp = h.plans_to_device(dict(plans, code=code))
+        ctx = h.heddle_create(0)
+        try:
+            h.heddle_load_cluster(ctx, w.cluster)
+            h.heddle_load_model(ctx, w.model)
+            pr = h.alloc_plan_results(n, 4)
+            us.append(pass_us(lambda: h.heddle_price_plans(ctx, dp, pr)))
+            assert (pr["placed"] >= 2).float().mean() > 0.3
+            assert h.heddle_device_errors(ctx) == 0
+        finally:
+            h.heddle_destroy(ctx)
+    assert us[1] < 1.33 * us[0], us
