@@ -49,6 +49,8 @@ namespace {
 constexpr int kPlanBlock = 128;
 constexpr int kPlanWarps = kPlanBlock / 32;
 constexpr unsigned kFull = 0xffffffffu;
+// queued plans of a CTA from which a thread walks each (see the head of this file)
+constexpr int kAloneMin = 20, kAlonePerStage = 5;
 
 inline size_t plan_smem(int NT, int vmax) { return (size_t)kPlanBlock * (2 * (size_t)NT * (vmax + 1) + 8 * kMaxTypes); }
 
@@ -85,8 +87,9 @@ __global__ void __launch_bounds__(kPlanBlock, 8) plan_kernel(PlanArgs a) {
     // such plans, and the others are queued in shared memory and walked a
     // warp each.
     __shared__ int32_t queue[2 * kPlanBlock];
-    __shared__ int queued, deepest;  // (of the queued plans' templates)
-    if (threadIdx.x == 0) queued = deepest = 0;
+    __shared__ int queued;
+    __shared__ int deep[kPlanWarps];  // per warp: the deepest template of the queued plans it looked at
+    if (threadIdx.x == 0) queued = 0;
     __syncthreads();
     // ---- one thread a plan: per-thread arrays in shared memory, interleaved
     // by thread (element e of thread t at [e * kPlanBlock + t]): the node
@@ -407,21 +410,15 @@ __global__ void __launch_bounds__(kPlanBlock, 8) plan_kernel(PlanArgs a) {
         if (more) {
             const int64_t c = c0 + threadIdx.x;
             bool walks = false;
-            int depth = 0;
             if ((int)threadIdx.x < a.per_pass && c < a.n) {
                 // a plan walks from its second template on; the others keep
                 // their slots as priced (templates past the first OK-alone
                 // prefix were priced SKIPPED) and take the first template's
                 // throughput if it is OK
                 const int nt = min((int)a.n_tmpl[c], a.slots);
-                for (int t = 0; t < a.slots; ++t) {  // (loads beside the status's)
-                    const int S = a.slot[t].S[c];
-                    if (t < nt) depth = max(depth, min(S, kMaxStages));
-                }
                 const bool ok0 = nt >= 1 && a.slot[0].status[c] == HEDDLE_CAND_OK;
                 walks = ok0 && nt >= 2;
                 if (!walks) {
-                    depth = 0;
                     double thr = 0.0;
                     if (ok0) {
                         const PlanSlot& s0 = a.slot[0];
@@ -438,22 +435,37 @@ __global__ void __launch_bounds__(kPlanBlock, 8) plan_kernel(PlanArgs a) {
                 if (lane == __ffs(wm) - 1) q0 = atomicAdd(&queued, __popc(wm));
                 q0 = __shfl_sync(0xffffffffu, q0, __ffs(wm) - 1);
                 if (walks) queue[q0 + __popc(wm & ((1u << lane) - 1))] = (int32_t)(c0 + threadIdx.x);
-                const int deep = (int)__reduce_max_sync(kFull, (unsigned)depth);
-                if (lane == 0) atomicMax(&deepest, deep);
             }
         }
         __syncthreads();
         const int have = queued;
-        const int alone_min = a.alone_min > 0 ? a.alone_min : 20 + 5 * deepest;
         __syncthreads();
         if (have >= kPlanBlock || !more) {
+            int alone_min = a.alone_min;
+            if (alone_min == 0) {  // by the depth of the queued plans
+                alone_min = kAloneMin;
+                if (have >= alone_min) {
+                    unsigned depth = 0;
+                    for (int i = threadIdx.x; i < have; i += kPlanBlock) {
+                        const int64_t c = queue[i];
+                        const int nt = min((int)a.n_tmpl[c], a.slots);
+                        for (int t = 0; t < nt; ++t) depth = max(depth, min((unsigned)a.slot[t].S[c], (unsigned)kMaxStages));
+                    }
+                    depth = __reduce_max_sync(kFull, depth);
+                    if (lane == 0) deep[warp] = (int)depth;
+                    __syncthreads();
+                    int deepest = 0;
+                    for (int w = 0; w < kPlanWarps; ++w) deepest = max(deepest, deep[w]);
+                    alone_min += kAlonePerStage * deepest;
+                }
+            }
             if (have >= alone_min) {  // 128 at a time, a thread each, while that many are left
                 const int n1 = min(have, kPlanBlock);
                 if (threadIdx.x < n1) walk_alone(queue[have - n1 + threadIdx.x]);
                 if (threadIdx.x == 0) queued = have - n1;
             } else {  // a warp each
                 for (int i = warp; i < have; i += kPlanWarps) walk(queue[i]);
-                if (threadIdx.x == 0) queued = deepest = 0;
+                if (threadIdx.x == 0) queued = 0;
             }
         }
         __syncthreads();
