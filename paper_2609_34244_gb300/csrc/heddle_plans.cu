@@ -52,7 +52,28 @@ constexpr unsigned kFull = 0xffffffffu;
 // queued plans of a CTA from which a thread walks each (see the head of this file)
 constexpr int kAloneMin = 20, kAlonePerStage = 5;
 
-inline size_t plan_smem(int NT, int vmax) { return (size_t)kPlanBlock * (2 * (size_t)NT * (vmax + 1) + 8 * kMaxTypes); }
+// Dynamic shared memory: per thread (interleaved by thread, element e of thread t
+// at [e * kPlanBlock + t]) the demand word per type and the node histogram, or,
+// while warps walk, an area per warp in the same place.
+constexpr size_t plan_smem(int NT, int vmax) {
+    return (size_t)kPlanBlock * (2 * (size_t)NT * (vmax + 1) + 8 * kMaxTypes);
+}
+struct WarpWalk {
+    uint16_t hist[kMaxTypes][kPlanMaxNode + 1];  // nodes of type g with v free GPUs
+    uint32_t dem[4 * kMaxTypes];                 // GPUs of groups of size class e on type g, at [4 g + e]
+};
+static_assert(sizeof(WarpWalk) * kPlanWarps <= plan_smem(1, 1), "the warps' areas fit where the threads' lie");
+struct PlanShared {
+    alignas(4) uint16_t init[kMaxTypes][kPlanMaxNode + 1];  // the cluster's nodes per type and GPU count
+    int32_t queue[2 * kPlanBlock];
+    int queued;
+    int deep[kPlanWarps];  // per warp: the deepest template of the queued plans it looked at
+};
+// Thread walks wait on shared and global memory, so the CTAs an SM holds decide
+// them: on eight types in nodes of up to eight GPUs, seven (120,000 plans of up
+// to two stages, most of which walk: 910 us a call with six, the warps' areas
+// beside the threads', 585 with seven; 800,000: 2.86 and 2.59 ms).
+static_assert(7 * (plan_smem(8, 8) + sizeof(PlanShared) + 1024) <= 227 * 1024, "seven CTAs an SM");
 
 __global__ void __launch_bounds__(kPlanBlock, 8) plan_kernel(PlanArgs a) {
     const Layout& y = a.lay;
@@ -64,14 +85,12 @@ __global__ void __launch_bounds__(kPlanBlock, 8) plan_kernel(PlanArgs a) {
     const int32_t* maxn = reinterpret_cast<const int32_t*>(a.img + y.offMaxN);
     const int32_t* pow2 = reinterpret_cast<const int32_t*>(a.img + y.offPow2);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // per warp: nodes of type g with v free GPUs, and the GPUs of groups of
-    // size class e on type g (at [4 g + e])
-    __shared__ uint16_t hists[kPlanWarps][kMaxTypes][kPlanMaxNode + 1];
-    __shared__ uint32_t demands[kPlanWarps][4 * kMaxTypes];
-    auto& hist = hists[warp];
-    uint32_t* dem = demands[warp];
-    // the cluster's nodes per type and GPU count, shared by the CTA
-    __shared__ __align__(4) uint16_t init[kMaxTypes][kPlanMaxNode + 1];
+    extern __shared__ __align__(16) unsigned char psm[];
+    __shared__ PlanShared sh;
+    WarpWalk& ww = reinterpret_cast<WarpWalk*>(psm)[warp];
+    auto& hist = ww.hist;
+    uint32_t* dem = ww.dem;
+    auto& init = sh.init;
     for (int i = threadIdx.x; i < kMaxTypes * (kPlanMaxNode + 1); i += blockDim.x) (&init[0][0])[i] = 0;
     __syncthreads();
     for (int b = threadIdx.x; b < a.n_nodes; b += blockDim.x) {
@@ -86,16 +105,12 @@ __global__ void __launch_bounds__(kPlanBlock, 8) plan_kernel(PlanArgs a) {
     // its degree, split and T are the standalone ones): a quick pass writes
     // such plans, and the others are queued in shared memory and walked a
     // warp each.
-    __shared__ int32_t queue[2 * kPlanBlock];
-    __shared__ int queued;
-    __shared__ int deep[kPlanWarps];  // per warp: the deepest template of the queued plans it looked at
+    int32_t* queue = sh.queue;
+    int& queued = sh.queued;
     if (threadIdx.x == 0) queued = 0;
     __syncthreads();
-    // ---- one thread a plan: per-thread arrays in shared memory, interleaved
-    // by thread (element e of thread t at [e * kPlanBlock + t]): the node
-    // histogram H(g, v) and the demand word my_dem[g] (GPUs of groups per size
-    // class e in 16-bit field e)
-    extern __shared__ __align__(16) unsigned char psm[];
+    // ---- one thread a plan: the node histogram H(g, v) and the demand word
+    // my_dem[g] (GPUs of groups per size class e in 16-bit field e)
     uint64_t* my_dem = reinterpret_cast<uint64_t*>(psm) + threadIdx.x;  // [g * kPlanBlock]
     uint16_t* my_hist = reinterpret_cast<uint16_t*>(psm + (size_t)8 * kMaxTypes * kPlanBlock) + threadIdx.x;
     auto H = [&](int g, int v) -> uint16_t& { return my_hist[(size_t)(g * (V + 1) + v) * kPlanBlock]; };
@@ -452,10 +467,10 @@ __global__ void __launch_bounds__(kPlanBlock, 8) plan_kernel(PlanArgs a) {
                         for (int t = 0; t < nt; ++t) depth = max(depth, min((unsigned)a.slot[t].S[c], (unsigned)kMaxStages));
                     }
                     depth = __reduce_max_sync(kFull, depth);
-                    if (lane == 0) deep[warp] = (int)depth;
+                    if (lane == 0) sh.deep[warp] = (int)depth;
                     __syncthreads();
                     int deepest = 0;
-                    for (int w = 0; w < kPlanWarps; ++w) deepest = max(deepest, deep[w]);
+                    for (int w = 0; w < kPlanWarps; ++w) deepest = max(deepest, sh.deep[w]);
                     alone_min += kAlonePerStage * deepest;
                 }
             }
