@@ -492,8 +492,9 @@ heddle_status heddle_create(heddle_ctx** out, int32_t device) {
     if (e == cudaSuccess)
         e = cudaMalloc(&x->d_scratch, sizeof(hd::TopkEntry) * hd::kTopkListCap * x->scratch_blocks);
     if (e == cudaSuccess) e = alloc_worklist(x->wl[0]);
-    if (e == cudaSuccess) e = cudaMalloc(&x->d_meet, sizeof(hd::TopkMeet));
-    if (e == cudaSuccess) e = cudaMemset(x->d_meet, 0, sizeof(hd::TopkMeet));
+    const size_t meet = hd::TopkMeet::bytes(x->scratch_blocks);
+    if (e == cudaSuccess) e = cudaMalloc(&x->d_meet, meet);
+    if (e == cudaSuccess) e = cudaMemset(x->d_meet, 0, meet);
 
     if (e != cudaSuccess) {
         heddle_destroy(x);

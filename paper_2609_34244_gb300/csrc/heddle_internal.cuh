@@ -329,10 +329,14 @@ constexpr int kWlSurv = kWlMeta - 1;             // the survivor count (see Pric
 
 // Entries a CTA of the top-k hands to the last one.
 constexpr int kTopkListCap = 128;
-// What the CTAs of one top-k launch share.
-struct TopkMeet {
+// What the CTAs of one top-k launch share; behind it, for each of the max_blocks
+// CTAs, the bar that it posts and whether it has.
+struct alignas(16) TopkMeet {
     int32_t tickets;  // CTAs that have handed over
     int32_t entries;  // entries in the scratch list
+    __host__ __device__ TopkEntry* bars() { return reinterpret_cast<TopkEntry*>(this + 1); }
+    __host__ __device__ int32_t* posted(int max_blocks) { return reinterpret_cast<int32_t*>(bars() + max_blocks); }
+    static size_t bytes(int max_blocks) { return sizeof(TopkMeet) + (sizeof(TopkEntry) + sizeof(int32_t)) * max_blocks; }
 };
 
 struct TopkArgs {

@@ -8,14 +8,15 @@
 // are ranked against each other, and the k-th of them is a bar: k entries
 // rank no lower, so none below it can enter the top-k.  Then the entries not
 // below the bar (the incoming state's k-th, once it holds k) are gathered
-// unsorted: little more than k of them in any but a sorted order.  The rank
-// order is strict, ties in throughput going to the smaller index, so many
-// equal throughputs -- a small structure space drawn many times -- pass no
-// more entries than others.  The CTA that draws the last ticket does the
-// same once more over all CTAs' gathered entries and the incoming state,
-// ranks what is left exactly against each other, and writes the state.  No
-// CTA waits on another.  Where a gather overflows its buffer the CTA falls
-// back on sorted warp lists and their tree merge (heddle_rank.cuh).
+// unsorted: little more than k of them, several times k in a sorted order or
+// among ties.  The rank order is strict, ties in throughput going to the smaller
+// index, so many equal throughputs -- a small structure space drawn many times --
+// overflow no gather.  Over a large batch's results the CTAs also post their bars,
+// and each drops what falls below the best posted so far.  The CTA that draws the
+// last ticket does the same once more over all CTAs' gathered entries and the
+// incoming state, ranks what is left exactly against each other, and writes the
+// state.  No CTA waits on another.  Where a gather overflows its buffer the CTA
+// falls back on sorted warp lists and their tree merge (heddle_rank.cuh).
 //
 // What bounds it is latency: two passes over a few entries a thread and one
 // hand-over.  Top-k phase of a pricing call into an empty
@@ -42,6 +43,13 @@ static_assert(kCandCap >= kMaxTopK, "a fallback list of k entries fits a CTA's l
 // each CTA takes at least this many entries (four a thread): fewer only add
 // hand-overs
 constexpr int kPerCta = 4 * kSelBlock;
+// Above so many CTAs times k, the CTAs of a batch's top-k post their bars and drop
+// what falls below another's (a worklist's entries lie in no such order, and fused
+// calls have a running threshold).  Without it the last CTA reads all that they gather, several times k
+// entries each in a sorted order or among ties: 3e5 results, k = 64, random 74 us
+// a call, sorted 89, all equal 98; so 64, 35 and 37.  (Below, the exchange itself
+// costs one or two microseconds: 1.4e5 random results at k = 16 21 -> 22.)
+constexpr int kPostMin = 4096;
 constexpr float kMargin = 1.0f - 1.0f / 65536.0f;
 
 // One candidate entry: from a batch's results, or from the worklist of a
@@ -84,7 +92,7 @@ struct Groups {
 // The k-th of the group bests of the CTA's threads' entries (no_entry where
 // a thread has none): 64 groups of four threads, or 128 of two for k > 32.
 // Every thread of the CTA calls it; false: fewer than k groups hold an entry.
-__device__ bool cta_kth(TopkEntry e, int k, Groups& g, TopkEntry& kth) {
+__device__ __forceinline__ bool cta_kth(TopkEntry e, int k, Groups& g, TopkEntry& kth) {
     const int shift = k <= 32 ? 2 : 1;
     const int ngroups = kSelBlock >> shift;
     for (int o = 1; o < (1 << shift); o <<= 1) {
@@ -113,6 +121,35 @@ __device__ bool cta_kth(TopkEntry e, int k, Groups& g, TopkEntry& kth) {
     __syncthreads();
     kth = g.kth;
     return kth.idx <= INT64_MAX - kSelBlock;
+}
+
+// The best of the CTA's threads' entries (in every thread); tmp: one per warp.
+__device__ __forceinline__ TopkEntry cta_best(TopkEntry e, TopkEntry* tmp) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        TopkEntry x;
+        x.idx = __shfl_xor_sync(0xffffffffu, e.idx, o);
+        x.T = __shfl_xor_sync(0xffffffffu, e.T, o);
+        x.nM = __shfl_xor_sync(0xffffffffu, e.nM, o);
+        x.pad = 0;
+        if (better(x, e)) e = x;
+    }
+    if ((threadIdx.x & 31) == 0) tmp[threadIdx.x >> 5] = e;
+    __syncthreads();
+    e = tmp[0];
+    for (int w = 1; w < kSelWarps; ++w)
+        if (better(tmp[w], e)) e = tmp[w];
+    __syncthreads();
+    return e;
+}
+
+__device__ __forceinline__ int32_t load_acquire(const int32_t* p) {
+    int32_t v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void store_release(int32_t* p, int32_t v) {
+    asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // Append one entry per lane (want) to a list in shared memory; every lane
@@ -160,6 +197,9 @@ __global__ void __launch_bounds__(kSelBlock) topk_select_kernel(TopkArgs a) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t n = kWorklist ? min((int64_t)*a.wl_count, (int64_t)a.wl_cap) : a.n;
     const int ncta = (int)min((int64_t)gridDim.x, max((n + kPerCta - 1) / kPerCta, (int64_t)1));
+    TopkEntry* bars = a.meet->bars();
+    int32_t* posted = a.meet->posted(a.max_blocks);
+    const bool posts = !kWorklist && ncta * k > kPostMin;
     if ((int)blockIdx.x >= ncta) return;
     const int held = min(max(a.state->count, 0), k);  // entries of the incoming state
     const bool full = held >= k;
@@ -249,6 +289,10 @@ __global__ void __launch_bounds__(kSelBlock) topk_select_kernel(TopkArgs a) {
                 have_bar = true;
                 // it raises the call's threshold for the other CTAs
                 if (threadIdx.x == 0 && a.thr) atomicMax(a.thr, __float_as_uint(key_of(kth) * kMargin));
+                if (threadIdx.x == 0 && posts) {
+                    bars[blockIdx.x] = kth;
+                    store_release(posted + blockIdx.x, 1);
+                }
             }
             if (attempt == 0) attempt = 1;
         }
@@ -268,6 +312,31 @@ __global__ void __launch_bounds__(kSelBlock) topk_select_kernel(TopkArgs a) {
         mine = counts[0];
         for (int p = threadIdx.x; p < mine; p += kSelBlock) cand[p] = lists[p];
         __syncthreads();
+    }
+    // ---- drop what falls below the best of the bars posted so far: in a sorted
+    //      order, and among ties, every CTA gathers several times k entries,
+    //      and most of them stop here instead of at the last CTA
+    if (posts && mine > 0) {
+        TopkEntry best = have_bar ? bar : no_entry(threadIdx.x);
+        for (int i = threadIdx.x; i < ncta; i += kSelBlock)
+            if (load_acquire(posted + i)) {
+                const TopkEntry b = far_entry(bars + i);
+                if (better(b, best)) best = b;
+            }
+        best = cta_best(best, tmp);
+        if (best.idx <= INT64_MAX - kSelBlock) {
+            bar = best;
+            have_bar = true;
+        }
+        TopkEntry e = no_entry(0);
+        bool want = (int)threadIdx.x < mine;
+        if (want) e = cand[threadIdx.x];
+        if (want) want = !better(best, e);
+        if (threadIdx.x == 0) n_cand = 0;
+        __syncthreads();
+        gather(cand, &n_cand, kCandCap, want, e);
+        __syncthreads();
+        mine = n_cand;
     }
     // ---- hand over: the CTA reserves its places in the scratch list; the
     //      barrier gathers its stores, thread 0 fences them (fences are
@@ -366,6 +435,8 @@ __global__ void __launch_bounds__(kSelBlock) topk_select_kernel(TopkArgs a) {
             a.meet->entries = 0;
         }
     }
+    if (posts)
+        for (int i = threadIdx.x; i < ncta; i += kSelBlock) posted[i] = 0;
 }
 
 template <bool kWorklist>

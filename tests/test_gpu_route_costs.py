@@ -89,3 +89,30 @@ def test_plan_walk_cost_follows_the_depth(h, W):
         finally:
             h.heddle_destroy(ctx)
     assert us[1] < 1.33 * us[0], us
+
+
+def test_topk_cost_does_not_follow_the_order(h):
+    """300,000 results in random order, sorted either way and all equal: the
+    separate top-k reads the same planes."""
+    import torch
+    n = 300_000
+    T = torch.randint(1 << 30, 1 << 40, (n,), generator=torch.Generator().manual_seed(3)).cuda()
+    one = torch.ones(n, dtype=torch.int16, device="cuda")
+    cands = {"S": torch.ones(n, dtype=torch.uint8, device="cuda"), "M": one,
+             "code": torch.zeros((1, n), dtype=torch.uint8, device="cuda")}
+    ctx = h.heddle_create(0)
+    try:
+        state = h.alloc_topk_state()
+        us = {}
+        for order, t in (("random", T), ("rising", T.sort().values), ("falling", T.sort(descending=True).values),
+                         ("equal", torch.full_like(T, 1 << 35))):
+            res = {"T": t, "bottleneck": t, "n_dp": one, "status": torch.zeros(n, dtype=torch.uint8, device="cuda")}
+
+            def one_pass():
+                h.heddle_topk_reset(ctx, state, 64)
+                h.heddle_topk(ctx, cands, res, state)
+
+            us[order] = pass_us(one_pass)
+        assert max(us.values()) < 1.1 * us["random"], us
+    finally:
+        h.heddle_destroy(ctx)

@@ -149,3 +149,38 @@ def test_price_topk_keeps_iteration_times_of_zero(heddle_lib, oracle_mod, layers
             _same_state(h.topk_state_to_dict(state), exp, "%s k=%d host" % (layers, k))
         finally:
             h.heddle_destroy(ctx)
+
+
+@pytest.mark.parametrize("kind", ("random", "rising", "falling", "equal", "few_ok"))
+def test_topk_posted_bars(heddle_lib, oracle_mod, kind):
+    """CTA counts on both sides of the number from which bars are posted (4,096 /
+    k CTAs of 1,024 entries), in every order, thrice into one state and again
+    in another batch: the flags are clear for the next launch."""
+    h = heddle_lib
+    rng = np.random.default_rng(5)
+    ctx = h.heddle_create(0)
+    try:
+        for k, ns in ((64, (64_000, 66_000, 400_000)), (16, (261_000, 264_000, 400_000)), (13, (320_000,))):
+            for n in ns:
+                T = rng.integers(1 << 30, 1 << 40, 3 * n)
+                status = np.zeros(3 * n, np.uint8)
+                if kind == "rising":
+                    T.sort()
+                elif kind == "falling":
+                    T = np.sort(T)[::-1].copy()
+                elif kind == "equal":
+                    T[:] = 1 << 35
+                elif kind == "few_ok":
+                    status[:] = 1
+                    status[rng.choice(3 * n, 9, replace=False)] = 0
+                planes = {"T": T, "status": status, "n_dp": np.full(3 * n, 4, np.uint16),
+                          "M": np.full(3 * n, 16, np.uint16)}
+                state = h.alloc_topk_state()
+                h.heddle_topk_reset(ctx, state, k)
+                for i in range(3):
+                    lo, hi = i * n, (i + 1) * n
+                    got = _run_topk(h, ctx, {key: v[lo:hi] for key, v in planes.items()}, lo, state)
+                    part = {key: v[:hi] for key, v in planes.items()}
+                    _same_state(got, oracle_mod.topk(part, part["M"], k), "%s n=%d k=%d call %d" % (kind, n, k, i))
+    finally:
+        h.heddle_destroy(ctx)
