@@ -63,8 +63,8 @@ enum {
 typedef struct heddle_ctx heddle_ctx;
 
 /* Create a context on CUDA device `device`.  Allocates its device scratch
- * once (about 190 MB: the search worklist of 2^20 candidates with their 32
- * stage bytes, its per-depth index lists and the top-k merge lists) and
+ * once (about 210 MB: the search worklist of 2^20 candidates with their 32
+ * stage bytes, its per-depth index lists and the top-k's scratch) and
  * queries the SM count.
  * *out is NULL on failure. */
 heddle_status heddle_create(heddle_ctx** out, int32_t device);
@@ -182,10 +182,11 @@ typedef struct {
 
 /* Price a batch (PartitionLayers + Evaluate, §3.1, §5.2, §5.3).
  * Asynchronous on `stream`; no host round-trip.  Each chunk of the batch
- * (heddle_set_chunk, default and at most 2^20 candidates) takes two
- * launches: a screen (masks, DP degree, memory) that compacts the
+ * (heddle_set_chunk, default and at most 2^20 candidates) takes two or
+ * three launches: a screen (masks, DP degree, memory) that compacts the
  * candidates needing the threshold search into a worklist owned by the
- * context, then the search over that worklist.  A batch of one chunk runs
+ * context, then the search over that worklist, which is two kernels where
+ * a thread prices each entry or a warp does.  A batch of one chunk runs
  * on `stream` and allocates nothing.  A batch of several chunks
  * rotates five worklist sets over four context-owned work streams, so
  * the next chunks are screened and searched while chunk i finishes: each work
@@ -228,10 +229,10 @@ typedef struct {
 heddle_status heddle_topk_reset(heddle_ctx* ctx, heddle_topk_state* state, int32_t k,
                                 void* stream);
 
-/* Merge the OK candidates of a priced batch into *state (device): a
- * block-level top-k per CTA into context-owned scratch, then merge levels of
- * 16 lists per CTA, the last with the incoming state (two or three
- * launches, no inter-CTA waiting).
+/* Merge the OK candidates of a priced batch into *state (device): every CTA
+ * finds a bar that k of its entries reach and gathers what is not below it
+ * into context-owned scratch; the last CTA to finish ranks what all gathered
+ * with the incoming state (one launch, no inter-CTA waiting).
  * Asynchronous; reads cands->M, results->T/n_dp/status.  Errors: E_ARG,
  * E_STATE, E_CUDA.  Calls on one context must not overlap on the GPU (they
  * share the scratch): use one stream per context. */
@@ -240,11 +241,10 @@ heddle_status heddle_topk(heddle_ctx* ctx, const heddle_candidates* cands,
                           void* stream);
 
 /* Price a batch and merge its OK candidates into *state (device): after each
- * chunk's search, one top-k launch runs over that chunk's worklist of
- * searched candidates only (the screen already rejected the rest): per-CTA
- * lists, the last CTA of each group of 16 merges its group and the last
- * group merges the group lists into the state (tickets, no waiting) -- no
- * pass over the full results.
+ * chunk's search, one launch of heddle_topk's kernel runs over that chunk's
+ * worklist of searched candidates only (the screen already rejected the
+ * rest) -- on the equal-layer path only over those that reach the running
+ * k-th throughput of the call -- and not over the full results.
  * Same results and the same state as heddle_price_candidates followed by
  * heddle_topk.  Errors as for both. */
 heddle_status heddle_price_topk(heddle_ctx* ctx, const heddle_candidates* cands,
@@ -520,8 +520,8 @@ heddle_status heddle_work_counters(heddle_ctx* ctx, uint64_t out[3]);
  * each phase's time is its own kernels' elapsed time while they share the
  * GPU.  heddle_phase_times synchronises on them and returns, per
  * phase (SCREEN, SEARCH, TOPK), the summed elapsed milliseconds and the
- * number of kernels launched in it (one screen, one search and one top-k
- * kernel per chunk), then forgets them.  The events add no work to the
+ * number of launches (one screen, one search, whatever its kernels, and one
+ * top-k per chunk), then forgets them.  The events add no work to the
  * kernels; enabling or disabling changes no result.  Errors: E_ARG,
  * E_CUDA. */
 #define HEDDLE_PHASE_SCREEN 0

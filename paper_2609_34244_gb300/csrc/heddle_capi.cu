@@ -223,9 +223,9 @@ heddle_status build_image(heddle_ctx* x, const std::vector<heddle_layer>& layers
     lay = hd::make_layout(L, NT);
     CU(grow(img, img_cap, lay.bytes));
     CU(grow(qtab, q_cap, sizeof(int64_t) * (size_t)NT * 4 * L));
-    // the inputs packed into one pinned buffer and copied at once (the build
-    // used to allocate, copy and free each array: a third of the time a
-    // planner spent on reloading a small cluster and model)
+    // the inputs packed into one pinned buffer and copied at once (allocating,
+    // copying and freeing each array took a third of the time a planner
+    // spends on reloading a small cluster and model)
     const size_t b_types = hd::align16((uint32_t)(sizeof(heddle_gpu_type) * NT));
     const size_t b_nodes = (sizeof(heddle_node) * x->nodes.size() + 15) & ~(size_t)15;
     const size_t b_layers = hd::align16((uint32_t)(sizeof(heddle_layer) * L));

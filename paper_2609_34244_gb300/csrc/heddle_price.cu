@@ -85,8 +85,9 @@ constexpr int kRow = kScreenBlock + 16;  // bytes of a tile row: 256 candidates 
 // stage to every class of its type's demand, one run length that marks "no
 // layer fits" in its size; the DP degree is one minimum of float ratios over
 // the classes that can decide on this cluster.  1e6 candidates of the largest
-// workload: 40.0M -> 31.7M warp instructions, 65 -> 55 us alone; of the
-// 80-layer one 61 -> 51 us, of the expert one 39 -> 30.
+// workload: 33.3M warp instructions and 50 us alone (40.0M and 65 with tables
+// built by every CTA, integer quotients and rejections written in sorted order);
+// of the 80-layer one 50 us (61), of the expert one 29 (39).
 __global__ void __launch_bounds__(kScreenBlock) screen_kernel(PriceArgs a) {
     __shared__ ScreenTabs tab;
     __shared__ uint32_t dem[8 * kScreenBlock];  // per-thread demand word (see stage_desc), per type

@@ -21,10 +21,9 @@
 // What bounds it is latency: two passes over a few entries a thread and one
 // hand-over.  Top-k phase of a pricing call into an empty
 // state (events, launch included): 1,000 candidates of the 32-layer workload
-// 18.2 -> 12.2 us, 1e5 of them 30.3 -> 18.1, 1e6 of the 80-layer one 35 -> 22
-// (before: a bitonic merge per 32 entries for a floor on float keys, sorted
-// warp lists, two levels of tree merges).  The separate call took three
-// launches.
+// 12.2 us, 1e5 of them 18.1, 1e6 of the 80-layer one 22 (18.2, 30.3 and 35 with a
+// bitonic merge per 32 entries for a floor on float keys, sorted warp lists and
+// two levels of tree merges, three launches in the separate call).
 
 #include <algorithm>
 

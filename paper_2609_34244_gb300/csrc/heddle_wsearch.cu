@@ -11,8 +11,9 @@
 // (1 ns away, then 2^-7 of it and doubling) until both sides are known, then
 // bisects.  The sets
 // of the probe at B* give the canonical split; a feasible probe that closes
-// the bracket already holds them (every bound in [hi, B] takes the same
-// decisions), so only a bracket closed from below costs a final probe.
+// the bracket and built sets already holds them (every bound in [hi, B] takes
+// the same decisions).  A bracket closed from below, or by a probe that the
+// forward chain alone decided, costs a final probe for them.
 // The probe (heddle_wprobe.cuh) checks 32 positions per round with the
 // interval test of this file: stage time
 // P[j] - P[i] + c and memory against k times the GPU memory.  Evaluate runs

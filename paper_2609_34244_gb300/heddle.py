@@ -257,7 +257,7 @@ def heddle_price_mbs(ctx, cands, results, mbs=None, stream=None):
 
 def heddle_set_chunk(ctx, chunk: int):
     """Chunk size of the pricing calls (1 .. 2**20); a call of several
-    chunks pipelines them over two work streams."""
+    chunks pipelines them over four work streams."""
     _check(ctx, load_library().heddle_set_chunk(ctx, int(chunk)))
 
 
@@ -394,8 +394,9 @@ def heddle_set_search(ctx, mode: int):
 
 
 def heddle_set_thread_search_min(ctx, min_entries: int):
-    """Bucketed entries from which the general search runs its
-    thread-per-entry kernel (< 0: the default, 32 x the SM count)."""
+    """Entries from which the general search, and the split rule of
+    equal-layer models, run their thread-per-entry kernels, and queued plans
+    of a CTA from which a thread walks each (< 0: the defaults; 0: always)."""
     _check(ctx, load_library().heddle_set_thread_search_min(ctx, int(min_entries)))
 
 

@@ -21,7 +21,8 @@ def main():
     for name, n in cases:
         w = W.make_workload(name, seed=3, n=n)
         for mode, split, tmin in ((h.SEARCH_AUTO, "minmax", None), (h.SEARCH_GENERAL, "minmax", None),
-                                  (h.SEARCH_GENERAL, "minmax", 0), (h.SEARCH_DISTRIBUTE, "distribute", None)):
+                                  (h.SEARCH_GENERAL, "minmax", 0), (h.SEARCH_DISTRIBUTE, "distribute", None),
+                                  (h.SEARCH_DISTRIBUTE, "distribute", 0)):
             ref = O.Oracle(w.cluster, w.model).set_split(split).price(w.cands, threads=8)
             for fused in (False, True):
                 got = G.price_gpu(h, w.cluster, w.model, w.cands, k=16, search=mode, fused=fused, chunk=65536,
@@ -30,15 +31,16 @@ def main():
                 G.assert_same(got, ref, what="%s mode %d fused %s" % (name, mode, fused))
                 exp = O.topk(ref, w.cands["M"], 16)
                 assert got["topk"]["idx"].tolist() == exp["idx"].tolist(), (name, mode)
-    # plans: the per-slot SKIPPED mask and the walk
+    # plans: the slots that are SKIPPED, and both walks
     import test_gpu_plans as TP
     for name in ("dense32", "stress128"):
         w = W.make_workload(name, seed=4, n=3001)
         plans = W.make_plans(w, 3001, 4, seed=4)
         ref = O.Oracle(w.cluster, w.model).price_plans(plans)
-        got = TP.price_plans_gpu(h, w.cluster, w.model, plans, bounds=True)
-        assert got["errors"] == 0, "%s plans: device flags %#x" % (name, got["errors"])
-        TP._same(got, ref, "%s plans" % name)
+        for tmin in (None, 0):
+            got = TP.price_plans_gpu(h, w.cluster, w.model, plans, bounds=True, thread_min=tmin)
+            assert got["errors"] == 0, "%s plans: device flags %#x" % (name, got["errors"])
+            TP._same(got, ref, "%s plans" % name)
     w = W.make_workload("moe16", seed=2, n=20011)
     ref = O.Oracle(w.cluster, w.model).set_experts(w.model["expert_state_bytes"], w.model["expert_param_bytes"]) \
         .price(w.cands, threads=8)

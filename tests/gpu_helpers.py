@@ -16,8 +16,8 @@ def price_gpu(h, w_cluster, w_model, cands, k=16, bounds=True, batch=None, count
     merges in one call (heddle_price_topk); ``phases`` times the pricing
     phases with the library's events and returns them under "phases";
     ``chunk`` sets the library's chunk size (calls of several chunks are
-    pipelined over its work streams); ``thread_min`` sets the general
-    search's routing threshold (0: thread kernel whenever it has entries,
+    pipelined over its work streams); ``thread_min`` sets the
+    searches' routing threshold (0: thread kernel whenever it has entries,
     2**31 - 1: warp kernel only)."""
     import torch
     ctx = h.heddle_create(0)

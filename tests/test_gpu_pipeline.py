@@ -1,6 +1,6 @@
-"""Calls of several chunks: the library pipelines them over two work
-streams and two worklist sets (one chunk's screen and search overlap the
-previous chunk's search and top-k).  Results, bounds and the top-k must be
+"""Calls of several chunks: the library pipelines them over four work
+streams and five worklist sets (one chunk's screen and search overlap the
+earlier chunks' searches and top-k).  Results, bounds and the top-k must be
 bit-exact with one chunk per call and with the oracle, on every search
 path, for ragged chunk sizes."""
 

@@ -64,18 +64,23 @@ def _same(got, ref, what):
 @pytest.mark.parametrize("deepest", [1, 2, 4, 8])
 @pytest.mark.parametrize("n", [1, 127, 129, 20011])
 def test_plans_that_mostly_walk(h, W, oracle_mod, deepest, n):
-    """Shallow templates, most of which fit: a CTA's queue fills, and plans
-    are walked by a thread each, the rest by a warp each; bounds as well."""
+    """Shallow templates, most of which fit, on one plan and on all SMs (a CTA
+    queues at most 17 of 20,011, which it walks a warp each by default), and a
+    thread each; bounds as well."""
     w = W.make_workload("dense32", seed=5, n=n)
     plans = W.make_plans(w, n, 4, seed=5)
     plans["S"] = np.minimum(plans["S"], deepest).astype(plans["S"].dtype)
     plans["code"] = np.ascontiguousarray(plans["code"][:, :deepest])
     plans["code"][np.arange(deepest)[None, :, None] >= plans["S"][:, None, :]] = 0
-    ref = oracle_mod.Oracle(w.cluster, w.model).price_plans(plans)
+    orc = oracle_mod.Oracle(w.cluster, w.model)
+    ref = orc.price_plans(plans)
     for bounds in (False, True):
-        got = price_plans_gpu(h, w.cluster, w.model, plans, bounds=bounds)
-        assert got["errors"] == 0
-        _same(got, ref, "deepest %d" % deepest)
+        for thread_min in (None, 0):
+            got = price_plans_gpu(h, w.cluster, w.model, plans, bounds=bounds, thread_min=thread_min)
+            assert got["errors"] == 0
+            _same(got, ref, "deepest %d" % deepest)
+            if bounds:
+                _bounds_same(orc, plans, got)
 
 
 @pytest.mark.parametrize("name,n", [("tiny", 300), ("dense32", 4001), ("dense80", 1501), ("moe48", 4001),
