@@ -486,13 +486,14 @@ heddle_status heddle_get_search(heddle_ctx* ctx, int32_t* in_use);
  * the warp-per-entry search prices those it cannot decide; with fewer, the
  * warp search prices every entry (a thread search with too few entries runs
  * as long as its longest serial chain).  The split rule of equal-layer models
- * (DISTRIBUTE) has two such kernels as well, and heddle_price_plans two walks:
- * there min_entries counts the plans queued by one CTA (at most 255).
- * min_entries < 0 restores the defaults: 32 x the device's SM count for the
- * general search; 5,000 entries, and 550 more per stage of the deepest, for the
- * split rule; 20 queued plans, and 5 more per stage of the deepest, for the plan
- * walk.  0 always runs the thread kernels, and the memory probe ahead of the
- * tiled search, which otherwise runs from a batch size on.  All routes return
+ * (DISTRIBUTE) has two such kernels as well.  min_entries < 0 restores the
+ * defaults: 32 x the device's SM count for the general search; 5,000 entries,
+ * and 550 more per stage of the deepest, for the split rule.  0 always runs the
+ * thread kernels, and INT32_MAX never; these two also choose how
+ * heddle_price_plans walks its plans (by default a thread each where a CTA has
+ * queued at least 20, and 5 more per stage of the deepest of them, else a warp
+ * each), and 0 the memory probe ahead of the tiled search, which otherwise
+ * runs from a batch size on.  All routes return
  * identical results.  Errors: E_ARG (ctx NULL). */
 heddle_status heddle_set_thread_search_min(heddle_ctx* ctx, int32_t min_entries);
 

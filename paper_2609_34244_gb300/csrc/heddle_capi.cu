@@ -1327,7 +1327,8 @@ heddle_status heddle_price_plans(heddle_ctx* x, const heddle_plans* pl, const he
     a.node_gpus = x->d_node_gpus;
     a.n_nodes = (int32_t)nn;
     a.vmax = vmax;
-    a.alone_min = x->thread_min < 0 ? 0 : std::max(x->thread_min, 1);
+    // (the setting counts entries of a worklist: here it only forces a walk)
+    a.alone_min = x->thread_min == 0 ? 1 : x->thread_min == INT32_MAX ? INT32_MAX : 0;
     a.placed = pr->placed;
     a.thr = pr->thr;
     a.err = x->d_flags + 1;

@@ -395,8 +395,8 @@ def heddle_set_search(ctx, mode: int):
 
 def heddle_set_thread_search_min(ctx, min_entries: int):
     """Entries from which the general search, and the split rule of
-    equal-layer models, run their thread-per-entry kernels, and queued plans
-    of a CTA from which a thread walks each (< 0: the defaults; 0: always)."""
+    equal-layer models, run their thread-per-entry kernels (< 0: the defaults;
+    0: always, 2**31 - 1: never, and so for the plan walk)."""
     _check(ctx, load_library().heddle_set_thread_search_min(ctx, int(min_entries)))
 
 
